@@ -6,10 +6,10 @@
 //                  one thread per (cell, variable):
 //     k_reconstruct_tma       FP32C Euler, tables staged in shared memory by TMA
 //     k_reconstruct_f32c      FP32C scalar advection
-//     k_reconstruct           FP64
 //     k_reconstruct_char_tma  FP32C Euler, characteristic variables (four lanes
 //                             per cell exchange variables by shuffles)
-//     k_reconstruct_char      FP64, characteristic variables
+//     k_reconstruct_f64, k_reconstruct_char_f64   FP64 (kernels_f64.cuh): a
+//                             thread per (cell, variable, face)
 //   k_face         one thread per face: two Gauss points, rotated HLLC (Euler) or
 //                  upwind (scalar) flux, |l|/2 (F1 + F2) (Eqs. 5-6); at reflective
 //                  walls the outer state is the inner one mirrored, at inflow faces
@@ -44,8 +44,6 @@ template <> struct Sub<9> {
   static __device__ __forceinline__ int a(int j) { constexpr int t[9] = {1, 2, 3, 1, 2, 3, 3, 1, 2}; return t[j]; }
   static __device__ __forceinline__ int b(int j) { constexpr int t[9] = {2, 3, 1, 4, 5, 6, 7, 8, 9}; return t[j]; }
 };
-
-template <typename T> __device__ __forceinline__ T fabs_(T x) { return x < T(0) ? -x : x; }
 
 // Vector loads / stores of one cell's NV values.
 template <typename T, int NV>
@@ -142,84 +140,6 @@ __device__ __forceinline__ df df_mul(df a, df b) {
 }
 
 // ---------------------------------------------------------------- K1
-// Threads t in [0, N*NV): cell q = t / NV of the group, variable v = t % NV.
-template <typename T, int NV, int M, int G, bool COMP, bool WALLS>
-__global__ void __launch_bounds__(256) k_reconstruct(
-    const T* __restrict__ U, const T* __restrict__ Ulo, const int32_t* __restrict__ slot,
-    const T* __restrict__ gop, const T* __restrict__ dg, const T* __restrict__ gam,
-    const T* __restrict__ area, int64_t N, int64_t first, int64_t gbase, T* __restrict__ Wg,
-    T eps, T theta, int linear) {
-  const int64_t total = N * NV;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t q = t / NV;
-    const int v = (int)(t - q * NV);
-    const int64_t c = first + q;
-    const T w0 = __ldg(U + c * NV + v);
-    const T l0 = COMP ? __ldg(Ulo + c * NV + v) : T(0);
-    // differences to the stencil cells (slots 1..M), replacements already resolved
-    T dW[M + 1];
-    dW[0] = T(0);
-    const int32_t fm = flip_mask<WALLS, NV>(v);
-#pragma unroll
-    for (int s = 1; s <= M; ++s)
-      dW[s] = slot_delta<T, NV, WALLS, COMP>(U, Ulo, __ldg(slot + (int64_t)(s - 1) * N + q), v, fm, w0, l0);
-    // candidate gradients g_j = D_j^+ (dW_a, dW_b), beta_j = |Omega| |g_j|^2
-    T gx[M], gy[M], beta[M];
-    const T a0 = __ldg(area + c);
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-      const T da = dW[Sub<M>::a(j)], db = dW[Sub<M>::b(j)];
-      const T m0 = __ldg(gop + (int64_t)(j * 4 + 0) * N + q), m1 = __ldg(gop + (int64_t)(j * 4 + 1) * N + q);
-      const T m2 = __ldg(gop + (int64_t)(j * 4 + 2) * N + q), m3 = __ldg(gop + (int64_t)(j * 4 + 3) * N + q);
-      gx[j] = m0 * da + m1 * db;
-      gy[j] = m2 * da + m3 * db;
-      beta[j] = a0 * (gx[j] * gx[j] + gy[j] * gy[j]);
-    }
-    T* out = Wg + (gbase + q * G) * NV + v;
-#pragma unroll 1
-    for (int g = 0; g < G; ++g) {
-      const T dx = __ldg(dg + (int64_t)(g * 2) * N + q), dy = __ldg(dg + (int64_t)(g * 2 + 1) * N + q);
-      const T* gg = gam + (int64_t)(g * M) * N + q;
-      T incr;
-      if (linear) {
-        incr = T(0);
-#pragma unroll
-        for (int j = 0; j < M; ++j) incr += __ldg(gg + (int64_t)j * N) * (gx[j] * dx + gy[j] * dy);
-      } else {
-        // splitting of Section 3.4: gt+ = (gamma + theta |gamma|)/2, gt- = gt+ - gamma
-        T sp = T(0), sm = T(0);
-#pragma unroll
-        for (int j = 0; j < M; ++j) {
-          const T gj = __ldg(gg + (int64_t)j * N);
-          const T tp = T(0.5) * (gj + theta * fabs_(gj));
-          sp += tp;
-          sm += tp - gj;
-        }
-        const T isp = T(1) / sp, ism = T(1) / sm;
-        T Ap = T(0), Bp = T(0), Am = T(0), Bm = T(0);
-#pragma unroll
-        for (int j = 0; j < M; ++j) {
-          const T gj = __ldg(gg + (int64_t)j * N);
-          const T tp = T(0.5) * (gj + theta * fabs_(gj));
-          const T gp = tp * isp, gm = (tp - gj) * ism;
-          const T p = gx[j] * dx + gy[j] * dy;  // P^1_j(x_G) - W0
-          const T qp = gp * beta[j], qm = gm * beta[j];
-          const T bp = beta[j] * (T(1) + qp + qp * qp) + eps;  // new indicator + eps
-          const T bm = beta[j] * (T(1) + qm + qm * qm) + eps;
-          const T ap = gp / (bp * bp), am = gm / (bm * bm);
-          Ap += ap;
-          Bp += ap * p;
-          Am += am;
-          Bm += am * p;
-        }
-        // R - W0 = sigma+ sum delta+ p - sigma- sum delta- p
-        incr = sp * (Bp / Ap) - sm * (Bm / Am);
-      }
-      out[(int64_t)g * NV] = COMP ? w0 + (l0 + incr) : w0 + incr;
-    }
-  }
-}
-
 // FP32C variant of K1 (same arithmetic in FP32 with approximate reciprocals).
 // Tables: gop4[j][q] = (o0 o1 o2 o3) of D_j^+, dg2[g][q] = x_G - c0,
 // gam4[g][k][q] = gamma_{4k..4k+3}, gam1[g][q] = gamma_8 (triangles).
@@ -997,8 +917,6 @@ __global__ void k_advance_time(double* __restrict__ t, const double* __restrict_
 // reconstructs field l, and returns variable l of W0 + R dU with row l of R.
 // Reconstructing the increment dU (zero for constant data) keeps constant
 // states exact whatever the rounding of R R^-1.
-template <typename T> __device__ __forceinline__ T rcp_exact(T x) { return T(1) / x; }
-
 template <typename T>
 __device__ __forceinline__ T lane_sum4(const T c[4], T x, int base) {
   T r = T(0);
@@ -1036,102 +954,6 @@ __device__ __forceinline__ void roe_rows(const T Wl[4], const T Wr[4], T nx, T n
     Lr[0] = T(0.5) * (b2 - qn * ia); Lr[1] = T(0.5) * (nx * ia - b1 * u);
     Lr[2] = T(0.5) * (ny * ia - b1 * v); Lr[3] = T(0.5) * b1;
     Rr[0] = H - a * qn; Rr[1] = kin; Rr[2] = qt; Rr[3] = H + a * qn;
-  }
-}
-
-template <typename T, int M, int G, bool COMP, bool WALLS>
-__global__ void __launch_bounds__(256) k_reconstruct_char(
-    const T* __restrict__ U, const T* __restrict__ Ulo, const int32_t* __restrict__ slot,
-    const T* __restrict__ gop, const T* __restrict__ dg, const T* __restrict__ gam,
-    const T* __restrict__ area, int64_t N, int64_t first, int64_t gbase, T* __restrict__ Wg,
-    T eps, T theta, T gas_gamma, int linear) {
-  const int lane = threadIdx.x & 31, base = lane & ~3, l = lane & 3;
-  const int64_t total = N * 4;
-  // warp-uniform loop: every lane reaches the shuffles; lanes past the end work on cell 0
-  for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); t0 < total;
-       t0 += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t t = t0 + lane;
-    const bool act = t < total;
-    const int64_t q = act ? (t >> 2) : 0;
-    const int64_t c = first + q;
-    T W0[4];
-    load_vec<T, 4>(U + c * 4, W0);
-    const T w0 = W0[l];
-    const T l0 = COMP ? __ldg(Ulo + c * 4 + l) : T(0);
-    T dW[M + 1];
-    dW[0] = T(0);
-    const int32_t fm = flip_mask<WALLS, 4>(l);
-#pragma unroll
-    for (int s = 1; s <= M; ++s)
-      dW[s] = slot_delta<T, 4, WALLS, COMP>(U, Ulo, __ldg(slot + (int64_t)(s - 1) * N + q), l, fm, w0, l0);
-    const T a0 = __ldg(area + c);
-#pragma unroll 1
-    for (int k = 0; k < G / 2; ++k) {
-      // face frame: Roe average with the neighbour, outward normal from the face's two Gauss points
-      T Wn[4];
-      slot_state4<T, WALLS>(U, __ldg(slot + (int64_t)k * N + q), Wn);  // slot k+1: across face k
-      const T x0 = __ldg(dg + (int64_t)(4 * k) * N + q), y0 = __ldg(dg + (int64_t)(4 * k + 1) * N + q);
-      const T x1 = __ldg(dg + (int64_t)(4 * k + 2) * N + q), y1 = __ldg(dg + (int64_t)(4 * k + 3) * N + q);
-      const T tx = x1 - x0, ty = y1 - y0, it = T(1) / sqrt(tx * tx + ty * ty);
-      T Lr[4], Rr[4];
-      roe_rows<T>(W0, Wn, ty * it, -tx * it, gas_gamma - T(1), l, Lr, Rr);
-      // project the stencil differences onto field l, then candidate gradients and indicators
-      T dU[M + 1];
-      dU[0] = T(0);
-#pragma unroll
-      for (int s = 1; s <= M; ++s) dU[s] = lane_sum4(Lr, dW[s], base);
-      T gx[M], gy[M], beta[M];
-#pragma unroll
-      for (int j = 0; j < M; ++j) {
-        const T da = dU[Sub<M>::a(j)], db = dU[Sub<M>::b(j)];
-        const T m0 = __ldg(gop + (int64_t)(j * 4 + 0) * N + q), m1 = __ldg(gop + (int64_t)(j * 4 + 1) * N + q);
-        const T m2 = __ldg(gop + (int64_t)(j * 4 + 2) * N + q), m3 = __ldg(gop + (int64_t)(j * 4 + 3) * N + q);
-        gx[j] = m0 * da + m1 * db;
-        gy[j] = m2 * da + m3 * db;
-        beta[j] = a0 * (gx[j] * gx[j] + gy[j] * gy[j]);
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int g = 2 * k + h;
-        const T dx = __ldg(dg + (int64_t)(g * 2) * N + q), dy = __ldg(dg + (int64_t)(g * 2 + 1) * N + q);
-        const T* gg = gam + (int64_t)(g * M) * N + q;
-        T incr;
-        if (linear) {
-          incr = T(0);
-#pragma unroll
-          for (int j = 0; j < M; ++j) incr += __ldg(gg + (int64_t)j * N) * (gx[j] * dx + gy[j] * dy);
-        } else {
-          T sp = T(0), sm = T(0);
-#pragma unroll
-          for (int j = 0; j < M; ++j) {
-            const T gj = __ldg(gg + (int64_t)j * N);
-            const T tp = T(0.5) * (gj + theta * fabs_(gj));
-            sp += tp;
-            sm += tp - gj;
-          }
-          const T isp = T(1) / sp, ism = T(1) / sm;
-          T Ap = T(0), Bp = T(0), Am = T(0), Bm = T(0);
-#pragma unroll
-          for (int j = 0; j < M; ++j) {
-            const T gj = __ldg(gg + (int64_t)j * N);
-            const T tp = T(0.5) * (gj + theta * fabs_(gj));
-            const T gp = tp * isp, gmn = (tp - gj) * ism;
-            const T p = gx[j] * dx + gy[j] * dy;
-            const T qp = gp * beta[j], qm = gmn * beta[j];
-            const T bp = beta[j] * (T(1) + qp + qp * qp) + eps;
-            const T bm = beta[j] * (T(1) + qm + qm * qm) + eps;
-            const T ap = gp / (bp * bp), am = gmn / (bm * bm);
-            Ap += ap;
-            Bp += ap * p;
-            Am += am;
-            Bm += am * p;
-          }
-          incr = sp * (Bp / Ap) - sm * (Bm / Am);
-        }
-        const T dWl = lane_sum4(Rr, incr, base);  // variable l of R dU
-        if (act) Wg[(gbase + q * G + g) * 4 + l] = COMP ? w0 + (l0 + dWl) : w0 + dWl;
-      }
-    }
   }
 }
 

@@ -1,0 +1,367 @@
+// FP64 reconstruction (K1) and its arithmetic: component-wise and characteristic variables.
+//
+// What bounds it: the FP64 pipe.  GB300 has 2 FP64 lanes per clock and SM, 1/64 of its FP32 rate
+// (0.62 T FMA/s measured), so a double-precision instruction costs what about sixty others do, and
+// the tables' bytes are small beside it.  Hence every choice below removes FP64 instructions, at the
+// price of integer work, shuffles, shared-memory traffic or larger tables:
+//   - the splitting of the linear weights (geometry only) is done once per solver (k_split_weights),
+//   - differences, gradients and indicators are computed once per (cell, variable) and shared through
+//     shared memory by the threads of the cell's faces,
+//   - the new indicator is a polynomial in the split weight, two fused multiply-adds,
+//   - reciprocals start from the special-function unit's 20-bit seed and take one third-order step.
+// Measured (one pass, before = one thread per (cell, variable) with IEEE division and the splitting
+// repeated by every variable, 5,350 FP64 issue slots a thread on quads; now 535 in each of 4 threads):
+// 17,920 Euler quads 662 -> 277 us, 15,360 triangles 384 -> 144 us (the FP64 pipe busy throughout);
+// 1,600 scalar quads, 332 -> 30 us; 40,000 quads in characteristic variables, 2,151 -> 804 us.
+#pragma once
+
+#include "kernels.cuh"
+
+namespace weno {
+namespace dev {
+
+__device__ __forceinline__ uint32_t hi_word(double x) { return (uint32_t)__double2hiint(x); }
+
+// 1/x by the third-order Householder iteration x0 (1 + e + e^2), e = 1 - x x0 (the series of 1/(1 - e)
+// cut after e^2), from the seed of rcp.approx.ftz.f64 (20 bits, so e^3 < 2^-60): three FP64
+// instructions, last-bit accurate.  Valid where rcp_safe(hi_word(x)); outside it the caller divides.
+__device__ __forceinline__ double rcp_seed(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  return r;
+}
+__device__ __forceinline__ double rcp_f64(double x) {
+  const double r = rcp_seed(x), e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+// Positive normal numbers well inside the exponent range (2^-1021 <= x < 2^1021): one unsigned compare
+// that zeros, subnormals, infinities, NaN and negative numbers fail.
+constexpr uint32_t kHiMin = 0x00200000u, kHiMax = 0x7fc00000u;
+__device__ __forceinline__ bool rcp_safe(uint32_t hi_min, uint32_t hi_max) { return hi_min >= kHiMin && hi_max < kHiMax; }
+
+// a / b of two sums of weights: b > 0 unless the weights left the FP64 range.
+__device__ __forceinline__ double quotient_f64(double a, double b) {
+  const uint32_t h = hi_word(b);
+  return rcp_safe(h, h) ? a * rcp_f64(b) : a / b;
+}
+
+// Split linear weights of a group from its linear weights gam [g][j][q] (Section 3.4):
+// gt+ = (gamma + theta |gamma|) / 2, gt- = gt+ - gamma, sigma+- = sum gt+-, gamma+- = gt+- / sigma+-.
+// wt [g][j][q] = (gamma+, gamma-) and sig [g][q] = (sigma+, sigma-), rows of `pitch` cells.
+template <int M>
+__global__ void k_split_weights(const double* __restrict__ gam, int64_t N, int G, double theta, int64_t pitch,
+                                double2* __restrict__ wt, double2* __restrict__ sig) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= N * G) return;
+  const int64_t g = t / N, q = t - g * N;
+  double tp[M], tm[M], sp = 0.0, sm = 0.0;
+#pragma unroll
+  for (int j = 0; j < M; ++j) {
+    const double x = gam[(g * M + j) * N + q];
+    tp[j] = 0.5 * (x + theta * fabs(x));
+    tm[j] = tp[j] - x;
+    sp += tp[j];
+    sm += tm[j];
+  }
+  sig[g * pitch + q] = make_double2(sp, sm);
+  const double isp = 1.0 / sp, ism = 1.0 / sm;
+#pragma unroll
+  for (int j = 0; j < M; ++j) wt[(g * M + j) * pitch + q] = make_double2(tp[j] * isp, tm[j] * ism);
+}
+
+// Members of candidate j (slot numbers 1..M), four bits each, for a j known at run time only.
+template <int M> struct SubBits;
+template <> struct SubBits<12> { static constexpr uint64_t A = 0x422433114321ull, B = 0xcba987651432ull; };
+template <> struct SubBits<9> { static constexpr uint64_t A = 0x213321321ull, B = 0x987654132ull; };
+template <int M> __device__ __forceinline__ int sub_a(int j) { return (int)(SubBits<M>::A >> (4 * j)) & 15; }
+template <int M> __device__ __forceinline__ int sub_b(int j) { return (int)(SubBits<M>::B >> (4 * j)) & 15; }
+
+// What a Gauss point needs of one candidate: gradient, beta + eps, beta^2, beta^3.
+struct CandF64 { double gx, gy, be, b2, b3; };
+
+__device__ __forceinline__ CandF64 candidate_f64(double m0, double m1, double m2, double m3, double da, double db,
+                                                 double a0, double eps) {
+  CandF64 c;
+  c.gx = m0 * da + m1 * db;
+  c.gy = m2 * da + m3 * db;
+  const double b = a0 * (c.gx * c.gx + c.gy * c.gy);
+  c.be = b + eps;
+  c.b2 = b * b;
+  c.b3 = c.b2 * b;
+  return c;
+}
+
+// Increments R(x_G) - W0 at the two Gauss points of one face (Section 3.4), from the candidates
+// cand(j) and the split weights w[h][j * pitch] = (gamma+, gamma-) of point h:
+//   alpha+- = gamma+- / (beta~+- + eps)^2,  beta~+- + eps = (beta + eps) + gamma (beta^2 + gamma beta^3),
+//   R - W0 = sigma+ sum alpha+ p / sum alpha+  -  sigma- sum alpha- p / sum alpha-.
+// 20 FP64 instructions per point and candidate.  Returns false if a square of an indicator left the
+// range of rcp_f64 (or was NaN): the increments are then redone by face_points_ieee.
+template <int M, int UNROLL, typename Cand>
+__device__ __forceinline__ bool face_points_f64(Cand cand, const double2* __restrict__ w0, const double2* __restrict__ w1,
+                                                int64_t pitch, const double dx[2], const double dy[2],
+                                                const double2 sig[2], double incr[2]) {
+  double Ap[2] = {0.0, 0.0}, Bp[2] = {0.0, 0.0}, Am[2] = {0.0, 0.0}, Bm[2] = {0.0, 0.0};
+  uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll UNROLL
+  for (int j = 0; j < M; ++j) {
+    const CandF64 c = cand(j);
+    const double2 w[2] = {__ldg(w0 + j * pitch), __ldg(w1 + j * pitch)};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const double p = c.gx * dx[h] + c.gy * dy[h];
+      const double dp = fma(w[h].x, fma(w[h].x, c.b3, c.b2), c.be), dn = fma(w[h].y, fma(w[h].y, c.b3, c.b2), c.be);
+      const double sp = dp * dp, sn = dn * dn;
+      lo = min(lo, min(hi_word(sp), hi_word(sn)));
+      hi = max(hi, max(hi_word(sp), hi_word(sn)));
+      const double ap = w[h].x * rcp_f64(sp), an = w[h].y * rcp_f64(sn);
+      Ap[h] += ap;
+      Bp[h] = fma(ap, p, Bp[h]);
+      Am[h] += an;
+      Bm[h] = fma(an, p, Bm[h]);
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) incr[h] = sig[h].x * quotient_f64(Bp[h], Ap[h]) - sig[h].y * quotient_f64(Bm[h], Am[h]);
+  return rcp_safe(lo, hi);
+}
+
+// The same with IEEE division and the indicator as printed, beta (1 + q + q^2) with q = gamma beta:
+// for indicators whose powers leave the FP64 range, and NaN states.
+template <int M, typename Cand>
+__device__ __forceinline__ void face_points_ieee(Cand cand, const double2* __restrict__ w0, const double2* __restrict__ w1,
+                                                 int64_t pitch, const double dx[2], const double dy[2],
+                                                 const double2 sig[2], double a0, double eps, double incr[2]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    double Ap = 0.0, Bp = 0.0, Am = 0.0, Bm = 0.0;
+#pragma unroll 1
+    for (int j = 0; j < M; ++j) {
+      const CandF64 c = cand(j);
+      const double2 w = __ldg((h ? w1 : w0) + j * pitch);
+      const double p = c.gx * dx[h] + c.gy * dy[h], b = a0 * (c.gx * c.gx + c.gy * c.gy);
+      const double qp = w.x * b, qn = w.y * b;
+      const double dp = b * (1.0 + qp + qp * qp) + eps, dn = b * (1.0 + qn + qn * qn) + eps;
+      const double ap = w.x / (dp * dp), an = w.y / (dn * dn);
+      Ap += ap;
+      Bp += ap * p;
+      Am += an;
+      Bm += an * p;
+    }
+    incr[h] = sig[h].x * (Bp / Ap) - sig[h].y * (Bm / Am);
+  }
+}
+
+// Layout of a block of either kernel: `width` = cells x variables of its tile; thread t holds column
+// t % width (cell (t % width) / NV, variable or field t % NV) and face t / width of the cell.
+constexpr int kF64MaxWidth = 32;
+
+// Component-wise FP64 K1.  A thread gathers 3 of its column's M stencil differences, then forms 3 of
+// its M candidates, both into shared memory, then evaluates the two Gauss points of its face.
+template <int NV, int M, int G, bool WALLS>
+__global__ void __launch_bounds__(kF64MaxWidth * G / 2) k_reconstruct_f64(
+    const double* __restrict__ U, const int32_t* __restrict__ slot, const double* __restrict__ gop,
+    const double* __restrict__ dg, const double* __restrict__ gam, const double2* __restrict__ wt,
+    const double2* __restrict__ sigma, const double* __restrict__ area, int64_t N, int64_t pitch, int64_t first,
+    int64_t gbase, double* __restrict__ Wg, double eps, int linear, int width) {
+  constexpr int F = G / 2, PER = M / F;
+  static_assert(PER * F == M, "each face's threads take an equal share of the slots and candidates");
+  extern __shared__ double sm[];
+  double* dW = sm;                                      // [slot - 1][column]
+  double *gx = sm + M * width, *gy = gx + M * width;    // [candidate][column]
+  double *be = gy + M * width, *b2 = be + M * width, *b3 = b2 + M * width;
+  const int col = threadIdx.x % width, face = threadIdx.x / width, v = col % NV;
+  const int64_t qr = (int64_t)blockIdx.x * (width / NV) + col / NV;
+  const int64_t q = qr < N ? qr : N - 1;  // columns past the end work on the last cell and store nothing
+  const int64_t c = first + q;
+  const double w0 = __ldg(U + c * NV + v), a0 = __ldg(area + c);
+  const int32_t fm = flip_mask<WALLS, NV>(v);
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    const int s = face * PER + i;
+    dW[s * width + col] =
+        slot_delta<double, NV, WALLS, false>(U, nullptr, __ldg(slot + (int64_t)s * N + q), v, fm, w0, 0.0);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    const int j = face * PER + i;
+    const double* o = gop + (int64_t)(j * 4) * N + q;
+    const CandF64 cd = candidate_f64(__ldg(o), __ldg(o + N), __ldg(o + 2 * N), __ldg(o + 3 * N),
+                                     dW[(sub_a<M>(j) - 1) * width + col], dW[(sub_b<M>(j) - 1) * width + col], a0, eps);
+    const int k = j * width + col;
+    gx[k] = cd.gx; gy[k] = cd.gy; be[k] = cd.be; b2[k] = cd.b2; b3[k] = cd.b3;
+  }
+  __syncthreads();
+  const int g = 2 * face;
+  const double* d = dg + (int64_t)(2 * g) * N + q;
+  const double dx[2] = {__ldg(d), __ldg(d + 2 * N)}, dy[2] = {__ldg(d + N), __ldg(d + 3 * N)};
+  double incr[2] = {0.0, 0.0};
+  if (linear) {
+    const double* gg = gam + (int64_t)(g * M) * N + q;
+#pragma unroll 3
+    for (int j = 0; j < M; ++j) {
+      const double x = gx[j * width + col], y = gy[j * width + col];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) incr[h] += __ldg(gg + (int64_t)(h * M + j) * N) * (x * dx[h] + y * dy[h]);
+    }
+  } else {
+    auto cand = [&](int j) {
+      const int k = j * width + col;
+      return CandF64{gx[k], gy[k], be[k], b2[k], b3[k]};
+    };
+    const double2 *wa = wt + (int64_t)(g * M) * pitch + q, *wb = wa + (int64_t)M * pitch;
+    const double2 sig[2] = {__ldg(sigma + (int64_t)g * pitch + q), __ldg(sigma + (int64_t)(g + 1) * pitch + q)};
+    if (!face_points_f64<M, 3>(cand, wa, wb, pitch, dx, dy, sig, incr))
+      face_points_ieee<M>(cand, wa, wb, pitch, dx, dy, sig, a0, eps, incr);
+  }
+  if (qr < N) {
+    double* out = Wg + (gbase + q * G + g) * NV + v;
+    out[0] = w0 + incr[0];
+    out[NV] = w0 + incr[1];
+  }
+}
+
+// 1/sqrt(x), last-bit accurate: with e = 1 - x y0^2 from the 20-bit seed y0 of rsqrt.approx.ftz.f64,
+// 1/sqrt(x) = y0 (1 + e/2 + 3/8 e^2 + ...), the binomial series of (1 - e)^(-1/2) cut below 2^-60.
+__device__ __forceinline__ double rsqrt_f64(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+// sqrt(x) = x / sqrt(x), from the same seed: s0 = x y0, sqrt(x) = s0 (1 + e/2 + 3/8 e^2 + ...).
+__device__ __forceinline__ double sqrt_f64(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double s = x * y, e = fma(-s, y, 1.0);
+  return fma(s * e, fma(e, 0.375, 0.5), s);
+}
+// Guarded forms: IEEE outside the range the iterations are valid in.
+__device__ __noinline__ double rcp_ieee(double x) { return 1.0 / x; }
+__device__ __noinline__ double sqrt_ieee(double x) { return sqrt(x); }
+__device__ __noinline__ double rsqrt_ieee(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ double rcp_any(double x) {
+  const uint32_t h = hi_word(x) & 0x7fffffffu;
+  return rcp_safe(h, h) ? rcp_f64(x) : rcp_ieee(x);
+}
+__device__ __forceinline__ double sqrt_any(double x) {
+  const uint32_t h = hi_word(x);
+  return rcp_safe(h, h) ? sqrt_f64(x) : sqrt_ieee(x);
+}
+__device__ __forceinline__ double rsqrt_any(double x) {
+  const uint32_t h = hi_word(x);
+  return rcp_safe(h, h) ? rsqrt_f64(x) : rsqrt_ieee(x);
+}
+
+// Roe frame of one face: R^-1 (fr[4 f + v]) and R (fr[16 + 4 v + f]), fields f ordered q_n - a, entropy,
+// shear, q_n + a, from the two cells' averages and the outward normal (tx, ty rotated by -90 degrees).
+__device__ __forceinline__ void roe_frame_f64(const double Wl[4], const double Wr[4], double tx, double ty, double gm1,
+                                              double* __restrict__ fr) {
+  const double it = rsqrt_any(tx * tx + ty * ty), nx = ty * it, ny = -tx * it;
+  const double il = rcp_any(Wl[0]), ir = rcp_any(Wr[0]);
+  const double ul = Wl[1] * il, vl = Wl[2] * il, ur = Wr[1] * ir, vr = Wr[2] * ir;
+  const double hl = (Wl[3] + gm1 * (Wl[3] - 0.5 * Wl[0] * (ul * ul + vl * vl))) * il;
+  const double hr = (Wr[3] + gm1 * (Wr[3] - 0.5 * Wr[0] * (ur * ur + vr * vr))) * ir;
+  const double sl = sqrt_any(Wl[0]), sr = sqrt_any(Wr[0]), iw = rcp_any(sl + sr);
+  const double u = (sl * ul + sr * ur) * iw, v = (sl * vl + sr * vr) * iw, H = (sl * hl + sr * hr) * iw;
+  const double kin = 0.5 * (u * u + v * v), a2 = gm1 * (H - kin), ia = rsqrt_any(a2), a = a2 * ia;
+  const double qn = u * nx + v * ny, qt = v * nx - u * ny;
+  const double b1 = gm1 * ia * ia, b2 = b1 * kin;
+  fr[0] = 0.5 * (b2 + qn * ia); fr[1] = -0.5 * (b1 * u + nx * ia); fr[2] = -0.5 * (b1 * v + ny * ia); fr[3] = 0.5 * b1;
+  fr[4] = 1.0 - b2; fr[5] = b1 * u; fr[6] = b1 * v; fr[7] = -b1;
+  fr[8] = -qt; fr[9] = -ny; fr[10] = nx; fr[11] = 0.0;
+  fr[12] = 0.5 * (b2 - qn * ia); fr[13] = 0.5 * (nx * ia - b1 * u); fr[14] = 0.5 * (ny * ia - b1 * v); fr[15] = 0.5 * b1;
+  fr[16] = 1.0; fr[17] = 1.0; fr[18] = 0.0; fr[19] = 1.0;
+  fr[20] = u - a * nx; fr[21] = u; fr[22] = -ny; fr[23] = u + a * nx;
+  fr[24] = v - a * ny; fr[25] = v; fr[26] = nx; fr[27] = v + a * ny;
+  fr[28] = H - a * qn; fr[29] = kin; fr[30] = qt; fr[31] = H + a * qn;
+}
+
+// FP64 K1 in characteristic variables (see the comment at the FP32C kernels below for the method).
+// Thread (cell, field l, face): the block's first threads build the Roe frames, one thread a frame
+// instead of four lanes each repeating it; every thread projects the shared stencil differences onto
+// its field with row l of R^-1, evaluates its face's two points, and returns variable l of R dU.
+constexpr int kFrame = 33;  // doubles a frame takes in shared memory (32, padded against bank conflicts)
+
+template <int M, int G, bool WALLS>
+__global__ void __launch_bounds__(kF64MaxWidth * G / 2) k_reconstruct_char_f64(
+    const double* __restrict__ U, const int32_t* __restrict__ slot, const double* __restrict__ gop,
+    const double* __restrict__ dg, const double* __restrict__ gam, const double2* __restrict__ wt,
+    const double2* __restrict__ sigma, const double* __restrict__ area, int64_t N, int64_t pitch, int64_t first,
+    int64_t gbase, double* __restrict__ Wg, double eps, double gas_gamma, int linear, int width) {
+  constexpr int F = G / 2, PER = M / F;
+  extern __shared__ double sm[];
+  const int tile = width / 4, threads = width * F;
+  double* dW = sm;                      // [slot - 1][column]
+  double* dU = dW + M * width;          // [slot - 1][thread]
+  double* fr = dU + M * threads;        // [face][cell] frames
+  double* inc = fr + kFrame * tile * F; // [point][thread]
+  const int t = threadIdx.x, col = t % width, face = t / width, l = col % 4, cl = col / 4;
+  const int64_t q0 = (int64_t)blockIdx.x * tile, qr = q0 + cl;
+  const int64_t q = qr < N ? qr : N - 1;  // columns past the end work on the last cell and store nothing
+  const int64_t c = first + q;
+  const double w0 = __ldg(U + c * 4 + l), a0 = __ldg(area + c);
+  const int32_t fm = flip_mask<WALLS, 4>(l);
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    const int s = face * PER + i;
+    dW[s * width + col] =
+        slot_delta<double, 4, WALLS, false>(U, nullptr, __ldg(slot + (int64_t)s * N + q), l, fm, w0, 0.0);
+  }
+  if (t < tile * F) {  // frame of face t / tile of cell t % tile; the neighbour across face k is slot k + 1
+    const int k = t / tile;
+    const int64_t fq = q0 + t % tile < N ? q0 + t % tile : N - 1;
+    double Wl[4], Wn[4];
+    load_vec<double, 4>(U + (first + fq) * 4, Wl);
+    slot_state4<double, WALLS>(U, __ldg(slot + (int64_t)k * N + fq), Wn);
+    const double* d = dg + (int64_t)(4 * k) * N + fq;
+    roe_frame_f64(Wl, Wn, __ldg(d + 2 * N) - __ldg(d), __ldg(d + 3 * N) - __ldg(d + N), gas_gamma - 1.0, fr + kFrame * t);
+  }
+  __syncthreads();
+  const double* f0 = fr + kFrame * (face * tile + cl);
+  const double L0 = f0[4 * l], L1 = f0[4 * l + 1], L2 = f0[4 * l + 2], L3 = f0[4 * l + 3];
+#pragma unroll 4
+  for (int s = 0; s < M; ++s) {
+    const double* x = dW + s * width + 4 * cl;
+    dU[s * threads + t] = L0 * x[0] + L1 * x[1] + L2 * x[2] + L3 * x[3];
+  }
+  const int g = 2 * face;
+  const double* d = dg + (int64_t)(2 * g) * N + q;
+  const double dx[2] = {__ldg(d), __ldg(d + 2 * N)}, dy[2] = {__ldg(d + N), __ldg(d + 3 * N)};
+  auto cand = [&](int j) {
+    const double* o = gop + (int64_t)(j * 4) * N + q;
+    return candidate_f64(__ldg(o), __ldg(o + N), __ldg(o + 2 * N), __ldg(o + 3 * N),
+                         dU[(sub_a<M>(j) - 1) * threads + t], dU[(sub_b<M>(j) - 1) * threads + t], a0, eps);
+  };
+  double incr[2] = {0.0, 0.0};
+  if (linear) {
+    const double* gg = gam + (int64_t)(g * M) * N + q;
+#pragma unroll 3
+    for (int j = 0; j < M; ++j) {
+      const CandF64 x = cand(j);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) incr[h] += __ldg(gg + (int64_t)(h * M + j) * N) * (x.gx * dx[h] + x.gy * dy[h]);
+    }
+  } else {
+    const double2 *wa = wt + (int64_t)(g * M) * pitch + q, *wb = wa + (int64_t)M * pitch;
+    const double2 sig[2] = {__ldg(sigma + (int64_t)g * pitch + q), __ldg(sigma + (int64_t)(g + 1) * pitch + q)};
+    if (!face_points_f64<M, 3>(cand, wa, wb, pitch, dx, dy, sig, incr))
+      face_points_ieee<M>(cand, wa, wb, pitch, dx, dy, sig, a0, eps, incr);
+  }
+  inc[t] = incr[0];
+  inc[threads + t] = incr[1];
+  __syncthreads();
+  if (qr < N) {  // variable l of R dU
+    const double* r = f0 + 16 + 4 * l;
+    double* out = Wg + (gbase + q * G + g) * 4 + l;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const double* x = inc + h * threads + (t & ~3);
+      out[h * 4] = w0 + (r[0] * x[0] + r[1] * x[1] + r[2] * x[2] + r[3] * x[3]);
+    }
+  }
+}
+
+}  // namespace dev
+}  // namespace weno

@@ -13,7 +13,7 @@
 
 #include "host_lsq.hpp"
 #include "host_mesh.hpp"
-#include "kernels.cuh"
+#include "kernels_f64.cuh"
 #include "weno3.h"
 
 namespace weno {
@@ -91,13 +91,15 @@ struct weno_solver_s {
   int64_t nQ = 0, nT = 0, N = 0, nF = 0, n_boundary = 0;
   int n_inst = 1;
   // device tables
-  // FP64: SoA tables [entry][cell] (gop, dg, gam).  FP32C: packed rows of float4 / float2
+  // FP64: SoA tables [entry][cell] (gop, dg; gam for the linear scheme, otherwise the split weights
+  // wt [g][j][cell] and their sums sig [g][cell], rows of q_pitch / t_pitch cells).  FP32C: packed rows of float4 / float2
   // with the cell fastest: gop = D_j^+ entries, dg = (x_G - c0, sigma+, sigma-),
   // gam = gamma+ then gamma- rows, gam1 = (gamma+_8, gamma-_8) of triangles.
   void *q_gop = nullptr, *q_dg = nullptr, *q_gam = nullptr, *t_gop = nullptr, *t_dg = nullptr, *t_gam = nullptr;
   void *q_gam1 = nullptr, *t_gam1 = nullptr;
   void *q_pgam = nullptr, *q_pdg = nullptr, *t_pgam = nullptr, *t_pdg = nullptr;  // point-pair tables (Euler FP32C)
-  int64_t q_pitch = 0, t_pitch = 0;  // row pitch (cells) of the packed FP32C tables
+  double2 *q_wt = nullptr, *q_sig = nullptr, *t_wt = nullptr, *t_sig = nullptr;   // FP64 split weights
+  int64_t q_pitch = 0, t_pitch = 0;  // row pitch (cells) of the packed FP32C tables and the FP64 split weights
   bool tma = false;                   // Euler FP32C: reconstruction with TMA-staged tables
   CUtensorMap q_map_gop{}, t_map_gop{};  // gradient operators
   CUtensorMap q_map_pgam{}, q_map_pdg{}, t_map_pgam{}, t_map_pdg{};  // point-pair tables (both FP32C Euler kernels)
@@ -186,6 +188,24 @@ unsigned fix_grid(const S& s, int64_t n) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(chunks, 4 * s.nsm));
 }
 
+// Grid of an FP64 reconstruction over n cells of F faces and M candidates: blocks of `width` (cell,
+// variable) columns, one thread per column and face, with the kernel's shared memory.  The FP64 pipe is
+// the bound, so the SMs have to share the columns evenly: tiles shrink from 32 columns to 8 until every
+// SM has four blocks.
+struct F64Grid {
+  int width;
+  unsigned blocks, threads;
+  size_t smem;
+};
+F64Grid f64_grid(const S& s, int64_t n, int nv, int M, int F, bool characteristic) {
+  int width = weno::dev::kF64MaxWidth;
+  while (width > 8 && n * nv < (int64_t)4 * s.nsm * width) width /= 2;
+  const int tile = width / nv;
+  const size_t doubles = characteristic ? (size_t)M * width + (size_t)(M + 2) * width * F + weno::dev::kFrame * tile * F
+                                        : (size_t)6 * M * width;
+  return {width, (unsigned)((n + tile - 1) / tile), (unsigned)(width * F), doubles * sizeof(double)};
+}
+
 // Cell reconstruction into the Gauss-value array wg.  which: bit 0 = quad group,
 // bit 1 = triangle group.
 template <typename T, int NV, bool COMP, bool WALLS>
@@ -193,7 +213,7 @@ void launch_reconstruct_impl(S& s, const void* U, const void* Ulo, void* wg, cud
                              uint8_t* redo) {
   const T* u = static_cast<const T*>(U);
   const T* ul = static_cast<const T*>(Ulo);
-  const T eps = (T)s.prm.eps, th = (T)s.prm.theta;
+  const T eps = (T)s.prm.eps;
   if constexpr (NV == 4) {
     if (s.prm.characteristic) {
       const T gg = (T)s.prm.gas_gamma;
@@ -221,14 +241,18 @@ void launch_reconstruct_impl(S& s, const void* U, const void* Ulo, void* wg, cud
               8 * s.nQ, (float*)wg, eps, gg, s.prm.linear, redo_t, cells_t, s.err, s.debug_stall);
         }
       } else {
-        if (s.nQ && (which & 1))
-          weno::dev::k_reconstruct_char<T, 12, 8, COMP, WALLS><<<grid_of(s.k1q, s.nQ * 4), s.k1q.block, 0, st>>>(
-              u, ul, s.q_slot, (const T*)s.q_gop, (const T*)s.q_dg, (const T*)s.q_gam, (const T*)s.area, s.nQ, 0,
-              0, (T*)wg, eps, th, gg, s.prm.linear);
-        if (s.nT && (which & 2))
-          weno::dev::k_reconstruct_char<T, 9, 6, COMP, WALLS><<<grid_of(s.k1t, s.nT * 4), s.k1t.block, 0, st>>>(
-              u, ul, s.t_slot, (const T*)s.t_gop, (const T*)s.t_dg, (const T*)s.t_gam, (const T*)s.area, s.nT,
-              s.nQ, 8 * s.nQ, (T*)wg, eps, th, gg, s.prm.linear);
+        if (s.nQ && (which & 1)) {
+          const F64Grid g = f64_grid(s, s.nQ, 4, 12, 4, true);
+          weno::dev::k_reconstruct_char_f64<12, 8, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
+              u, s.q_slot, (const double*)s.q_gop, (const double*)s.q_dg, (const double*)s.q_gam, s.q_wt, s.q_sig,
+              (const double*)s.area, s.nQ, s.q_pitch, 0, 0, (double*)wg, eps, gg, s.prm.linear, g.width);
+        }
+        if (s.nT && (which & 2)) {
+          const F64Grid g = f64_grid(s, s.nT, 4, 9, 3, true);
+          weno::dev::k_reconstruct_char_f64<9, 6, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
+              u, s.t_slot, (const double*)s.t_gop, (const double*)s.t_dg, (const double*)s.t_gam, s.t_wt, s.t_sig,
+              (const double*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (double*)wg, eps, gg, s.prm.linear, g.width);
+        }
       }
       return;
     }
@@ -270,14 +294,18 @@ void launch_reconstruct_impl(S& s, const void* U, const void* Ulo, void* wg, cud
           (const float2*)s.t_gam1, (const float*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (float*)wg, eps,
           s.prm.linear);
   } else {
-    if (s.nQ && (which & 1))
-      weno::dev::k_reconstruct<T, NV, 12, 8, COMP, WALLS><<<grid_of(s.k1q, s.nQ * NV), s.k1q.block, 0, st>>>(
-          u, ul, s.q_slot, (const T*)s.q_gop, (const T*)s.q_dg, (const T*)s.q_gam, (const T*)s.area, s.nQ, 0, 0,
-          (T*)wg, eps, th, s.prm.linear);
-    if (s.nT && (which & 2))
-      weno::dev::k_reconstruct<T, NV, 9, 6, COMP, WALLS><<<grid_of(s.k1t, s.nT * NV), s.k1t.block, 0, st>>>(
-          u, ul, s.t_slot, (const T*)s.t_gop, (const T*)s.t_dg, (const T*)s.t_gam, (const T*)s.area, s.nT, s.nQ,
-          8 * s.nQ, (T*)wg, eps, th, s.prm.linear);
+    if (s.nQ && (which & 1)) {
+      const F64Grid g = f64_grid(s, s.nQ, NV, 12, 4, false);
+      weno::dev::k_reconstruct_f64<NV, 12, 8, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
+          u, s.q_slot, (const double*)s.q_gop, (const double*)s.q_dg, (const double*)s.q_gam, s.q_wt, s.q_sig,
+          (const double*)s.area, s.nQ, s.q_pitch, 0, 0, (double*)wg, eps, s.prm.linear, g.width);
+    }
+    if (s.nT && (which & 2)) {
+      const F64Grid g = f64_grid(s, s.nT, NV, 9, 3, false);
+      weno::dev::k_reconstruct_f64<NV, 9, 6, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
+          u, s.t_slot, (const double*)s.t_gop, (const double*)s.t_dg, (const double*)s.t_gam, s.t_wt, s.t_sig,
+          (const double*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (double*)wg, eps, s.prm.linear, g.width);
+    }
   }
 }
 
@@ -533,6 +561,31 @@ int upload_pairs(S& s, const GroupTables& T, int64_t P, double theta, void** gam
   CK(cudaStreamSynchronize(st));  // the host vectors go out of scope
   *gam = pa;
   *dg = pb;
+  return WENO_OK;
+}
+
+// FP64 tables of the linear weights: gam itself for the linear scheme, otherwise the split weights,
+// formed on the device from a temporary copy of gam.
+template <int M>
+int upload_split(S& s, const GroupTables& T, int64_t pitch, void** gam, double2** wt, double2** sig, cudaStream_t st) {
+  if (s.prm.linear) return upload_real(s, gam, T.gam, st);
+  int r;
+  if ((r = s.alloc(wt, sizeof(double2) * (size_t)T.G * M * pitch))) return r;
+  if ((r = s.alloc(sig, sizeof(double2) * (size_t)T.G * pitch))) return r;
+  if (!T.N) return WENO_OK;
+  double* tmp = nullptr;
+  cudaError_t e = cudaMalloc(&tmp, T.gam.size() * sizeof(double));
+  if (e != cudaSuccess) return fail(WENO_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  e = cudaMemcpyAsync(tmp, T.gam.data(), T.gam.size() * sizeof(double), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) {
+    weno::dev::k_split_weights<M><<<(unsigned)((T.N * T.G + 127) / 128), 128, 0, st>>>(tmp, T.N, T.G, s.prm.theta, pitch,
+                                                                                       *wt, *sig);
+    e = cudaGetLastError();
+  }
+  const cudaError_t es = cudaStreamSynchronize(st);
+  cudaFree(tmp);
+  if (e == cudaSuccess) e = es;
+  if (e != cudaSuccess) return fail(WENO_ECUDA, std::string("split weights: ") + cudaGetErrorString(e));
   return WENO_OK;
 }
 
@@ -834,10 +887,14 @@ int weno_solver_create(weno_mesh_t mesh, const weno_params* params, void* cuda_s
   if (d.fp64) {
     if ((r = upload_real(d, &d.q_gop, tq.gop, st))) return r;
     if ((r = upload_real(d, &d.q_dg, tq.dg, st))) return r;
-    if ((r = upload_real(d, &d.q_gam, tq.gam, st))) return r;
     if ((r = upload_real(d, &d.t_gop, tt.gop, st))) return r;
     if ((r = upload_real(d, &d.t_dg, tt.dg, st))) return r;
-    if ((r = upload_real(d, &d.t_gam, tt.gam, st))) return r;
+    d.q_pitch = (d.nQ + 7) / 8 * 8;
+    d.t_pitch = (d.nT + 7) / 8 * 8;
+    if ((r = upload_split<12>(d, tq, d.q_pitch, &d.q_gam, &d.q_wt, &d.q_sig, st))) return r;
+    if ((r = upload_split<9>(d, tt, d.t_pitch, &d.t_gam, &d.t_wt, &d.t_sig, st))) return r;
+    // the FP64 reconstruction's block follows from the mesh (f64_grid) and is not tuned
+    if (d.nQ) d.k1q.block = (int)f64_grid(d, d.nQ, d.nv, 12, 4, p.characteristic).threads;
   } else {
     d.q_pitch = (d.nQ + 63) / 64 * 64;
     d.t_pitch = (d.nT + 63) / 64 * 64;
@@ -1174,8 +1231,8 @@ int weno_autotune(weno_solver_t s, const void* U, const void* U_lo, void* cuda_s
   void* u = const_cast<void*>(U);
   void* ul = const_cast<void*>(U_lo);
   const std::vector<Launch>& k1c = d.tma ? tma : generic;
-  if (d.nQ) tune(d.k1q, [&] { WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st, 1); }, k1c);
-  if (d.nT) tune(d.k1t, [&] { WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st, 2); }, k1c);
+  if (d.nQ && !d.fp64) tune(d.k1q, [&] { WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st, 1); }, k1c);
+  if (d.nT && !d.fp64) tune(d.k1t, [&] { WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st, 2); }, k1c);
   tune(d.k2, [&] { WENO_DISPATCH(d, launch_face, d, st); }, generic);
   if (d.nQ) tune(d.k3q, [&] { WENO_DISPATCH(d, launch_gather, d, 0, u, ul, d.Ws, st, 1); }, generic);
   if (d.nT) tune(d.k3t, [&] { WENO_DISPATCH(d, launch_gather, d, 0, u, ul, d.Ws, st, 2); }, generic);
