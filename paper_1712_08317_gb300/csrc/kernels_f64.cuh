@@ -1,6 +1,7 @@
-// FP64 reconstruction (K1) and its arithmetic: component-wise and characteristic variables.
+// FP64 kernels and their arithmetic: reconstruction (K1), component-wise and in characteristic
+// variables, and face fluxes (K2).
 //
-// What bounds it: the FP64 pipe.  GB300 has 2 FP64 lanes per clock and SM, 1/64 of its FP32 rate
+// What bounds them: the FP64 pipe.  GB300 has 2 FP64 lanes per clock and SM, 1/64 of its FP32 rate
 // (0.62 T FMA/s measured), so a double-precision instruction costs what about sixty others do, and
 // the tables' bytes are small beside it.  Hence every choice below removes FP64 instructions, at the
 // price of integer work, shuffles, shared-memory traffic or larger tables:
@@ -9,7 +10,7 @@
 //     shared memory by the threads of the cell's faces,
 //   - the new indicator is a polynomial in the split weight, two fused multiply-adds,
 //   - reciprocals start from the special-function unit's 20-bit seed and take one third-order step.
-// Measured (one pass, before = one thread per (cell, variable) with IEEE division and the splitting
+// K1 measured (one pass, before = one thread per (cell, variable) with IEEE division and the splitting
 // repeated by every variable, 5,350 FP64 issue slots a thread on quads; now 535 in each of 4 threads):
 // 17,920 Euler quads 662 -> 277 us, 15,360 triangles 384 -> 144 us (the FP64 pipe busy throughout);
 // 1,600 scalar quads, 332 -> 30 us; 40,000 quads in characteristic variables, 2,151 -> 804 us.
@@ -359,6 +360,123 @@ __global__ void __launch_bounds__(kF64MaxWidth * G / 2) k_reconstruct_char_f64(
     for (int h = 0; h < 2; ++h) {
       const double* x = inc + h * threads + (t & ~3);
       out[h * 4] = w0 + (r[0] * x[0] + r[1] * x[1] + r[2] * x[2] + r[3] * x[3]);
+    }
+  }
+}
+
+// ---------------------------------------------------------------- K2
+// HLLC flux of one Gauss point, as hllc in kernels.cuh with the divisions and square roots of this file,
+// one reciprocal fewer on the star side (k p / m = p / (S_K - S*)) and the side taken by selection
+// instead of branches: about 130 FP64 instructions.  Returns false, and no flux, unless every quantity
+// it takes a reciprocal or a root of is in the range of the iterations; in particular a state that
+// passes has rho > 0, p > 0 and a finite energy.
+__device__ __forceinline__ bool hllc_f64(const double wl[4], const double wr[4], double nx, double ny, double gam,
+                                         double out[4]) {
+  const double gm1 = gam - 1.0;
+  const double rl = wl[0], rr = wr[0], El = wl[3], Er = wr[3];
+  const double il = rcp_f64(rl), ir = rcp_f64(rr);
+  const double nl = wl[1] * nx + wl[2] * ny, tl = wl[2] * nx - wl[1] * ny;  // normal and tangential momentum
+  const double nr = wr[1] * nx + wr[2] * ny, tr = wr[2] * nx - wr[1] * ny;
+  const double ul = nl * il, vl = tl * il, ur = nr * ir, vr = tr * ir;
+  const double pl = gm1 * (El - 0.5 * (nl * ul + tl * vl)), pr = gm1 * (Er - 0.5 * (nr * ur + tr * vr));
+  const double al2 = gam * pl * il, ar2 = gam * pr * ir;
+  const double al = sqrt_f64(al2), ar = sqrt_f64(ar2);
+  const double sl = sqrt_f64(rl), sr = sqrt_f64(rr), iw = rcp_f64(sl + sr);
+  const double u = (sl * ul + sr * ur) * iw, v = (sl * vl + sr * vr) * iw;
+  const double H = (sl * ((El + pl) * il) + sr * ((Er + pr) * ir)) * iw;
+  const double a2 = gm1 * (H - 0.5 * (u * u + v * v)), a = sqrt_f64(a2);
+  const double SL = fmin(ul - al, u - a), SR = fmax(ur + ar, u + a);
+  const double ml = rl * (SL - ul), mr = rr * (SR - ur), dm = ml - mr;
+  const double SS = (pr - pl + ul * ml - ur * mr) * rcp_f64(dm);
+  const bool left = SL >= 0.0 || SS >= 0.0;
+  const double S = left ? SL : SR, dS = S - SS, id = rcp_f64(dS);
+  const double r = left ? rl : rr, mn = left ? nl : nr, mt = left ? tl : tr, E = left ? El : Er;
+  const double un = left ? ul : ur, ut = left ? vl : vr, p = left ? pl : pr, ri = left ? il : ir, m = left ? ml : mr;
+  const double k = m * id;  // rho of the star state
+  const double Es = k * (E * ri + (SS - un) * SS) + (SS - un) * (p * id);
+  const double Se = (left ? SL >= 0.0 : !(SR > 0.0)) ? 0.0 : S;  // no star term beyond the outer waves
+  const double f0 = mn + Se * (k - r), f1 = mn * un + p + Se * (k * SS - mn);
+  const double f2 = mn * ut + Se * (k * ut - mt), f3 = (E + p) * un + Se * (Es - E);
+  out[0] = f0;
+  out[1] = f1 * nx - f2 * ny;
+  out[2] = f1 * ny + f2 * nx;
+  out[3] = f3;
+  const uint32_t h[7] = {hi_word(rl), hi_word(rr), hi_word(al2), hi_word(ar2), hi_word(a2), hi_word(dm) & 0x7fffffffu,
+                         hi_word(dS) & 0x7fffffffu};
+  uint32_t lo = h[0], hi = h[0];
+#pragma unroll
+  for (int i = 1; i < 7; ++i) {
+    lo = min(lo, h[i]);
+    hi = max(hi, h[i]);
+  }
+  return rcp_safe(lo, hi);
+}
+
+// The general form, for states that hllc_f64 declines (and to find out whether they are non-physical).
+__device__ __noinline__ void hllc_ieee(const double* wl, const double* wr, double nx, double ny, double gam, double* out,
+                                       bool* bad) {
+  hllc<double>(wl, wr, nx, ny, gam, out, *bad);
+}
+
+// FP64 K2: thread (face, Gauss point), the two points of a face on neighbouring lanes, which add their
+// fluxes and store half of the face's variables each.  Twice the threads of the FP32 kernel: the FP64
+// pipe is filled on meshes half the size, and each lane's two states are 64 contiguous bytes with its
+// neighbour's.  Flags and boundary states as k_face.
+template <int NV, bool INFLOW>
+__global__ void __launch_bounds__(256) k_face_f64(
+    const double* __restrict__ Wg, const int32_t* __restrict__ gl, const int32_t* __restrict__ gr,
+    const double* __restrict__ fnx, const double* __restrict__ fny, const double* __restrict__ flen, int64_t nF,
+    double* __restrict__ F, Prm<double> prm, int* __restrict__ flag, const int32_t* __restrict__ inst, int64_t nQ,
+    Inflow<double> inf) {
+  const int64_t total = 2 * nF;
+  // the loop is uniform over a warp, whose lanes exchange fluxes; lanes past the end repeat the last face
+  for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); t0 < total;
+       t0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t t = t0 + (threadIdx.x & 31);
+    const bool act = t < total;
+    const int64_t f = act ? t >> 1 : nF - 1;
+    const int k = (int)(t & 1);
+    const int64_t il = __ldg(gl + f), ir = __ldg(gr + f);
+    const double nx = __ldg(fnx + f), ny = __ldg(fny + f);
+    double wl[NV], wr[NV], fk[NV];
+    load_vec<double, NV>(Wg + (il + k) * NV, wl);
+    if (ir >= 0) {
+      load_vec<double, NV>(Wg + (ir + 1 - k) * NV, wr);
+    } else {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) wr[v] = wl[v];
+      if (NV == 4 && ir == -2) {
+        const double mn = wl[1] * nx + wl[2] * ny;
+        wr[1] = wl[1] - 2.0 * mn * nx;
+        wr[2] = wl[2] - 2.0 * mn * ny;
+      }
+      if constexpr (INFLOW && NV == 4) {
+        if (ir <= -3) {
+          const int i = inst ? __ldg(inst + cell_of_gauss(il, nQ)) : 0;
+          const bool a = __ldg(inf.xi + 2 * (-3 - ir) + k) < inf.speed * (inf.t[i] + inf.c * inf.dt[i]);
+#pragma unroll
+          for (int v = 0; v < 4; ++v) wr[v] = a ? inf.wa[v] : inf.wb[v];
+        }
+      }
+    }
+    bool bad = false;
+    if constexpr (NV == 4) {
+      if (!hllc_f64(wl, wr, nx, ny, prm.gas_gamma, fk)) hllc_ieee(wl, wr, nx, ny, prm.gas_gamma, fk, &bad);
+    } else {
+      const double an = prm.ax * nx + prm.ay * ny;
+      fk[0] = an * (an >= 0.0 ? wl[0] : wr[0]);
+      bad = !(fk[0] == fk[0]);
+    }
+    const double hl = 0.5 * __ldg(flen + f);
+    double sum[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) sum[v] = hl * (fk[v] + __shfl_xor_sync(0xffffffffu, fk[v], 1));
+    if (act) {
+      if constexpr (NV == 4)
+        reinterpret_cast<double2*>(F + f * 4)[k] = k ? make_double2(sum[2], sum[3]) : make_double2(sum[0], sum[1]);
+      else if (k == 0)
+        F[f] = sum[0];
+      if (bad) flag[inst ? __ldg(inst + cell_of_gauss(il, nQ)) : 0] = 1;  // every writer stores the same value
     }
   }
 }

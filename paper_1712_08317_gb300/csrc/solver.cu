@@ -9,6 +9,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "host_lsq.hpp"
@@ -340,17 +341,18 @@ void launch_face_into(S& s, const void* wg, void* fl, double c, cudaStream_t st)
   in.dt = s.dt_dev;
   in.speed = s.prm.inflow_line[3];
   in.c = c;
-  if constexpr (NV == 4) {  // inflow faces exist for the Euler equations only
-    if (s.n_in) {
-      weno::dev::k_face<T, NV, true><<<grid_of(s.k2, s.nF), s.k2.block, 0, st>>>(
-          (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
-          s.inst, s.nQ, in);
-      return;
-    }
+  // inflow faces exist for the Euler equations only
+  if constexpr (std::is_same<T, double>::value) {
+    const auto kernel = NV == 4 && s.n_in ? weno::dev::k_face_f64<NV, NV == 4> : weno::dev::k_face_f64<NV, false>;
+    kernel<<<grid_of(s.k2, 2 * s.nF), s.k2.block, 0, st>>>(
+        (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
+        s.inst, s.nQ, in);
+  } else {
+    const auto kernel = NV == 4 && s.n_in ? weno::dev::k_face<T, NV, NV == 4> : weno::dev::k_face<T, NV, false>;
+    kernel<<<grid_of(s.k2, s.nF), s.k2.block, 0, st>>>(
+        (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
+        s.inst, s.nQ, in);
   }
-  weno::dev::k_face<T, NV, false><<<grid_of(s.k2, s.nF), s.k2.block, 0, st>>>(
-      (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
-      s.inst, s.nQ, in);
 }
 
 template <typename T, int NV, bool COMP>
@@ -893,6 +895,7 @@ int weno_solver_create(weno_mesh_t mesh, const weno_params* params, void* cuda_s
     d.t_pitch = (d.nT + 7) / 8 * 8;
     if ((r = upload_split<12>(d, tq, d.q_pitch, &d.q_gam, &d.q_wt, &d.q_sig, st))) return r;
     if ((r = upload_split<9>(d, tt, d.t_pitch, &d.t_gam, &d.t_wt, &d.t_sig, st))) return r;
+    d.k2.block = 128;  // a warp for each quarter of an SM: the FP64 pipe is split four ways
     // the FP64 reconstruction's block follows from the mesh (f64_grid) and is not tuned
     if (d.nQ) d.k1q.block = (int)f64_grid(d, d.nQ, d.nv, 12, 4, p.characteristic).threads;
   } else {
