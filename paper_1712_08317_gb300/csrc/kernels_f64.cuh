@@ -9,11 +9,12 @@
 //   - differences, gradients and indicators are computed once per (cell, variable) and shared through
 //     shared memory by the threads of the cell's faces,
 //   - the new indicator is a polynomial in the split weight, two fused multiply-adds,
-//   - reciprocals start from the special-function unit's 20-bit seed and take one third-order step.
-// K1 measured (one pass, before = one thread per (cell, variable) with IEEE division and the splitting
-// repeated by every variable, 5,350 FP64 issue slots a thread on quads; now 535 in each of 4 threads):
-// 17,920 Euler quads 662 -> 277 us, 15,360 triangles 384 -> 144 us (the FP64 pipe busy throughout);
-// 1,600 scalar quads, 332 -> 30 us; 40,000 quads in characteristic variables, 2,151 -> 804 us.
+//   - the nonlinear weights gamma / d^2 are formed on the integer pipe (alpha_f64),
+//   - other reciprocals start from the special-function unit's 20-bit seed and take one third-order step.
+// K1 measured (one pass; first: one thread per (cell, variable), IEEE division, the splitting repeated
+// by every variable, 5,350 FP64 issue slots a thread on quads; then: a thread per face, 535 slots;
+// now: with alpha_f64, about 300): 17,920 Euler quads 662 -> 277 -> 154 us, 15,360 triangles
+// 384 -> 144 -> 83 us, the FP64 pipe busy throughout.
 #pragma once
 
 #include "kernels.cuh"
@@ -92,12 +93,42 @@ __device__ __forceinline__ CandF64 candidate_f64(double m0, double m1, double m2
   return c;
 }
 
+// gamma / d^2 for 0 <= gamma <= 1 and d in [2^-510, 2^400) on the integer pipe, to 0.52 ulp (5 FP64
+// instructions, 320 cycles of a warp, in FP64; here about 55 integer ones and a single-precision
+// reciprocal, none of which the FP64 pipe sees).  With d = m 2^e, m in [1, 2), as the 64-bit fixed-point
+// number M = m 2^63, Newton's iteration r <- r + r (1 - r m) takes 1/m from the reciprocal's seed, biased
+// to stay below it (so that 1 - r m >= 0 and the products are unsigned), to 2^-38 cut to 32 bits and on
+// to 2^-58; then r^2 and r^2 gamma are 64-bit products, and the result is rounded once.  gamma below
+// 2^-1022 and results below it count as zero.
+__device__ __forceinline__ double alpha_f64(double gamma, double d) {
+  const uint32_t dh = hi_word(d), dl = (uint32_t)__double2loint(d), gh = hi_word(gamma), gl = (uint32_t)__double2loint(gamma);
+  const uint32_t mh = 0x80000000u | __funnelshift_l(dl, dh, 11), ml = dl << 11;
+  const float seed = rcp_approx(__uint_as_float(0x3f800000u | ((mh >> 8) & 0x7fffffu)));
+  const uint32_t r0 = __float_as_uint(fmaf(seed, 1.0f - 0x1p-20f, 1.0f)) << 9;  // 2^32 / m, low by 2^-21 to 2^-19
+  const uint64_t e1 = (1ull << 63) - (uint64_t)r0 * mh;                         // < 2^44
+  const uint32_t r1 = r0 + (__umulhi(r0, (uint32_t)(e1 >> 12)) >> 19) - 2u;     // low by at most 2^-29
+  const uint64_t e2 = (1ull << 63) - ((uint64_t)r1 * mh + __umulhi(r1, ml));    // < 2^34
+  const uint64_t r2 = ((uint64_t)r1 << 32) + (((uint64_t)r1 * (uint32_t)(e2 >> 2)) >> 29);  // 2^64 / m
+  const uint32_t rh = (uint32_t)(r2 >> 32), rl = (uint32_t)r2;
+  const uint64_t s = (uint64_t)rh * rh + (((uint64_t)rh * rl) >> 31);           // 2^64 / m^2
+  const uint32_t sh = (uint32_t)(s >> 32), sl = (uint32_t)s;
+  const uint32_t g1 = 0x80000000u | __funnelshift_l(gl, gh, 11), g0 = gl << 11;
+  uint64_t t = (uint64_t)sh * g1 + __umulhi(sh, g0) + __umulhi(sl, g1);         // in (2^61, 2^64)
+  const int lz = __clz((int)(uint32_t)(t >> 32));
+  t <<= lz;
+  const int e = (int)(gh >> 20) - 2 * (int)(dh >> 20) + 2046 - lz;              // biased exponent
+  const uint64_t bits = (t >> 11) + ((t >> 10) & 1u) + ((uint64_t)(uint32_t)(e - 1) << 52);
+  return e <= 0 || gh < 0x00100000u ? 0.0 : __longlong_as_double((long long)bits);
+}
+// The range of d above, as bounds of its high word.
+constexpr uint32_t kAlphaHiMin = (1023u - 510u) << 20, kAlphaHiMax = (1023u + 400u) << 20;
+
 // Increments R(x_G) - W0 at the two Gauss points of one face (Section 3.4), from the candidates
 // cand(j) and the split weights w[h][j * pitch] = (gamma+, gamma-) of point h:
 //   alpha+- = gamma+- / (beta~+- + eps)^2,  beta~+- + eps = (beta + eps) + gamma (beta^2 + gamma beta^3),
 //   R - W0 = sigma+ sum alpha+ p / sum alpha+  -  sigma- sum alpha- p / sum alpha-.
-// 20 FP64 instructions per point and candidate.  Returns false if a square of an indicator left the
-// range of rcp_f64 (or was NaN): the increments are then redone by face_points_ieee.
+// 10 FP64 instructions per point and candidate.  Returns false if an indicator left the range of
+// alpha_f64 (or was NaN): the increments are then redone by face_points_ieee.
 template <int M, int UNROLL, typename Cand>
 __device__ __forceinline__ bool face_points_f64(Cand cand, const double2* __restrict__ w0, const double2* __restrict__ w1,
                                                 int64_t pitch, const double dx[2], const double dy[2],
@@ -112,10 +143,9 @@ __device__ __forceinline__ bool face_points_f64(Cand cand, const double2* __rest
     for (int h = 0; h < 2; ++h) {
       const double p = c.gx * dx[h] + c.gy * dy[h];
       const double dp = fma(w[h].x, fma(w[h].x, c.b3, c.b2), c.be), dn = fma(w[h].y, fma(w[h].y, c.b3, c.b2), c.be);
-      const double sp = dp * dp, sn = dn * dn;
-      lo = min(lo, min(hi_word(sp), hi_word(sn)));
-      hi = max(hi, max(hi_word(sp), hi_word(sn)));
-      const double ap = w[h].x * rcp_f64(sp), an = w[h].y * rcp_f64(sn);
+      lo = min(lo, min(hi_word(dp), hi_word(dn)));
+      hi = max(hi, max(hi_word(dp), hi_word(dn)));
+      const double ap = alpha_f64(w[h].x, dp), an = alpha_f64(w[h].y, dn);
       Ap[h] += ap;
       Bp[h] = fma(ap, p, Bp[h]);
       Am[h] += an;
@@ -124,7 +154,7 @@ __device__ __forceinline__ bool face_points_f64(Cand cand, const double2* __rest
   }
 #pragma unroll
   for (int h = 0; h < 2; ++h) incr[h] = sig[h].x * quotient_f64(Bp[h], Ap[h]) - sig[h].y * quotient_f64(Bm[h], Am[h]);
-  return rcp_safe(lo, hi);
+  return lo >= kAlphaHiMin && hi < kAlphaHiMax;
 }
 
 // The same with IEEE division and the indicator as printed, beta (1 + q + q^2) with q = gamma beta:
