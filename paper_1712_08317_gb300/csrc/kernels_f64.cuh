@@ -12,9 +12,10 @@
 //   - the nonlinear weights gamma / d^2 are formed on the integer pipe (alpha_f64),
 //   - other reciprocals start from the special-function unit's 20-bit seed and take one third-order step.
 // K1 measured (one pass; first: one thread per (cell, variable), IEEE division, the splitting repeated
-// by every variable, 5,350 FP64 issue slots a thread on quads; then: a thread per face, 535 slots;
-// now: with alpha_f64, about 300): 17,920 Euler quads 662 -> 277 -> 154 us, 15,360 triangles
-// 384 -> 144 -> 83 us, the FP64 pipe busy throughout.
+// by every variable, 5,350 FP64 issue slots a (cell, variable) of quads; then: as here with all of the
+// weights in FP64, 2,140 slots; then: gamma / d^2 on the integer pipe, 1,200; now: their sums too, 940):
+// 17,920 Euler quads 662 -> 277 -> 154 -> 124 us, 15,360 triangles 384 -> 144 -> 83 -> 68 us, 1,600 scalar
+// quads 332 -> 30 us and now 18; the FP64 pipe is 86 % busy, the issue slots 32 %.
 #pragma once
 
 #include "kernels.cuh"
@@ -40,12 +41,6 @@ __device__ __forceinline__ double rcp_f64(double x) {
 // that zeros, subnormals, infinities, NaN and negative numbers fail.
 constexpr uint32_t kHiMin = 0x00200000u, kHiMax = 0x7fc00000u;
 __device__ __forceinline__ bool rcp_safe(uint32_t hi_min, uint32_t hi_max) { return hi_min >= kHiMin && hi_max < kHiMax; }
-
-// a / b of two sums of weights: b > 0 unless the weights left the FP64 range.
-__device__ __forceinline__ double quotient_f64(double a, double b) {
-  const uint32_t h = hi_word(b);
-  return rcp_safe(h, h) ? a * rcp_f64(b) : a / b;
-}
 
 // Split linear weights of a group from its linear weights gam [g][j][q] (Section 3.4):
 // gt+ = (gamma + theta |gamma|) / 2, gt- = gt+ - gamma, sigma+- = sum gt+-, gamma+- = gt+- / sigma+-.
@@ -93,87 +88,118 @@ __device__ __forceinline__ CandF64 candidate_f64(double m0, double m1, double m2
   return c;
 }
 
-// gamma / d^2 for 0 <= gamma <= 1 and d in [2^-510, 2^400) on the integer pipe, to 0.52 ulp (5 FP64
-// instructions, 320 cycles of a warp, in FP64; here about 55 integer ones and a single-precision
-// reciprocal, none of which the FP64 pipe sees).  With d = m 2^e, m in [1, 2), as the 64-bit fixed-point
-// number M = m 2^63, Newton's iteration r <- r + r (1 - r m) takes 1/m from the reciprocal's seed, biased
-// to stay below it (so that 1 - r m >= 0 and the products are unsigned), to 2^-38 cut to 32 bits and on
-// to 2^-58; then r^2 and r^2 gamma are 64-bit products, and the result is rounded once.  gamma below
-// 2^-1022 and results below it count as zero.
-__device__ __forceinline__ double alpha_f64(double gamma, double d) {
-  const uint32_t dh = hi_word(d), dl = (uint32_t)__double2loint(d), gh = hi_word(gamma), gl = (uint32_t)__double2loint(gamma);
-  const uint32_t mh = 0x80000000u | __funnelshift_l(dl, dh, 11), ml = dl << 11;
+// Positive numbers t 2^(e - 1086) with a 64-bit t (the value of a biased FP64 exponent e and a mantissa
+// left-justified in t): the nonlinear weights and their sums are formed on the integer pipe, which the
+// FP64 pipe never sees.
+struct PosNum { uint64_t t; int e; };
+
+// 2^64 / m for m = (mh, ml) / 2^63 in [1, 2), low by at most 2^-58: Newton's iteration r <- r + r (1 - r m)
+// from the single-precision reciprocal's seed, biased to stay below 1/m (so that 1 - r m >= 0 and all
+// products are unsigned), to 2^-38 cut to 32 bits and on to 2^-58.
+__device__ __forceinline__ uint64_t recip_fixed(uint32_t mh, uint32_t ml) {
   const float seed = rcp_approx(__uint_as_float(0x3f800000u | ((mh >> 8) & 0x7fffffu)));
-  const uint32_t r0 = __float_as_uint(fmaf(seed, 1.0f - 0x1p-20f, 1.0f)) << 9;  // 2^32 / m, low by 2^-21 to 2^-19
+  const uint32_t r0 = __float_as_uint(fmaf(seed, 1.0f - 0x1p-20f, 1.0f)) << 9;  // low by 2^-21 to 2^-19
   const uint64_t e1 = (1ull << 63) - (uint64_t)r0 * mh;                         // < 2^44
   const uint32_t r1 = r0 + (__umulhi(r0, (uint32_t)(e1 >> 12)) >> 19) - 2u;     // low by at most 2^-29
   const uint64_t e2 = (1ull << 63) - ((uint64_t)r1 * mh + __umulhi(r1, ml));    // < 2^34
-  const uint64_t r2 = ((uint64_t)r1 << 32) + (((uint64_t)r1 * (uint32_t)(e2 >> 2)) >> 29);  // 2^64 / m
-  const uint32_t rh = (uint32_t)(r2 >> 32), rl = (uint32_t)r2;
-  const uint64_t s = (uint64_t)rh * rh + (((uint64_t)rh * rl) >> 31);           // 2^64 / m^2
+  return ((uint64_t)r1 << 32) + (((uint64_t)r1 * (uint32_t)(e2 >> 2)) >> 29);
+}
+
+// FP64 value of t 2^(e - 1086) with the top bit of t set, rounded to nearest (halves away from zero);
+// zero below the normal range.
+__device__ __forceinline__ double pos_to_f64(uint64_t t, int e) {
+  const uint64_t bits = (t >> 11) + ((t >> 10) & 1u) + ((uint64_t)(uint32_t)(e - 1) << 52);
+  return e <= 0 ? 0.0 : __longlong_as_double((long long)bits);
+}
+
+// gamma / d^2 for 0 <= gamma <= 1 and d in [2^-510, 2^400): 5 FP64 instructions, 320 cycles of a warp, in
+// FP64; here about 55 integer ones and a single-precision reciprocal, good to 2^-57.  gamma below 2^-1022
+// comes out smaller than 2^-900 of any weight that matters.
+__device__ __forceinline__ PosNum alpha_f64(double gamma, double d) {
+  const uint32_t dh = hi_word(d), dl = (uint32_t)__double2loint(d), gh = hi_word(gamma), gl = (uint32_t)__double2loint(gamma);
+  const uint64_t r = recip_fixed(0x80000000u | __funnelshift_l(dl, dh, 11), dl << 11);
+  const uint32_t rh = (uint32_t)(r >> 32), rl = (uint32_t)r;
+  const uint64_t s = (uint64_t)rh * rh + (((uint64_t)rh * rl) >> 31);  // 2^64 / m^2
   const uint32_t sh = (uint32_t)(s >> 32), sl = (uint32_t)s;
   const uint32_t g1 = 0x80000000u | __funnelshift_l(gl, gh, 11), g0 = gl << 11;
-  uint64_t t = (uint64_t)sh * g1 + __umulhi(sh, g0) + __umulhi(sl, g1);         // in (2^61, 2^64)
+  const uint64_t t = (uint64_t)sh * g1 + __umulhi(sh, g0) + __umulhi(sl, g1);  // in (2^61, 2^64)
   const int lz = __clz((int)(uint32_t)(t >> 32));
-  t <<= lz;
-  const int e = (int)(gh >> 20) - 2 * (int)(dh >> 20) + 2046 - lz;              // biased exponent
-  const uint64_t bits = (t >> 11) + ((t >> 10) & 1u) + ((uint64_t)(uint32_t)(e - 1) << 52);
-  return e <= 0 || gh < 0x00100000u ? 0.0 : __longlong_as_double((long long)bits);
+  return PosNum{t << lz, (int)(gh >> 20) - 2 * (int)(dh >> 20) + 2046 - lz};
 }
 // The range of d above, as bounds of its high word.
 constexpr uint32_t kAlphaHiMin = (1023u - 510u) << 20, kAlphaHiMax = (1023u + 400u) << 20;
 
-// Increments R(x_G) - W0 at the two Gauss points of one face (Section 3.4), from the candidates
-// cand(j) and the split weights w[h][j * pitch] = (gamma+, gamma-) of point h:
+// Sum of up to 16 weights: four bits of headroom in t instead of a carry, so 2^-59 of the sum is lost.
+__device__ __forceinline__ PosNum pos_first(PosNum a) { return PosNum{a.t >> 4, a.e}; }
+__device__ __forceinline__ PosNum pos_add(PosNum s, PosNum a) {
+  const int de = s.e - a.e;
+  const uint64_t t = a.t >> 4;
+  const uint64_t big = de < 0 ? t : s.t, small = de < 0 ? s.t : t;
+  return PosNum{big + (small >> min(abs(de), 63)), max(s.e, a.e)};
+}
+// Reciprocal of such a sum.
+__device__ __forceinline__ double pos_rcp(PosNum s) {
+  const int lz = __clzll((long long)s.t);
+  const uint64_t m = s.t << lz;
+  uint64_t r = recip_fixed((uint32_t)(m >> 32), (uint32_t)m);
+  const int low = (int)(r >> 63) ^ 1;  // r falls just short of 2^63 where m is next to 2
+  return pos_to_f64(r << low, 2041 - s.e + lz - low);
+}
+
+// Increments R(x_G) - W0 at PTS Gauss points of one face (Section 3.4), from the candidates cand(j) and
+// the split weights w[j * pitch] = (gamma+, gamma-) of the first point, step entries on for the second:
 //   alpha+- = gamma+- / (beta~+- + eps)^2,  beta~+- + eps = (beta + eps) + gamma (beta^2 + gamma beta^3),
 //   R - W0 = sigma+ sum alpha+ p / sum alpha+  -  sigma- sum alpha- p / sum alpha-.
-// 10 FP64 instructions per point and candidate.  Returns false if an indicator left the range of
+// 8 FP64 instructions per point and candidate.  Returns false if an indicator left the range of
 // alpha_f64 (or was NaN): the increments are then redone by face_points_ieee.
-template <int M, int UNROLL, typename Cand>
-__device__ __forceinline__ bool face_points_f64(Cand cand, const double2* __restrict__ w0, const double2* __restrict__ w1,
-                                                int64_t pitch, const double dx[2], const double dy[2],
-                                                const double2 sig[2], double incr[2]) {
-  double Ap[2] = {0.0, 0.0}, Bp[2] = {0.0, 0.0}, Am[2] = {0.0, 0.0}, Bm[2] = {0.0, 0.0};
+template <int M, int PTS, typename Cand>
+__device__ __forceinline__ bool face_points_f64(Cand cand, const double2* __restrict__ w, int64_t step, int64_t pitch,
+                                                const double* dx, const double* dy, const double2* sig, double* incr) {
+  PosNum Ap[PTS], Am[PTS];
+  double Bp[PTS], Bm[PTS];
   uint32_t lo = 0xffffffffu, hi = 0u;
-#pragma unroll UNROLL
-  for (int j = 0; j < M; ++j) {
+  auto one = [&](int j, bool first) {
     const CandF64 c = cand(j);
-    const double2 w[2] = {__ldg(w0 + j * pitch), __ldg(w1 + j * pitch)};
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < PTS; ++h) {
+      const double2 g = __ldg(w + h * step + j * pitch);
       const double p = c.gx * dx[h] + c.gy * dy[h];
-      const double dp = fma(w[h].x, fma(w[h].x, c.b3, c.b2), c.be), dn = fma(w[h].y, fma(w[h].y, c.b3, c.b2), c.be);
+      const double dp = fma(g.x, fma(g.x, c.b3, c.b2), c.be), dn = fma(g.y, fma(g.y, c.b3, c.b2), c.be);
       lo = min(lo, min(hi_word(dp), hi_word(dn)));
       hi = max(hi, max(hi_word(dp), hi_word(dn)));
-      const double ap = alpha_f64(w[h].x, dp), an = alpha_f64(w[h].y, dn);
-      Ap[h] += ap;
-      Bp[h] = fma(ap, p, Bp[h]);
-      Am[h] += an;
-      Bm[h] = fma(an, p, Bm[h]);
+      const PosNum ap = alpha_f64(g.x, dp), an = alpha_f64(g.y, dn);
+      const double vp = pos_to_f64(ap.t, ap.e), vn = pos_to_f64(an.t, an.e);
+      Ap[h] = first ? pos_first(ap) : pos_add(Ap[h], ap);
+      Am[h] = first ? pos_first(an) : pos_add(Am[h], an);
+      Bp[h] = first ? vp * p : fma(vp, p, Bp[h]);
+      Bm[h] = first ? vn * p : fma(vn, p, Bm[h]);
     }
-  }
+  };
+  one(0, true);
+#pragma unroll 2
+  for (int j = 1; j < M; ++j) one(j, false);
 #pragma unroll
-  for (int h = 0; h < 2; ++h) incr[h] = sig[h].x * quotient_f64(Bp[h], Ap[h]) - sig[h].y * quotient_f64(Bm[h], Am[h]);
+  for (int h = 0; h < PTS; ++h) incr[h] = sig[h].x * (Bp[h] * pos_rcp(Ap[h])) - sig[h].y * (Bm[h] * pos_rcp(Am[h]));
   return lo >= kAlphaHiMin && hi < kAlphaHiMax;
 }
 
 // The same with IEEE division and the indicator as printed, beta (1 + q + q^2) with q = gamma beta:
 // for indicators whose powers leave the FP64 range, and NaN states.
-template <int M, typename Cand>
-__device__ __forceinline__ void face_points_ieee(Cand cand, const double2* __restrict__ w0, const double2* __restrict__ w1,
-                                                 int64_t pitch, const double dx[2], const double dy[2],
-                                                 const double2 sig[2], double a0, double eps, double incr[2]) {
+template <int M, int PTS, typename Cand>
+__device__ __forceinline__ void face_points_ieee(Cand cand, const double2* __restrict__ w, int64_t step, int64_t pitch,
+                                                 const double* dx, const double* dy, const double2* sig, double a0,
+                                                 double eps, double* incr) {
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < PTS; ++h) {
     double Ap = 0.0, Bp = 0.0, Am = 0.0, Bm = 0.0;
 #pragma unroll 1
     for (int j = 0; j < M; ++j) {
       const CandF64 c = cand(j);
-      const double2 w = __ldg((h ? w1 : w0) + j * pitch);
+      const double2 g = __ldg(w + h * step + j * pitch);
       const double p = c.gx * dx[h] + c.gy * dy[h], b = a0 * (c.gx * c.gx + c.gy * c.gy);
-      const double qp = w.x * b, qn = w.y * b;
+      const double qp = g.x * b, qn = g.y * b;
       const double dp = b * (1.0 + qp + qp * qp) + eps, dn = b * (1.0 + qn + qn * qn) + eps;
-      const double ap = w.x / (dp * dp), an = w.y / (dn * dn);
+      const double ap = g.x / (dp * dp), an = g.y / (dn * dn);
       Ap += ap;
       Bp += ap * p;
       Am += an;
@@ -184,24 +210,27 @@ __device__ __forceinline__ void face_points_ieee(Cand cand, const double2* __res
 }
 
 // Layout of a block of either kernel: `width` = cells x variables of its tile; thread t holds column
-// t % width (cell (t % width) / NV, variable or field t % NV) and face t / width of the cell.
+// t % width (cell (t % width) / NV, variable or field t % NV) and, of the cell's G Gauss points, one, or
+// in characteristic variables PTS, from PTS (t / width) on.
 constexpr int kF64MaxWidth = 32;
 
-// Component-wise FP64 K1.  A thread gathers 3 of its column's M stencil differences, then forms 3 of
-// its M candidates, both into shared memory, then evaluates the two Gauss points of its face.
+// Component-wise FP64 K1.  The threads of a column share out its M stencil differences, then its M
+// candidates, both into shared memory; then each evaluates its Gauss point.  A thread a point: no FP64
+// instruction is repeated (a warp takes whole shares of the candidates), 62 registers leave 30 warps an
+// SM, and the last wave is short (with both points of a face in a thread, 96 registers and 16 to 19
+// warps: triangles 79 us a pass on the mesh above against 68, quads 124 either way).
 template <int NV, int M, int G, bool WALLS>
-__global__ void __launch_bounds__(kF64MaxWidth * G / 2) k_reconstruct_f64(
+__global__ void __launch_bounds__(kF64MaxWidth * G) k_reconstruct_f64(
     const double* __restrict__ U, const int32_t* __restrict__ slot, const double* __restrict__ gop,
     const double* __restrict__ dg, const double* __restrict__ gam, const double2* __restrict__ wt,
     const double2* __restrict__ sigma, const double* __restrict__ area, int64_t N, int64_t pitch, int64_t first,
     int64_t gbase, double* __restrict__ Wg, double eps, int linear, int width) {
-  constexpr int F = G / 2, PER = M / F;
-  static_assert(PER * F == M, "each face's threads take an equal share of the slots and candidates");
+  constexpr int PER = (M + G - 1) / G;
   extern __shared__ double sm[];
   double* dW = sm;                                      // [slot - 1][column]
   double *gx = sm + M * width, *gy = gx + M * width;    // [candidate][column]
   double *be = gy + M * width, *b2 = be + M * width, *b3 = b2 + M * width;
-  const int col = threadIdx.x % width, face = threadIdx.x / width, v = col % NV;
+  const int col = threadIdx.x % width, g = threadIdx.x / width, v = col % NV;
   const int64_t qr = (int64_t)blockIdx.x * (width / NV) + col / NV;
   const int64_t q = qr < N ? qr : N - 1;  // columns past the end work on the last cell and store nothing
   const int64_t c = first + q;
@@ -209,14 +238,15 @@ __global__ void __launch_bounds__(kF64MaxWidth * G / 2) k_reconstruct_f64(
   const int32_t fm = flip_mask<WALLS, NV>(v);
 #pragma unroll
   for (int i = 0; i < PER; ++i) {
-    const int s = face * PER + i;
-    dW[s * width + col] =
+    const int s = g + i * G;
+    if (s < M) dW[s * width + col] =
         slot_delta<double, NV, WALLS, false>(U, nullptr, __ldg(slot + (int64_t)s * N + q), v, fm, w0, 0.0);
   }
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < PER; ++i) {
-    const int j = face * PER + i;
+    const int j = g + i * G;
+    if (j >= M) break;
     const double* o = gop + (int64_t)(j * 4) * N + q;
     const CandF64 cd = candidate_f64(__ldg(o), __ldg(o + N), __ldg(o + 2 * N), __ldg(o + 3 * N),
                                      dW[(sub_a<M>(j) - 1) * width + col], dW[(sub_b<M>(j) - 1) * width + col], a0, eps);
@@ -224,33 +254,24 @@ __global__ void __launch_bounds__(kF64MaxWidth * G / 2) k_reconstruct_f64(
     gx[k] = cd.gx; gy[k] = cd.gy; be[k] = cd.be; b2[k] = cd.b2; b3[k] = cd.b3;
   }
   __syncthreads();
-  const int g = 2 * face;
-  const double* d = dg + (int64_t)(2 * g) * N + q;
-  const double dx[2] = {__ldg(d), __ldg(d + 2 * N)}, dy[2] = {__ldg(d + N), __ldg(d + 3 * N)};
-  double incr[2] = {0.0, 0.0};
+  const double dx = __ldg(dg + (int64_t)(2 * g) * N + q), dy = __ldg(dg + (int64_t)(2 * g + 1) * N + q);
+  double incr = 0.0;
   if (linear) {
     const double* gg = gam + (int64_t)(g * M) * N + q;
 #pragma unroll 3
-    for (int j = 0; j < M; ++j) {
-      const double x = gx[j * width + col], y = gy[j * width + col];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) incr[h] += __ldg(gg + (int64_t)(h * M + j) * N) * (x * dx[h] + y * dy[h]);
-    }
+    for (int j = 0; j < M; ++j)
+      incr += __ldg(gg + (int64_t)j * N) * (gx[j * width + col] * dx + gy[j * width + col] * dy);
   } else {
     auto cand = [&](int j) {
       const int k = j * width + col;
       return CandF64{gx[k], gy[k], be[k], b2[k], b3[k]};
     };
-    const double2 *wa = wt + (int64_t)(g * M) * pitch + q, *wb = wa + (int64_t)M * pitch;
-    const double2 sig[2] = {__ldg(sigma + (int64_t)g * pitch + q), __ldg(sigma + (int64_t)(g + 1) * pitch + q)};
-    if (!face_points_f64<M, 3>(cand, wa, wb, pitch, dx, dy, sig, incr))
-      face_points_ieee<M>(cand, wa, wb, pitch, dx, dy, sig, a0, eps, incr);
+    const double2* w = wt + (int64_t)(g * M) * pitch + q;
+    const double2 sig = __ldg(sigma + (int64_t)g * pitch + q);
+    if (!face_points_f64<M, 1>(cand, w, 0, pitch, &dx, &dy, &sig, &incr))
+      face_points_ieee<M, 1>(cand, w, 0, pitch, &dx, &dy, &sig, a0, eps, &incr);
   }
-  if (qr < N) {
-    double* out = Wg + (gbase + q * G + g) * NV + v;
-    out[0] = w0 + incr[0];
-    out[NV] = w0 + incr[1];
-  }
+  if (qr < N) Wg[(gbase + q * G + g) * NV + v] = w0 + incr;
 }
 
 // 1/sqrt(x), last-bit accurate: with e = 1 - x y0^2 from the 20-bit seed y0 of rsqrt.approx.ftz.f64,
@@ -310,25 +331,27 @@ __device__ __forceinline__ void roe_frame_f64(const double Wl[4], const double W
 }
 
 // FP64 K1 in characteristic variables (see the comment at the FP32C kernels below for the method).
-// Thread (cell, field l, face): the block's first threads build the Roe frames, one thread a frame
+// Thread (cell, field l, PTS points of a face): the two points share the projection and the candidates,
+// 168 of about 470 FP64 instructions, so they go to two threads only on meshes too small to fill the
+// FP64 pipe otherwise (f64_grid).  The block's first threads build the Roe frames, one thread a frame
 // instead of four lanes each repeating it; every thread projects the shared stencil differences onto
-// its field with row l of R^-1, evaluates its face's two points, and returns variable l of R dU.
+// its field with row l of R^-1, evaluates its points, and returns variable l of R dU there.
 constexpr int kFrame = 33;  // doubles a frame takes in shared memory (32, padded against bank conflicts)
 
-template <int M, int G, bool WALLS>
-__global__ void __launch_bounds__(kF64MaxWidth * G / 2) k_reconstruct_char_f64(
+template <int M, int G, int PTS, bool WALLS>
+__global__ void __launch_bounds__(kF64MaxWidth * G / PTS) k_reconstruct_char_f64(
     const double* __restrict__ U, const int32_t* __restrict__ slot, const double* __restrict__ gop,
     const double* __restrict__ dg, const double* __restrict__ gam, const double2* __restrict__ wt,
     const double2* __restrict__ sigma, const double* __restrict__ area, int64_t N, int64_t pitch, int64_t first,
     int64_t gbase, double* __restrict__ Wg, double eps, double gas_gamma, int linear, int width) {
-  constexpr int F = G / 2, PER = M / F;
+  constexpr int F = G / 2, PARTS = G / PTS, PER = (M + PARTS - 1) / PARTS;
   extern __shared__ double sm[];
-  const int tile = width / 4, threads = width * F;
+  const int tile = width / 4, threads = width * PARTS;
   double* dW = sm;                      // [slot - 1][column]
   double* dU = dW + M * width;          // [slot - 1][thread]
   double* fr = dU + M * threads;        // [face][cell] frames
   double* inc = fr + kFrame * tile * F; // [point][thread]
-  const int t = threadIdx.x, col = t % width, face = t / width, l = col % 4, cl = col / 4;
+  const int t = threadIdx.x, col = t % width, part = t / width, l = col % 4, cl = col / 4;
   const int64_t q0 = (int64_t)blockIdx.x * tile, qr = q0 + cl;
   const int64_t q = qr < N ? qr : N - 1;  // columns past the end work on the last cell and store nothing
   const int64_t c = first + q;
@@ -336,8 +359,8 @@ __global__ void __launch_bounds__(kF64MaxWidth * G / 2) k_reconstruct_char_f64(
   const int32_t fm = flip_mask<WALLS, 4>(l);
 #pragma unroll
   for (int i = 0; i < PER; ++i) {
-    const int s = face * PER + i;
-    dW[s * width + col] =
+    const int s = part + i * PARTS;
+    if (s < M) dW[s * width + col] =
         slot_delta<double, 4, WALLS, false>(U, nullptr, __ldg(slot + (int64_t)s * N + q), l, fm, w0, 0.0);
   }
   if (t < tile * F) {  // frame of face t / tile of cell t % tile; the neighbour across face k is slot k + 1
@@ -350,44 +373,51 @@ __global__ void __launch_bounds__(kF64MaxWidth * G / 2) k_reconstruct_char_f64(
     roe_frame_f64(Wl, Wn, __ldg(d + 2 * N) - __ldg(d), __ldg(d + 3 * N) - __ldg(d + N), gas_gamma - 1.0, fr + kFrame * t);
   }
   __syncthreads();
-  const double* f0 = fr + kFrame * (face * tile + cl);
+  const double* f0 = fr + kFrame * (part * PTS / 2 * tile + cl);
   const double L0 = f0[4 * l], L1 = f0[4 * l + 1], L2 = f0[4 * l + 2], L3 = f0[4 * l + 3];
 #pragma unroll 4
   for (int s = 0; s < M; ++s) {
     const double* x = dW + s * width + 4 * cl;
     dU[s * threads + t] = L0 * x[0] + L1 * x[1] + L2 * x[2] + L3 * x[3];
   }
-  const int g = 2 * face;
+  const int g = PTS * part;
   const double* d = dg + (int64_t)(2 * g) * N + q;
-  const double dx[2] = {__ldg(d), __ldg(d + 2 * N)}, dy[2] = {__ldg(d + N), __ldg(d + 3 * N)};
+  double dx[PTS], dy[PTS], incr[PTS];
+#pragma unroll
+  for (int h = 0; h < PTS; ++h) {
+    dx[h] = __ldg(d + 2 * h * N);
+    dy[h] = __ldg(d + (2 * h + 1) * N);
+    incr[h] = 0.0;
+  }
   auto cand = [&](int j) {
     const double* o = gop + (int64_t)(j * 4) * N + q;
     return candidate_f64(__ldg(o), __ldg(o + N), __ldg(o + 2 * N), __ldg(o + 3 * N),
                          dU[(sub_a<M>(j) - 1) * threads + t], dU[(sub_b<M>(j) - 1) * threads + t], a0, eps);
   };
-  double incr[2] = {0.0, 0.0};
   if (linear) {
     const double* gg = gam + (int64_t)(g * M) * N + q;
 #pragma unroll 3
     for (int j = 0; j < M; ++j) {
       const CandF64 x = cand(j);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) incr[h] += __ldg(gg + (int64_t)(h * M + j) * N) * (x.gx * dx[h] + x.gy * dy[h]);
+      for (int h = 0; h < PTS; ++h) incr[h] += __ldg(gg + (int64_t)(h * M + j) * N) * (x.gx * dx[h] + x.gy * dy[h]);
     }
   } else {
-    const double2 *wa = wt + (int64_t)(g * M) * pitch + q, *wb = wa + (int64_t)M * pitch;
-    const double2 sig[2] = {__ldg(sigma + (int64_t)g * pitch + q), __ldg(sigma + (int64_t)(g + 1) * pitch + q)};
-    if (!face_points_f64<M, 3>(cand, wa, wb, pitch, dx, dy, sig, incr))
-      face_points_ieee<M>(cand, wa, wb, pitch, dx, dy, sig, a0, eps, incr);
+    const double2* w = wt + (int64_t)(g * M) * pitch + q;
+    double2 sig[PTS];
+#pragma unroll
+    for (int h = 0; h < PTS; ++h) sig[h] = __ldg(sigma + (int64_t)(g + h) * pitch + q);
+    if (!face_points_f64<M, PTS>(cand, w, (int64_t)M * pitch, pitch, dx, dy, sig, incr))
+      face_points_ieee<M, PTS>(cand, w, (int64_t)M * pitch, pitch, dx, dy, sig, a0, eps, incr);
   }
-  inc[t] = incr[0];
-  inc[threads + t] = incr[1];
+#pragma unroll
+  for (int h = 0; h < PTS; ++h) inc[h * threads + t] = incr[h];
   __syncthreads();
   if (qr < N) {  // variable l of R dU
     const double* r = f0 + 16 + 4 * l;
     double* out = Wg + (gbase + q * G + g) * 4 + l;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < PTS; ++h) {
       const double* x = inc + h * threads + (t & ~3);
       out[h * 4] = w0 + (r[0] * x[0] + r[1] * x[1] + r[2] * x[2] + r[3] * x[3]);
     }

@@ -189,22 +189,25 @@ unsigned fix_grid(const S& s, int64_t n) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(chunks, 4 * s.nsm));
 }
 
-// Grid of an FP64 reconstruction over n cells of F faces and M candidates: blocks of `width` (cell,
-// variable) columns, one thread per column and face, with the kernel's shared memory.  The FP64 pipe is
-// the bound, so the SMs have to share the columns evenly: tiles shrink from 32 columns to 8 until every
-// SM has four blocks.
+// Grid of an FP64 reconstruction over n cells of G Gauss points and M candidates: blocks of `width` (cell,
+// variable) columns with a thread for every pts points of a column, and the kernel's shared memory.  The
+// FP64 pipe, split between the quarters of the SMs, is the bound and has to be shared out evenly: tiles
+// shrink from 32 columns to 8 until every SM has four blocks (1,600 scalar quads: 18 us with 8 columns),
+// and in characteristic variables the two points of a face go to two threads below four warps for every
+// quarter.
 struct F64Grid {
-  int width;
+  int width, pts;
   unsigned blocks, threads;
   size_t smem;
 };
-F64Grid f64_grid(const S& s, int64_t n, int nv, int M, int F, bool characteristic) {
+F64Grid f64_grid(const S& s, int64_t n, int nv, int M, int G, bool characteristic) {
+  const int pts = !characteristic || n * nv * (G / 2) < (int64_t)4 * 4 * 32 * s.nsm ? 1 : 2;
   int width = weno::dev::kF64MaxWidth;
   while (width > 8 && n * nv < (int64_t)4 * s.nsm * width) width /= 2;
-  const int tile = width / nv;
-  const size_t doubles = characteristic ? (size_t)M * width + (size_t)(M + 2) * width * F + weno::dev::kFrame * tile * F
+  const int tile = width / nv, threads = width * G / pts;
+  const size_t doubles = characteristic ? (size_t)M * width + (size_t)(M + pts) * threads + weno::dev::kFrame * tile * (G / 2)
                                         : (size_t)6 * M * width;
-  return {width, (unsigned)((n + tile - 1) / tile), (unsigned)(width * F), doubles * sizeof(double)};
+  return {width, pts, (unsigned)((n + tile - 1) / tile), (unsigned)threads, doubles * sizeof(double)};
 }
 
 // Cell reconstruction into the Gauss-value array wg.  which: bit 0 = quad group,
@@ -243,14 +246,18 @@ void launch_reconstruct_impl(S& s, const void* U, const void* Ulo, void* wg, cud
         }
       } else {
         if (s.nQ && (which & 1)) {
-          const F64Grid g = f64_grid(s, s.nQ, 4, 12, 4, true);
-          weno::dev::k_reconstruct_char_f64<12, 8, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
+          const F64Grid g = f64_grid(s, s.nQ, 4, 12, 8, true);
+          const auto kernel = g.pts == 1 ? weno::dev::k_reconstruct_char_f64<12, 8, 1, WALLS>
+                                         : weno::dev::k_reconstruct_char_f64<12, 8, 2, WALLS>;
+          kernel<<<g.blocks, g.threads, g.smem, st>>>(
               u, s.q_slot, (const double*)s.q_gop, (const double*)s.q_dg, (const double*)s.q_gam, s.q_wt, s.q_sig,
               (const double*)s.area, s.nQ, s.q_pitch, 0, 0, (double*)wg, eps, gg, s.prm.linear, g.width);
         }
         if (s.nT && (which & 2)) {
-          const F64Grid g = f64_grid(s, s.nT, 4, 9, 3, true);
-          weno::dev::k_reconstruct_char_f64<9, 6, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
+          const F64Grid g = f64_grid(s, s.nT, 4, 9, 6, true);
+          const auto kernel = g.pts == 1 ? weno::dev::k_reconstruct_char_f64<9, 6, 1, WALLS>
+                                         : weno::dev::k_reconstruct_char_f64<9, 6, 2, WALLS>;
+          kernel<<<g.blocks, g.threads, g.smem, st>>>(
               u, s.t_slot, (const double*)s.t_gop, (const double*)s.t_dg, (const double*)s.t_gam, s.t_wt, s.t_sig,
               (const double*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (double*)wg, eps, gg, s.prm.linear, g.width);
         }
@@ -296,13 +303,13 @@ void launch_reconstruct_impl(S& s, const void* U, const void* Ulo, void* wg, cud
           s.prm.linear);
   } else {
     if (s.nQ && (which & 1)) {
-      const F64Grid g = f64_grid(s, s.nQ, NV, 12, 4, false);
+      const F64Grid g = f64_grid(s, s.nQ, NV, 12, 8, false);
       weno::dev::k_reconstruct_f64<NV, 12, 8, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
           u, s.q_slot, (const double*)s.q_gop, (const double*)s.q_dg, (const double*)s.q_gam, s.q_wt, s.q_sig,
           (const double*)s.area, s.nQ, s.q_pitch, 0, 0, (double*)wg, eps, s.prm.linear, g.width);
     }
     if (s.nT && (which & 2)) {
-      const F64Grid g = f64_grid(s, s.nT, NV, 9, 3, false);
+      const F64Grid g = f64_grid(s, s.nT, NV, 9, 6, false);
       weno::dev::k_reconstruct_f64<NV, 9, 6, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
           u, s.t_slot, (const double*)s.t_gop, (const double*)s.t_dg, (const double*)s.t_gam, s.t_wt, s.t_sig,
           (const double*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (double*)wg, eps, s.prm.linear, g.width);
@@ -897,7 +904,7 @@ int weno_solver_create(weno_mesh_t mesh, const weno_params* params, void* cuda_s
     if ((r = upload_split<9>(d, tt, d.t_pitch, &d.t_gam, &d.t_wt, &d.t_sig, st))) return r;
     d.k2.block = 128;  // a warp for each quarter of an SM: the FP64 pipe is split four ways
     // the FP64 reconstruction's block follows from the mesh (f64_grid) and is not tuned
-    if (d.nQ) d.k1q.block = (int)f64_grid(d, d.nQ, d.nv, 12, 4, p.characteristic).threads;
+    if (d.nQ) d.k1q.block = (int)f64_grid(d, d.nQ, d.nv, 12, 8, p.characteristic).threads;
   } else {
     d.q_pitch = (d.nQ + 63) / 64 * 64;
     d.t_pitch = (d.nT + 63) / 64 * 64;
