@@ -10,12 +10,14 @@
 //                             per cell exchange variables by shuffles)
 //     k_reconstruct_f64, k_reconstruct_char_f64   FP64 (kernels_f64.cuh): a
 //                             thread per (cell, variable, face)
-//   k_face         one thread per face: two Gauss points, rotated HLLC (Euler) or
-//                  upwind (scalar) flux, |l|/2 (F1 + F2) (Eqs. 5-6); at reflective
-//                  walls the outer state is the inner one mirrored, at inflow faces
-//                  the prescribed state at the stage time.
-//   k_gather       one thread per cell: signed gather of its face fluxes
+//   K2 (face fluxes, Eqs. 5-6): two Gauss points a face, rotated HLLC (Euler) or
+//                  upwind (scalar), |l|/2 (F1 + F2); at reflective walls the outer
+//                  state is the inner one mirrored, at inflow faces the prescribed
+//                  state at the stage time: k_face_f64, k_face_f32, k_face_scalar.
+//   K3 k_gather    one thread per cell: signed gather of its face fluxes
 //                  (Eq. 4, no atomics) fused with the RK3 stage (Section 4).
+//   K2 + K3 k_update_f32c   FP32C Euler, small meshes: fluxes, gather and stage
+//                  in one pass.
 //   k_advance_time after the third stage of a step: t += dt per instance.
 // The reconstruction kernels take WALLS = true on meshes with reflective walls:
 // stencil entries then carry momentum flips for mirror images.
@@ -754,7 +756,7 @@ template <typename T> struct FluxMath {
 #if WENO_K2_FAST
 template <> struct FluxMath<float> {
   static __device__ __forceinline__ float rcp(float x) { return rcp_approx(x); }
-  static __device__ __forceinline__ float div(float a, float b) { return a * rcp_approx(b); }
+  static __device__ __forceinline__ float div(float a, float b) { return __fmul_rn(a, rcp_approx(b)); }
   static __device__ __forceinline__ float sqr(float x) {
     float r;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -763,63 +765,50 @@ template <> struct FluxMath<float> {
 };
 #endif
 
-template <typename T>
-__device__ __forceinline__ void euler_x_flux(T r, T un, T ut, T E, T p, T f[4]) {
-  f[0] = r * un;
-  f[1] = r * un * un + p;
-  f[2] = r * un * ut;
-  f[3] = (E + p) * un;
-}
+// Products that the compiler may not merge into a following addition.
+__device__ __forceinline__ float mulr(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mulr(double a, double b) { return __dmul_rn(a, b); }
 
-// HLLC in the frame of the unit normal (nx, ny); returns the flux rotated back.
+// HLLC in the frame of the unit normal (nx, ny); returns the flux rotated back.  The side of the contact
+// is taken by selection, not by branches: a warp's faces rarely agree on one.  Every product is either
+// inside an explicit fma or rounded, so that a flux has the same bits in whichever kernel it is inlined
+// (k_face_f32 and k_update_f32c: a mesh alone and as part of a larger batch give the same results).
 template <typename T>
 __device__ __forceinline__ void hllc(const T wl[4], const T wr[4], T nx, T ny, T gam, T out[4], bool& bad) {
-  const T rl = wl[0], rr = wr[0];
   using FM = FluxMath<T>;
-  const T irl = FM::rcp(rl), irr = FM::rcp(rr);
-  const T ul = (wl[1] * nx + wl[2] * ny) * irl, vl = (wl[2] * nx - wl[1] * ny) * irl;
-  const T ur = (wr[1] * nx + wr[2] * ny) * irr, vr = (wr[2] * nx - wr[1] * ny) * irr;
-  const T pl = (gam - T(1)) * (wl[3] - T(0.5) * rl * (ul * ul + vl * vl));
-  const T pr = (gam - T(1)) * (wr[3] - T(0.5) * rr * (ur * ur + vr * vr));
-  bad |= !(rl > T(0)) || !(rr > T(0)) || !(pl > T(0)) || !(pr > T(0)) || !(wl[3] == wl[3]) || !(wr[3] == wr[3]);
-  const T cl = FM::sqr(gam * pl * irl), cr = FM::sqr(gam * pr * irr);
+  const T gm1 = gam - T(1);
+  const T rl = wl[0], rr = wr[0], El = wl[3], Er = wr[3];
+  const T il = FM::rcp(rl), ir = FM::rcp(rr);
+  const T nl = fma(wl[1], nx, mulr(wl[2], ny)), tl = fma(wl[2], nx, -mulr(wl[1], ny));  // normal and tangential
+  const T nr = fma(wr[1], nx, mulr(wr[2], ny)), tr = fma(wr[2], nx, -mulr(wr[1], ny));  // momentum
+  const T ul = mulr(nl, il), vl = mulr(tl, il), ur = mulr(nr, ir), vr = mulr(tr, ir);
+  const T pl = mulr(gm1, fma(-mulr(T(0.5), rl), fma(ul, ul, mulr(vl, vl)), El));
+  const T pr = mulr(gm1, fma(-mulr(T(0.5), rr), fma(ur, ur, mulr(vr, vr)), Er));
+  bad |= !(rl > T(0) && rr > T(0) && pl > T(0) && pr > T(0));  // a NaN fails; a NaN energy shows in p
+  const T cl = FM::sqr(mulr(mulr(gam, pl), il)), cr = FM::sqr(mulr(mulr(gam, pr), ir));
   // Roe averages
   const T sl = FM::sqr(rl), sr = FM::sqr(rr), iw = FM::rcp(sl + sr);
-  const T ua = (sl * ul + sr * ur) * iw, va = (sl * vl + sr * vr) * iw;
-  const T Hl = (wl[3] + pl) * irl, Hr = (wr[3] + pr) * irr;
-  const T Ha = (sl * Hl + sr * Hr) * iw;
-  const T ca = FM::sqr((gam - T(1)) * (Ha - T(0.5) * (ua * ua + va * va)));
+  const T ua = mulr(fma(sl, ul, mulr(sr, ur)), iw), va = mulr(fma(sl, vl, mulr(sr, vr)), iw);
+  const T Ha = mulr(fma(sl, mulr(El + pl, il), mulr(sr, mulr(Er + pr, ir))), iw);
+  const T ca = FM::sqr(mulr(gm1, fma(T(-0.5), fma(ua, ua, mulr(va, va)), Ha)));
   const T SL = fmin(ul - cl, ua - ca), SR = fmax(ur + cr, ua + ca);
-  const T ml = rl * (SL - ul), mr = rr * (SR - ur);
-  const T SS = FM::div(pr - pl + ul * ml - ur * mr, ml - mr);
-  T f[4];
-  if (SL >= T(0)) {
-    euler_x_flux(rl, ul, vl, wl[3], pl, f);
-  } else if (SS >= T(0)) {
-    euler_x_flux(rl, ul, vl, wl[3], pl, f);
-    const T k = FM::div(ml, SL - SS);  // rho* of the left star state
-    const T Es = k * (wl[3] * irl + (SS - ul) * (SS + FM::div(pl, ml)));
-    f[0] += SL * (k - rl);
-    f[1] += SL * (k * SS - rl * ul);
-    f[2] += SL * (k * vl - rl * vl);
-    f[3] += SL * (Es - wl[3]);
-  } else if (SR > T(0)) {
-    euler_x_flux(rr, ur, vr, wr[3], pr, f);
-    const T k = FM::div(mr, SR - SS);
-    const T Es = k * (wr[3] * irr + (SS - ur) * (SS + FM::div(pr, mr)));
-    f[0] += SR * (k - rr);
-    f[1] += SR * (k * SS - rr * ur);
-    f[2] += SR * (k * vr - rr * vr);
-    f[3] += SR * (Es - wr[3]);
-  } else {
-    euler_x_flux(rr, ur, vr, wr[3], pr, f);
-  }
-  out[0] = f[0];
-  out[1] = f[1] * nx - f[2] * ny;
-  out[2] = f[1] * ny + f[2] * nx;
-  out[3] = f[3];
+  const T ml = mulr(rl, SL - ul), mr = mulr(rr, SR - ur);
+  const T SS = FM::div(fma(-ur, mr, fma(ul, ml, pr - pl)), ml - mr);
+  const bool left = SL >= T(0) || SS >= T(0);
+  const T S = left ? SL : SR, m = left ? ml : mr, r = left ? rl : rr, E = left ? El : Er;
+  const T mn = left ? nl : nr, mt = left ? tl : tr, un = left ? ul : ur, ut = left ? vl : vr;
+  const T p = left ? pl : pr, ri = left ? il : ir;
+  const T id = FM::rcp(S - SS), k = mulr(m, id);  // k: rho* of this side's star state
+  const T Es = fma(k, fma(SS - un, SS, mulr(E, ri)), mulr(SS - un, mulr(p, id)));
+  const bool star = left ? !(SL >= T(0)) : SR > T(0);  // between the outer waves
+  const T b1 = fma(mn, un, p), b2 = mulr(mn, ut), b3 = mulr(E + p, un);
+  const T f0 = star ? fma(S, k - r, mn) : mn, f1 = star ? fma(S, fma(k, SS, -mn), b1) : b1;
+  const T f2 = star ? fma(S, fma(k, ut, -mt), b2) : b2, f3 = star ? fma(S, Es - E, b3) : b3;
+  out[0] = f0;
+  out[1] = fma(f1, nx, -mulr(f2, ny));
+  out[2] = fma(f1, ny, mulr(f2, nx));
+  out[3] = f3;
 }
-
 
 // Prescribed outer state of the inflow faces (gr = -3 - q for inflow face q): wa at
 // the Gauss points whose xi = n . x_G - c0 (FP64, [q][2]) lies below speed * t_stage,
@@ -838,67 +827,94 @@ __device__ __forceinline__ int64_t cell_of_gauss(int64_t g, int64_t nQ) {
   return g < 8 * nQ ? g / 8 : nQ + (g - 8 * nQ) / 6;
 }
 
-// flag[instance] is set when a Gauss-point state of a face of that instance is
-// non-physical; nQ and inst map the left Gauss-value index back to its cell's
-// instance (inst == nullptr: a single instance).  INFLOW: the mesh has inflow faces.
-template <typename T, int NV, bool INFLOW>
-__global__ void __launch_bounds__(256) k_face(
-    const T* __restrict__ Wg, const int32_t* __restrict__ gl, const int32_t* __restrict__ gr,
-    const T* __restrict__ fnx, const T* __restrict__ fny, const T* __restrict__ flen, int64_t nF,
-    T* __restrict__ F, Prm<T> prm, int* __restrict__ flag, const int32_t* __restrict__ inst, int64_t nQ,
-    Inflow<T> inf) {
-  for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < nF; f += (int64_t)gridDim.x * blockDim.x) {
-    bool bad = false;
-    const int64_t il = __ldg(gl + f);
-    const int64_t ir = __ldg(gr + f);
-    double t_stage = 0.0;
-    if constexpr (INFLOW) {
-      if (ir <= -3) {
-        const int i = inst ? __ldg(inst + cell_of_gauss(il, nQ)) : 0;
-        t_stage = inf.t[i] + inf.c * inf.dt[i];
-      }
-    }
-    const T nx = __ldg(fnx + f), ny = __ldg(fny + f), len = __ldg(flen + f);
-    T acc[NV];
+// Euler state outside a boundary face at its point k (code: -1 outflow, -2 wall, -3 - q inflow face q)
+// from the state w inside; i is the instance.
+template <typename T, bool INFLOW>
+__device__ __forceinline__ void outer_state(const T w[4], int64_t code, T nx, T ny, int k, const Inflow<T>& inf, int i,
+                                            T out[4]) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] = T(0);
+  for (int v = 0; v < 4; ++v) out[v] = w[v];
+  if (code == -2) {  // reflective wall: normal momentum reversed
+    const T mn = T(-2) * fma(w[1], nx, mulr(w[2], ny));
+    out[1] = fma(mn, nx, w[1]);
+    out[2] = fma(mn, ny, w[2]);
+  }
+  if constexpr (INFLOW) {
+    if (code <= -3) {
+      const bool a = __ldg(inf.xi + 2 * (-3 - code) + k) < inf.speed * (inf.t[i] + inf.c * inf.dt[i]);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) out[v] = a ? inf.wa[v] : inf.wb[v];
+    }
+  }
+}
+
+// Flags: flag[instance] is set when a Gauss-point state of a face of that instance is non-physical;
+// nQ and inst map a Gauss-value index back to its cell's instance (inst == nullptr: a single instance).
+
+// Scalar upwind flux, FP32C: one thread per face.
+__global__ void __launch_bounds__(256) k_face_scalar(
+    const float* __restrict__ Wg, const int32_t* __restrict__ gl, const int32_t* __restrict__ gr,
+    const float* __restrict__ fnx, const float* __restrict__ fny, const float* __restrict__ flen, int64_t nF,
+    float* __restrict__ F, Prm<float> prm, int* __restrict__ flag, const int32_t* __restrict__ inst, int64_t nQ) {
+  for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < nF; f += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t il = __ldg(gl + f), ir = __ldg(gr + f);
+    const float an = prm.ax * __ldg(fnx + f) + prm.ay * __ldg(fny + f), len = __ldg(flen + f);
+    float acc = 0.f;
+    bool bad = false;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      T wl[NV], wr[NV], fk[NV];
-      load_vec<T, NV>(Wg + (il + k) * NV, wl);
-      // the right cell meets the left cell's point k at its point 1 - k
-      if (ir >= 0) load_vec<T, NV>(Wg + (ir + 1 - k) * NV, wr);
-      else {
-#pragma unroll
-        for (int v = 0; v < NV; ++v) wr[v] = wl[v];
-        if (NV == 4 && ir == -2) {  // reflective wall: normal momentum reversed
-          const T mn = wl[1] * nx + wl[2] * ny;
-          wr[1] = wl[1] - T(2) * mn * nx;
-          wr[2] = wl[2] - T(2) * mn * ny;
-        }
-        if constexpr (INFLOW && NV == 4) {
-          if (ir <= -3) {
-            const bool a = __ldg(inf.xi + 2 * (-3 - ir) + k) < inf.speed * t_stage;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) wr[v] = a ? inf.wa[v] : inf.wb[v];
-          }
-        }
-      }
-      if (NV == 4) {
-        hllc<T>(wl, wr, nx, ny, prm.gas_gamma, fk, bad);
-      } else {
-        const T an = prm.ax * nx + prm.ay * ny;
-        fk[0] = an * (an >= T(0) ? wl[0] : wr[0]);
-        bad |= !(fk[0] == fk[0]);
-      }
-#pragma unroll
-      for (int v = 0; v < NV; ++v) acc[v] += fk[v];
+      const float wl = __ldg(Wg + il + k), wr = ir >= 0 ? __ldg(Wg + ir + 1 - k) : wl;
+      const float fk = an * (an >= 0.f ? wl : wr);
+      bad |= !(fk == fk);
+      acc += fk;
     }
-#pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] *= T(0.5) * len;
-    store_vec<T, NV>(F + f * NV, acc);
+    F[f] = acc * (0.5f * len);
     if (bad) flag[inst ? __ldg(inst + cell_of_gauss(il, nQ)) : 0] = 1;  // every writer stores the same value
   }
+}
+
+// Euler HLLC flux, FP32C: one thread per face.
+template <bool INFLOW>
+__global__ void __launch_bounds__(256) k_face_f32(
+    const float* __restrict__ Wg, const int32_t* __restrict__ gl, const int32_t* __restrict__ gr,
+    const float* __restrict__ fnx, const float* __restrict__ fny, const float* __restrict__ flen, int64_t nF,
+    float* __restrict__ F, Prm<float> prm, int* __restrict__ flag, const int32_t* __restrict__ inst, int64_t nQ,
+    Inflow<float> inf) {
+  for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < nF; f += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t il = __ldg(gl + f), ir = __ldg(gr + f);
+    const float nx = __ldg(fnx + f), ny = __ldg(fny + f), len = __ldg(flen + f);
+    const int i = INFLOW && ir <= -3 && inst ? __ldg(inst + cell_of_gauss(il, nQ)) : 0;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      float wl[4], wr[4], fk[4];
+      load_vec<float, 4>(Wg + (il + k) * 4, wl);
+      // the right cell meets the left cell's point k at its point 1 - k
+      if (ir >= 0) load_vec<float, 4>(Wg + (ir + 1 - k) * 4, wr);
+      else outer_state<float, INFLOW>(wl, ir, nx, ny, k, inf, i, wr);
+      hllc<float>(wl, wr, nx, ny, prm.gas_gamma, fk, bad);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) acc[v] += fk[v];
+    }
+#pragma unroll
+    for (int v = 0; v < 4; ++v) acc[v] *= 0.5f * len;
+    store_vec<float, 4>(F + f * 4, acc);
+    if (bad) flag[inst ? __ldg(inst + cell_of_gauss(il, nQ)) : 0] = 1;  // every writer stores the same value
+  }
+}
+
+// The time steps of the next step: dt[i] = src[i], or v for every instance (src == nullptr), and for the
+// FP32C stages split[i] = (hi, lo) with hi + lo ~ dt[i] to 2^-48 (split once here: every cell would spend
+// FP64 instructions on it).
+__global__ void k_set_dt(double* __restrict__ dt, float2* __restrict__ split, const double* __restrict__ src, double v,
+                         int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double d = src ? src[i] : v;
+  const float hi = (float)d;
+  dt[i] = d;
+  split[i] = make_float2(hi, (float)(d - (double)hi));
 }
 
 // t[i] += dt[i] for every instance (after the third stage of a step).
@@ -1171,20 +1187,24 @@ __global__ void __launch_bounds__(WENO_K1_TILE * 4, WENO_KCHAR_MIN_BLOCKS * 64 /
 // (compensated two-sum), and 1/|Omega|, dt, the RK coefficient and the state
 // update use double-float arithmetic, so that sum_i |Omega_i| dW_i telescopes
 // to ~1e-14 of the fluxes and the hi + lo state keeps its ~48-bit precision.
-template <typename T, int NV, int NFACE, bool COMP, int MODE>
+// Quads (cells below nQ, face lists qcf [k][nQ]) and triangles (tcf [k][nT]) in one launch.
+template <typename T, int NV, bool COMP, int MODE>
 __global__ void __launch_bounds__(256) k_gather(
-    const T* __restrict__ F, const int32_t* __restrict__ cf, const T* __restrict__ inv_area,
-    const T* __restrict__ inv_area_lo, int64_t N, int64_t first, T* __restrict__ U, T* __restrict__ Ulo,
-    T* __restrict__ Ws, T* __restrict__ Wslo, T* __restrict__ R, const double* __restrict__ dt,
-    const int32_t* __restrict__ inst) {
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < N; q += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = first + q;
+    const T* __restrict__ F, const int32_t* __restrict__ qcf, const int32_t* __restrict__ tcf,
+    const T* __restrict__ inv_area, const T* __restrict__ inv_area_lo, int64_t nQ, int64_t nT, T* __restrict__ U,
+    T* __restrict__ Ulo, T* __restrict__ Ws, T* __restrict__ Wslo, T* __restrict__ R, const double* __restrict__ dt,
+    const float2* __restrict__ dt_split, const int32_t* __restrict__ inst) {
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nQ + nT; c += (int64_t)gridDim.x * blockDim.x) {
+    const bool quad = c < nQ;
+    const int32_t* cf = quad ? qcf + c : tcf + (c - nQ);
+    const int64_t row = quad ? nQ : nT;
     T acc[NV], comp[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) { acc[v] = T(0); comp[v] = T(0); }
 #pragma unroll
-    for (int k = 0; k < NFACE; ++k) {
-      const int32_t e = __ldg(cf + (int64_t)k * N + q);
+    for (int k = 0; k < 4; ++k) {
+      if (k == 3 && !quad) break;
+      const int32_t e = __ldg(cf + k * row);
       const int64_t f = e >= 0 ? e : ~e;
       T fv[NV];
       load_vec<T, NV>(F + f * NV, fv);
@@ -1208,12 +1228,12 @@ __global__ void __launch_bounds__(256) k_gather(
       for (int v = 0; v < NV; ++v) res[v] = COMP ? (acc[v] + comp[v]) * ia : acc[v] * ia;
       store_vec<T, NV>(R + c * NV, res);
     } else {
-      const double dtd = dt[inst ? __ldg(inst + c) : 0];
+      const int i = inst ? __ldg(inst + c) : 0;
       T un[NV], ws[NV], out[NV];
       load_vec<T, NV>(U + c * NV, un);
       if (MODE > 1) load_vec<T, NV>(Ws + c * NV, ws);
       if (!COMP) {
-        const T h = (T)dtd;
+        const T h = (T)__ldg(dt + i);
         const T cs = MODE == 1 ? T(1) : (MODE == 2 ? T(0.25) : T(2.0 / 3.0));
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
@@ -1222,8 +1242,8 @@ __global__ void __launch_bounds__(256) k_gather(
         }
         store_vec<T, NV>(MODE == 3 ? U + c * NV : Ws + c * NV, out);
       } else {
-        const float dth = (float)dtd;
-        const df h{dth, (float)(dtd - (double)dth)};
+        const float2 dts = __ldg(dt_split + i);
+        const df h{dts.x, dts.y};
         const df iad{(float)ia, (float)__ldg(inv_area_lo + c)};
         const df cs = MODE == 1 ? df{1.0f, 0.0f} : (MODE == 2 ? df{0.25f, 0.0f} : df{0.6666667f, -1.9868216e-08f});
         T unl[NV], wsl[NV], outl[NV];
@@ -1244,6 +1264,120 @@ __global__ void __launch_bounds__(256) k_gather(
         }
         store_vec<T, NV>(MODE == 3 ? U + c * NV : Ws + c * NV, out);
         store_vec<T, NV>(MODE == 3 ? Ulo + c * NV : Wslo + c * NV, outl);
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------- K2 + K3, FP32C Euler
+// One face of a cell as its cell sees it: the neighbour's Gauss value that meets the face's first point
+// of the cell (its own local point index; -1 outflow, -2 wall, -3 - q inflow face q), the face's unit
+// normal (L to R) and its length, negative where the cell is the face's R cell.
+struct CellFace { int32_t other; float nx, ny, slen; };
+
+// Face fluxes, gather and RK3 stage of the FP32C Euler path in one pass: four lanes per cell, lane k
+// with face k computes that face's flux, then (after a 4 x 4 transposition by shuffles) lane v sums and
+// updates variable v.  A flux is thus computed by both of the face's cells, from the same operands in
+// the same order (the cell's place on the face decides which is left), so both get the same bits and
+// sum_i |Omega_i| dW_i telescopes as if it had been stored once; what is saved is a launch and the wait
+// between the two kernels.  The sum and the stage are those of k_gather (COMP), operation by operation.
+// MODE as k_gather.  Used while all its lanes are resident at once (use_fused): computing every flux twice
+// costs 90 us a pass on 1.0M cells where k_face_f32 and k_gather take 37 + 27, but an 800-triangle step
+// takes 25.3 us instead of 30.7 (10,000 triangles in characteristic variables 43.7 instead of 47.1;
+// 51,200 triangles 61.5 either way).
+template <int MODE, bool INFLOW>
+__global__ void __launch_bounds__(256) k_update_f32c(
+    const float* __restrict__ Wg, const CellFace* __restrict__ cf, const float* __restrict__ inv_area,
+    const float* __restrict__ inv_area_lo, int64_t nQ, int64_t N, float* __restrict__ U, float* __restrict__ Ulo,
+    float* __restrict__ Ws, float* __restrict__ Wslo, float* __restrict__ R, const float2* __restrict__ dt,
+    const int32_t* __restrict__ inst, float gas_gamma, int* __restrict__ flag, Inflow<float> inf) {
+  // uniform over a warp, whose lanes exchange fluxes; lanes past the end repeat the last cell
+  for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); t0 < 4 * N;
+       t0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t t = t0 + (threadIdx.x & 31);
+    const bool act = t < 4 * N;
+    const int64_t c = act ? t >> 2 : N - 1;
+    const int k = (int)(t & 3);
+    const bool quad = c < nQ;
+    const int i = inst ? __ldg(inst + c) : 0;
+    float x[4] = {0.f, 0.f, 0.f, 0.f};
+    if (quad || k < 3) {
+      const float4 e = __ldg(reinterpret_cast<const float4*>(cf) + (quad ? 4 * c + k : 4 * nQ + 3 * (c - nQ) + k));
+      const int32_t other = __float_as_int(e.x);
+      const float nx = e.y, ny = e.z, slen = e.w;
+      const float4* own = reinterpret_cast<const float4*>(Wg) + (quad ? 8 * c : 8 * nQ + 6 * (c - nQ)) + 2 * k;
+      float a[2][4], b[2][4];  // own and outer states at the cell's points 2k, 2k + 1
+#pragma unroll
+      for (int h = 0; h < 2; ++h) load_vec<float, 4>(reinterpret_cast<const float*>(own + h), a[h]);
+      if (other >= 0) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) load_vec<float, 4>(Wg + ((int64_t)other - h) * 4, b[h]);
+      } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) outer_state<float, INFLOW>(a[h], other, nx, ny, h, inf, i, b[h]);
+      }
+      const bool left = slen > 0.f;
+      bool bad = false;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {  // the face's points in the order of its L cell
+        float wl[4], wr[4], fk[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          wl[v] = left ? a[h][v] : b[1 - h][v];
+          wr[v] = left ? b[h][v] : a[1 - h][v];
+        }
+        hllc<float>(wl, wr, nx, ny, gas_gamma, fk, bad);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) x[v] += fk[v];
+      }
+      const float w = -0.5f * slen;  // outward flux leaves the L cell
+#pragma unroll
+      for (int v = 0; v < 4; ++v) x[v] *= w;
+      if (bad && act) flag[i] = 1;  // every writer stores the same value
+    }
+    // x[v] of lane k becomes x[k] of lane v: exchange across bit 0, then bit 1 of the lane
+#pragma unroll
+    for (int bit = 1; bit <= 2; bit *= 2) {
+      const bool up = (k & bit) != 0;
+#pragma unroll
+      for (int m = 0; m < 2; ++m) {
+        const int lo = bit == 1 ? 2 * m : m, hi = lo + bit;
+        const float give = up ? x[lo] : x[hi];
+        const float got = __shfl_xor_sync(0xffffffffu, give, bit);
+        if (up) x[lo] = got;
+        else x[hi] = got;
+      }
+    }
+    const int64_t at = 4 * c + k;  // this lane's variable from here on
+    float acc = 0.f, comp = 0.f;
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      float s, err;
+      two_sum(acc, x[f], s, err);
+      if (f < 3 || quad) {
+        acc = s;
+        comp = __fadd_rn(comp, err);
+      }
+    }
+    const float ia = __ldg(inv_area + c);
+    if constexpr (MODE == 0) {
+      if (act) R[at] = (acc + comp) * ia;
+    } else {
+      const float2 dts = __ldg(dt + i);
+      const df h{dts.x, dts.y};
+      const df iad{ia, __ldg(inv_area_lo + c)};
+      const df cs = MODE == 1 ? df{1.0f, 0.0f} : (MODE == 2 ? df{0.25f, 0.0f} : df{0.6666667f, -1.9868216e-08f});
+      const float un = U[at], unl = Ulo[at];
+      df d = df_mul(h, df_mul(df_norm(acc, comp), iad));
+      if (MODE > 1) {
+        float s, e;
+        two_sum(Ws[at], -un, s, e);
+        d = df_add(d, df_norm(s, __fadd_rn(e, __fsub_rn(Wslo[at], unl))));
+      }
+      const df o = df_add(df{un, unl}, df_mul(cs, d));
+      if (act) {
+        (MODE == 3 ? U : Ws)[at] = o.hi;
+        (MODE == 3 ? Ulo : Wslo)[at] = o.lo;
       }
     }
   }

@@ -502,22 +502,11 @@ __global__ void __launch_bounds__(256) k_face_f64(
     load_vec<double, NV>(Wg + (il + k) * NV, wl);
     if (ir >= 0) {
       load_vec<double, NV>(Wg + (ir + 1 - k) * NV, wr);
+    } else if constexpr (NV == 4) {
+      const int i = INFLOW && ir <= -3 && inst ? __ldg(inst + cell_of_gauss(il, nQ)) : 0;
+      outer_state<double, INFLOW>(wl, ir, nx, ny, k, inf, i, wr);
     } else {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) wr[v] = wl[v];
-      if (NV == 4 && ir == -2) {
-        const double mn = wl[1] * nx + wl[2] * ny;
-        wr[1] = wl[1] - 2.0 * mn * nx;
-        wr[2] = wl[2] - 2.0 * mn * ny;
-      }
-      if constexpr (INFLOW && NV == 4) {
-        if (ir <= -3) {
-          const int i = inst ? __ldg(inst + cell_of_gauss(il, nQ)) : 0;
-          const bool a = __ldg(inf.xi + 2 * (-3 - ir) + k) < inf.speed * (inf.t[i] + inf.c * inf.dt[i]);
-#pragma unroll
-          for (int v = 0; v < 4; ++v) wr[v] = a ? inf.wa[v] : inf.wb[v];
-        }
-      }
+      wr[0] = wl[0];
     }
     bool bad = false;
     if constexpr (NV == 4) {

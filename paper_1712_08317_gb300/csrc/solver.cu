@@ -110,6 +110,7 @@ struct weno_solver_s {
   void *area = nullptr, *inv_area = nullptr, *inv_area_lo = nullptr;
   double* area64 = nullptr;
   int32_t *gl = nullptr, *gr = nullptr;
+  weno::dev::CellFace* cell_faces = nullptr;  // FP32C Euler: faces of each cell (4 per quad, then 3 per triangle)
   void *fnx = nullptr, *fny = nullptr, *flen = nullptr;
   double *fnx64 = nullptr, *fny64 = nullptr, *flen64 = nullptr;
   int32_t* inst = nullptr;
@@ -118,6 +119,7 @@ struct weno_solver_s {
   double* partial = nullptr;
   // scratch
   void *Wg = nullptr, *F = nullptr, *Ws = nullptr, *Wslo = nullptr;
+  float2* dt_split = nullptr;  // dt_dev as (hi, lo), for the FP32C stages
   double *dt_dev = nullptr, *red = nullptr, *cell_dt = nullptr;
   double* t_dev = nullptr;   // time of each instance (advanced by every step)
   int64_t n_in = 0;          // inflow faces
@@ -127,7 +129,8 @@ struct weno_solver_s {
   int debug_stall = 0;  // weno_solver_debug_stall
   bool walls = false;   // the mesh has reflective wall faces (stencil values carry momentum flips)
   std::vector<void*> allocs;
-  Launch k1q, k1t, k2, k3q, k3t;
+  Launch k1q, k1t, k2, k3;
+  bool fused = false;  // FP32C Euler: fluxes and update in one kernel (use_fused)
   cudaStream_t cap = nullptr;
   struct Graph {
     const void* U;
@@ -333,11 +336,8 @@ void launch_reconstruct(S& s, const void* U, const void* Ulo, cudaStream_t st, i
   launch_reconstruct_into<T, NV, COMP>(s, U, Ulo, s.Wg, st, which, s.fix_marks);
 }
 
-// Face fluxes of the Gauss values wg into fl; c places the stage in the step (time t + c dt).
-template <typename T, int NV>
-void launch_face_into(S& s, const void* wg, void* fl, double c, cudaStream_t st) {
-  if (!s.nF) return;
-  weno::dev::Prm<T> p{(T)s.prm.gas_gamma, (T)s.prm.adv[0], (T)s.prm.adv[1]};
+template <typename T>
+weno::dev::Inflow<T> inflow_of(const S& s, double c) {
   weno::dev::Inflow<T> in{};
   for (int v = 0; v < 4; ++v) {
     in.wa[v] = (T)s.in_wa[v];
@@ -348,47 +348,89 @@ void launch_face_into(S& s, const void* wg, void* fl, double c, cudaStream_t st)
   in.dt = s.dt_dev;
   in.speed = s.prm.inflow_line[3];
   in.c = c;
-  // inflow faces exist for the Euler equations only
+  return in;
+}
+
+// Face fluxes of the Gauss values wg into fl; c places the stage in the step (time t + c dt).
+template <typename T, int NV>
+void launch_face(S& s, const void* wg, void* fl, double c, cudaStream_t st) {
+  if (!s.nF) return;
+  const weno::dev::Prm<T> p{(T)s.prm.gas_gamma, (T)s.prm.adv[0], (T)s.prm.adv[1]};
   if constexpr (std::is_same<T, double>::value) {
+    // inflow faces exist for the Euler equations only
     const auto kernel = NV == 4 && s.n_in ? weno::dev::k_face_f64<NV, NV == 4> : weno::dev::k_face_f64<NV, false>;
     kernel<<<grid_of(s.k2, 2 * s.nF), s.k2.block, 0, st>>>(
         (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
-        s.inst, s.nQ, in);
-  } else {
-    const auto kernel = NV == 4 && s.n_in ? weno::dev::k_face<T, NV, NV == 4> : weno::dev::k_face<T, NV, false>;
+        s.inst, s.nQ, inflow_of<T>(s, c));
+  } else if constexpr (NV == 4) {
+    const auto kernel = s.n_in ? weno::dev::k_face_f32<true> : weno::dev::k_face_f32<false>;
     kernel<<<grid_of(s.k2, s.nF), s.k2.block, 0, st>>>(
         (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
-        s.inst, s.nQ, in);
+        s.inst, s.nQ, inflow_of<T>(s, c));
+  } else {
+    weno::dev::k_face_scalar<<<grid_of(s.k2, s.nF), s.k2.block, 0, st>>>(
+        (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
+        s.inst, s.nQ);
   }
-}
-
-template <typename T, int NV, bool COMP>
-void launch_face(S& s, cudaStream_t st, double c = 0.0) {
-  launch_face_into<T, NV>(s, s.Wg, s.F, c, st);
 }
 
 template <typename T, int NV, bool COMP, int MODE>
-void launch_gather_mode(S& s, void* U, void* Ulo, void* R, cudaStream_t st, int which) {
-  if (s.nQ && (which & 1))
-    weno::dev::k_gather<T, NV, 4, COMP, MODE><<<grid_of(s.k3q, s.nQ), s.k3q.block, 0, st>>>(
-        (const T*)s.F, s.q_cf, (const T*)s.inv_area, (const T*)s.inv_area_lo, s.nQ, 0, (T*)U, (T*)Ulo, (T*)s.Ws,
-        (T*)s.Wslo, (T*)R,
-        s.dt_dev, s.inst);
-  if (s.nT && (which & 2))
-    weno::dev::k_gather<T, NV, 3, COMP, MODE><<<grid_of(s.k3t, s.nT), s.k3t.block, 0, st>>>(
-        (const T*)s.F, s.t_cf, (const T*)s.inv_area, (const T*)s.inv_area_lo, s.nT, s.nQ, (T*)U, (T*)Ulo, (T*)s.Ws,
-        (T*)s.Wslo, (T*)R,
-        s.dt_dev, s.inst);
+void launch_gather_mode(S& s, const void* fl, void* U, void* Ulo, void* R, cudaStream_t st) {
+  weno::dev::k_gather<T, NV, COMP, MODE><<<grid_of(s.k3, s.N), s.k3.block, 0, st>>>(
+      (const T*)fl, s.q_cf, s.t_cf, (const T*)s.inv_area, (const T*)s.inv_area_lo, s.nQ, s.nT, (T*)U, (T*)Ulo,
+      (T*)s.Ws, (T*)s.Wslo, (T*)R, s.dt_dev, s.dt_split, s.inst);
 }
 
 template <typename T, int NV, bool COMP>
-void launch_gather(S& s, int mode, void* U, void* Ulo, void* R, cudaStream_t st, int which = 3) {
+void launch_gather(S& s, int mode, const void* fl, void* U, void* Ulo, void* R, cudaStream_t st) {
   switch (mode) {
-    case 0: launch_gather_mode<T, NV, COMP, 0>(s, U, Ulo, R, st, which); break;
-    case 1: launch_gather_mode<T, NV, COMP, 1>(s, U, Ulo, R, st, which); break;
-    case 2: launch_gather_mode<T, NV, COMP, 2>(s, U, Ulo, R, st, which); break;
-    default: launch_gather_mode<T, NV, COMP, 3>(s, U, Ulo, R, st, which); break;
+    case 0: launch_gather_mode<T, NV, COMP, 0>(s, fl, U, Ulo, R, st); break;
+    case 1: launch_gather_mode<T, NV, COMP, 1>(s, fl, U, Ulo, R, st); break;
+    case 2: launch_gather_mode<T, NV, COMP, 2>(s, fl, U, Ulo, R, st); break;
+    default: launch_gather_mode<T, NV, COMP, 3>(s, fl, U, Ulo, R, st); break;
   }
+}
+
+// FP32C Euler: fluxes, gather and stage in one pass.
+constexpr int kUpdateBlock = 128;
+// While the pass's four lanes per cell fit the SMs at once (its 60 registers allow 1,024 threads an SM).
+bool use_fused(const S& s) { return !s.fp64 && s.nv == 4 && 4 * s.N <= (int64_t)1024 * s.nsm; }
+template <int MODE>
+void launch_update_mode(S& s, const void* wg, double c, void* U, void* Ulo, void* R, cudaStream_t st) {
+  const auto kernel = s.n_in ? weno::dev::k_update_f32c<MODE, true> : weno::dev::k_update_f32c<MODE, false>;
+  kernel<<<grid_of(Launch{kUpdateBlock}, 4 * s.N), kUpdateBlock, 0, st>>>(
+      (const float*)wg, s.cell_faces, (const float*)s.inv_area, (const float*)s.inv_area_lo, s.nQ, s.N, (float*)U,
+      (float*)Ulo, (float*)s.Ws, (float*)s.Wslo, (float*)R, s.dt_split, s.inst, (float)s.prm.gas_gamma, s.flag,
+      inflow_of<float>(s, c));
+}
+
+// What follows the reconstruction in a stage: fluxes of the Gauss values wg (through fl where they are
+// stored), gather and, for mode 1..3, the RK3 stage; mode 0 writes the residual to R.
+template <typename T, int NV, bool COMP>
+void launch_update(S& s, int mode, double c, const void* wg, void* fl, void* U, void* Ulo, void* R, cudaStream_t st) {
+  if constexpr (COMP && NV == 4) {
+    if (s.fused) {
+      switch (mode) {
+        case 0: launch_update_mode<0>(s, wg, c, U, Ulo, R, st); break;
+        case 1: launch_update_mode<1>(s, wg, c, U, Ulo, R, st); break;
+        case 2: launch_update_mode<2>(s, wg, c, U, Ulo, R, st); break;
+        default: launch_update_mode<3>(s, wg, c, U, Ulo, R, st); break;
+      }
+      return;
+    }
+  }
+  launch_face<T, NV>(s, wg, fl, c, st);
+  launch_gather<T, NV, COMP>(s, mode, fl, U, Ulo, R, st);
+}
+
+// The passes after the reconstruction on their own (weno_pass, weno_autotune).
+template <typename T, int NV, bool COMP>
+void launch_pass2(S& s, cudaStream_t st) {
+  launch_face<T, NV>(s, s.Wg, s.F, 0.0, st);
+}
+template <typename T, int NV, bool COMP>
+void launch_pass3(S& s, cudaStream_t st) {
+  launch_gather<T, NV, COMP>(s, 0, s.F, nullptr, nullptr, s.Ws, st);
 }
 
 template <typename T, int NV, bool COMP>
@@ -399,8 +441,7 @@ void launch_step_body(S& s, void* U, void* Ulo, cudaStream_t st) {
     const void* src = stage == 1 ? U : s.Ws;
     const void* srclo = stage == 1 ? Ulo : s.Wslo;
     launch_reconstruct<T, NV, COMP>(s, src, srclo, st);
-    launch_face<T, NV, COMP>(s, st, kStageTime[stage - 1]);
-    launch_gather<T, NV, COMP>(s, stage, U, Ulo, nullptr, st);
+    launch_update<T, NV, COMP>(s, stage, kStageTime[stage - 1], s.Wg, s.F, U, Ulo, nullptr, st);
   }
   weno::dev::k_advance_time<<<(s.n_inst + 127) / 128, 128, 0, st>>>(s.t_dev, s.dt_dev, s.n_inst);
 }
@@ -665,7 +706,7 @@ int setup_tma(S& s) {
   return WENO_OK;
 }
 
-int capture_step(S& s, void* U, void* Ulo);
+int run_step(S& s, void* U, void* Ulo, const double* dts, double dt, cudaStream_t st);
 
 }  // namespace
 
@@ -980,6 +1021,18 @@ int weno_solver_create(weno_mesh_t mesh, const weno_params* params, void* cuda_s
       cons(p.inflow_a, d.in_wa);
       cons(p.inflow_b, d.in_wb);
     }
+    std::vector<weno::dev::CellFace> faces;
+    d.fused = use_fused(d);
+    if (d.fused) {
+      faces.resize((size_t)4 * d.nQ + (size_t)3 * d.nT);
+      for (int64_t f = 0; f < d.nF; ++f) {
+        const float nx = (float)m.fnx[f], ny = (float)m.fny[f], len = (float)m.flen[f];
+        auto at = [&](int64_t c, int k) { return c < d.nQ ? 4 * c + k : 4 * d.nQ + 3 * (c - d.nQ) + k; };
+        faces[at(m.fL[f], m.fkL[f])] = {gr[f] >= 0 ? gr[f] + 1 : gr[f], nx, ny, len};
+        if (gr[f] >= 0) faces[at(m.fR[f], m.fkR[f])] = {gl[f] + 1, nx, ny, -len};
+      }
+      if ((r = upload(d, &d.cell_faces, faces, st))) return r;
+    }
     if ((r = upload(d, &d.gl, gl, st))) return r;
     if ((r = upload(d, &d.gr, gr, st))) return r;
     if ((r = upload_real(d, &d.fnx, m.fnx, st))) return r;
@@ -1025,6 +1078,7 @@ int weno_solver_create(weno_mesh_t mesh, const weno_params* params, void* cuda_s
   if ((r = d.alloc(&d.Ws, (size_t)d.N * d.nv * d.esz))) return r;
   if (!d.fp64 && (r = d.alloc(&d.Wslo, (size_t)d.N * d.nv * d.esz))) return r;
   if ((r = d.alloc(&d.dt_dev, sizeof(double) * d.n_inst))) return r;
+  if ((r = d.alloc(&d.dt_split, sizeof(float2) * d.n_inst))) return r;
   if ((r = d.alloc(&d.t_dev, sizeof(double) * d.n_inst))) return r;
   CK(cudaMemsetAsync(d.t_dev, 0, sizeof(double) * d.n_inst, st));
   CK(cudaMemsetAsync(d.dt_dev, 0, sizeof(double) * d.n_inst, st));
@@ -1059,8 +1113,7 @@ int weno_residual(weno_solver_t s, const void* U, const void* U_lo, void* R, voi
   DeviceGuard g(s->dev);
   cudaStream_t st = (cudaStream_t)cuda_stream;
   WENO_DISPATCH(*s, launch_reconstruct, *s, U, U_lo, st);
-  WENO_DISPATCH(*s, launch_face, *s, st);
-  WENO_DISPATCH(*s, launch_gather, *s, 0, const_cast<void*>(U), const_cast<void*>(U_lo), R, st);
+  WENO_DISPATCH(*s, launch_update, *s, 0, 0.0, s->Wg, s->F, const_cast<void*>(U), const_cast<void*>(U_lo), R, st);
   return check_launch();
 }
 
@@ -1070,27 +1123,15 @@ int weno_pass(weno_solver_t s, int32_t pass, const void* U, const void* U_lo, vo
   DeviceGuard g(s->dev);
   cudaStream_t st = (cudaStream_t)cuda_stream;
   if (pass == 1) WENO_DISPATCH(*s, launch_reconstruct, *s, U, U_lo, st);
-  else if (pass == 2) WENO_DISPATCH(*s, launch_face, *s, st);
-  else WENO_DISPATCH(*s, launch_gather, *s, 0, nullptr, nullptr, s->Ws, st);
+  else if (pass == 2) WENO_DISPATCH(*s, launch_pass2, *s, st);
+  else WENO_DISPATCH(*s, launch_pass3, *s, st);
   return check_launch();
 }
 
 int weno_step_instances(weno_solver_t s, void* U, void* U_lo, const double* dt_dev, void* cuda_stream) {
   if (!s || !U || !dt_dev || (!s->fp64 && !U_lo)) return fail(WENO_EINVAL, "null argument");
   DeviceGuard g(s->dev);
-  cudaStream_t st = (cudaStream_t)cuda_stream;
-  if (dt_dev != s->dt_dev)
-    CK(cudaMemcpyAsync(s->dt_dev, dt_dev, sizeof(double) * s->n_inst, cudaMemcpyDeviceToDevice, st));
-  cudaGraphExec_t exec = nullptr;
-  for (auto& x : s->graphs)
-    if (x.U == U && x.Ulo == U_lo) exec = x.exec;
-  if (!exec) {
-    int r = capture_step(*s, U, U_lo);
-    if (r) return r;
-    exec = s->graphs.back().exec;
-  }
-  CK(cudaGraphLaunch(exec, st));
-  return WENO_OK;
+  return run_step(*s, U, U_lo, dt_dev, 0.0, (cudaStream_t)cuda_stream);
 }
 
 int weno_set_time(weno_solver_t s, double t, void* cuda_stream) {
@@ -1115,10 +1156,7 @@ int weno_step(weno_solver_t s, void* U, void* U_lo, double dt, void* cuda_stream
   if (!(dt >= 0)) return fail(WENO_EINVAL, "dt must be >= 0");
   DeviceGuard g(s->dev);
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  weno::dev::k_fill<<<(s->n_inst + 127) / 128, 128, 0, st>>>(s->dt_dev, dt, s->n_inst);
-  int r = check_launch();
-  if (r) return r;
-  return weno_step_instances(s, U, U_lo, s->dt_dev, cuda_stream);
+  return run_step(*s, U, U_lo, nullptr, dt, st);
 }
 
 int weno_max_dt(weno_solver_t s, const void* U, const void* U_lo, double cfl, double* dt_out, void* cuda_stream) {
@@ -1186,7 +1224,7 @@ int weno_solver_launch_config(weno_solver_t s, int32_t* cfg) {
   if (!s || !cfg) return fail(WENO_EINVAL, "null argument");
   cfg[0] = s->k1q.block; cfg[1] = s->k1q.grid;
   cfg[2] = s->k2.block;  cfg[3] = s->k2.grid;
-  cfg[4] = s->k3q.block; cfg[5] = s->k3q.grid;
+  cfg[4] = s->k3.block; cfg[5] = s->k3.grid;
   return WENO_OK;
 }
 
@@ -1238,14 +1276,11 @@ int weno_autotune(weno_solver_t s, const void* U, const void* U_lo, void* cuda_s
     return WENO_OK;
   };
   S& d = *s;
-  void* u = const_cast<void*>(U);
-  void* ul = const_cast<void*>(U_lo);
   const std::vector<Launch>& k1c = d.tma ? tma : generic;
   if (d.nQ && !d.fp64) tune(d.k1q, [&] { WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st, 1); }, k1c);
   if (d.nT && !d.fp64) tune(d.k1t, [&] { WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st, 2); }, k1c);
-  tune(d.k2, [&] { WENO_DISPATCH(d, launch_face, d, st); }, generic);
-  if (d.nQ) tune(d.k3q, [&] { WENO_DISPATCH(d, launch_gather, d, 0, u, ul, d.Ws, st, 1); }, generic);
-  if (d.nT) tune(d.k3t, [&] { WENO_DISPATCH(d, launch_gather, d, 0, u, ul, d.Ws, st, 2); }, generic);
+  tune(d.k2, [&] { WENO_DISPATCH(d, launch_pass2, d, st); }, generic);
+  tune(d.k3, [&] { WENO_DISPATCH(d, launch_pass3, d, st); }, generic);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   CK(cudaStreamSynchronize(st));
@@ -1280,6 +1315,22 @@ int capture_step(S& s, void* U, void* Ulo) {
     s.graphs.erase(s.graphs.begin());
   }
   s.graphs.push_back({U, Ulo, exec});
+  return WENO_OK;
+}
+
+// One step with the time steps dts[instance] (device), or dt for every instance.
+int run_step(S& s, void* U, void* Ulo, const double* dts, double dt, cudaStream_t st) {
+  weno::dev::k_set_dt<<<(s.n_inst + 127) / 128, 128, 0, st>>>(s.dt_dev, s.dt_split, dts, dt, s.n_inst);
+  int r = check_launch();
+  if (r) return r;
+  cudaGraphExec_t exec = nullptr;
+  for (auto& x : s.graphs)
+    if (x.U == U && x.Ulo == Ulo) exec = x.exec;
+  if (!exec) {
+    if ((r = capture_step(s, U, Ulo))) return r;
+    exec = s.graphs.back().exec;
+  }
+  CK(cudaGraphLaunch(exec, st));
   return WENO_OK;
 }
 
@@ -1325,15 +1376,7 @@ template <typename T, int NV, bool COMP>
 void launch_residual_static(S& s, const void* U, const void* Ulo, void* R, void* wg, void* fl, uint8_t* redo,
                             cudaStream_t st) {
   launch_reconstruct_into<T, NV, COMP>(s, U, Ulo, wg, st, 3, redo);
-  launch_face_into<T, NV>(s, wg, fl, 0.0, st);
-  if (s.nQ)
-    weno::dev::k_gather<T, NV, 4, COMP, 0><<<grid_of(s.k3q, s.nQ), s.k3q.block, 0, st>>>(
-        (const T*)fl, s.q_cf, (const T*)s.inv_area, (const T*)s.inv_area_lo, s.nQ, 0, nullptr, nullptr, nullptr,
-        nullptr, (T*)R, s.dt_dev, s.inst);
-  if (s.nT)
-    weno::dev::k_gather<T, NV, 3, COMP, 0><<<grid_of(s.k3t, s.nT), s.k3t.block, 0, st>>>(
-        (const T*)fl, s.t_cf, (const T*)s.inv_area, (const T*)s.inv_area_lo, s.nT, s.nQ, nullptr, nullptr, nullptr,
-        nullptr, (T*)R, s.dt_dev, s.inst);
+  launch_update<T, NV, COMP>(s, 0, 0.0, wg, fl, nullptr, nullptr, R, st);
 }
 
 }  // namespace
