@@ -2,14 +2,13 @@
 //
 //   K1 (reconstruction, Sections 3.1-3.4): candidate gradients from gathered
 //                  stencil averages, smoothness indicators, split linear weights,
-//                  new indicator, nonlinear weights and the Gauss-point values;
-//                  one thread per (cell, variable):
-//     k_reconstruct_tma       FP32C Euler, tables staged in shared memory by TMA
-//     k_reconstruct_f32c      FP32C scalar advection
-//     k_reconstruct_char_tma  FP32C Euler, characteristic variables (four lanes
-//                             per cell exchange variables by shuffles)
+//                  new indicator, nonlinear weights and the Gauss-point values:
+//     k_reconstruct_tma       FP32C Euler, tables staged in shared memory by TMA, one
+//                             thread per (cell, variable); in characteristic variables
+//                             the four lanes of a cell exchange variables by shuffles
+//     k_reconstruct_f32c      FP32C scalar advection, one thread per cell
 //     k_reconstruct_f64, k_reconstruct_char_f64   FP64 (kernels_f64.cuh): a
-//                             thread per (cell, variable, face)
+//                             thread per (cell, variable, Gauss points)
 //   K2 (face fluxes, Eqs. 5-6): two Gauss points a face, rotated HLLC (Euler) or
 //                  upwind (scalar), |l|/2 (F1 + F2); at reflective walls the outer
 //                  state is the inner one mirrored, at inflow faces the prescribed
@@ -32,6 +31,8 @@
 #include <type_traits>
 #include <cuda.h>
 #include <cuda_runtime.h>
+
+#include "arith_f64.cuh"
 
 namespace weno {
 namespace dev {
@@ -145,11 +146,6 @@ __device__ __forceinline__ df df_mul(df a, df b) {
 // FP32C variant of K1 (same arithmetic in FP32 with approximate reciprocals).
 // Tables: gop4[j][q] = (o0 o1 o2 o3) of D_j^+, dg2[g][q] = x_G - c0,
 // gam4[g][k][q] = gamma_{4k..4k+3}, gam1[g][q] = gamma_8 (triangles).
-__device__ __forceinline__ float rcp_approx(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
 
 #ifndef WENO_K1_MIN_BLOCKS
 #define WENO_K1_MIN_BLOCKS 2  // resident 256-thread blocks' worth of threads per SM the register budget is sized for
@@ -433,58 +429,6 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
 #endif
 static_assert(WENO_K1_TILE == 8 || WENO_K1_TILE == 16 || WENO_K1_TILE == 32 || WENO_K1_TILE == 64, "tile of 8, 16, 32 or 64 cells");
 
-constexpr int kFixupChunk = 128;  // tiles a warp of a fix-up pass scans with one 4-byte load per lane
-
-// The tiles a fix-up pass redoes, in the order it walks them: chunks blockIdx.x, + gridDim.x, ...
-// of kFixupChunk one-byte marks written by the pass before it.  Every warp of the block reads the
-// same words, so all warps walk the same sequence; next() returns ntiles at the end.  The marks
-// are 4-byte aligned and readable up to the next multiple of 4 bytes past the last tile.
-struct MarkScan {
-  const uint8_t* redo;
-  int64_t ntiles, chunk;
-  uint32_t lanes = 0u, nib = 0u, mine = 0u;
-  int cur = 0;
-  __device__ MarkScan(const uint8_t* r, int64_t n) : redo(r), ntiles(n), chunk((int64_t)blockIdx.x - gridDim.x) {}
-  __device__ int64_t next() {
-    while (nib == 0u) {
-      while (lanes == 0u) {
-        chunk += gridDim.x;
-        if (chunk * kFixupChunk >= ntiles) return ntiles;
-        const int64_t t0 = chunk * kFixupChunk + 4 * (threadIdx.x & 31);
-        const uint32_t w = t0 < ntiles ? *reinterpret_cast<const uint32_t*>(redo + t0) : 0u;
-        mine = 0u;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (t0 + j < ntiles && ((w >> (8 * j)) & 0xffu)) mine |= 1u << j;
-        lanes = __ballot_sync(0xffffffffu, mine != 0u);
-      }
-      cur = __ffs(lanes) - 1;
-      lanes &= lanes - 1u;
-      nib = __shfl_sync(0xffffffffu, mine, cur);
-    }
-    const int j = __ffs(nib) - 1;
-    nib &= nib - 1u;
-    return chunk * kFixupChunk + 4 * cur + j;
-  }
-};
-
-// Marks of a pass whose lanes 4c..4c+3 of warp w hold cell 8w + c of a TILE-cell tile: redo[tile]
-// = 1 if a lane of the tile has `bad` set, else 0; a marked tile also writes one bit per cell to
-// cells[tile * TILE / 8 ...].  Called by every thread of the block.
-template <int TILE>
-__device__ __forceinline__ void write_marks(bool bad, int64_t tile, uint8_t* __restrict__ redo,
-                                            uint8_t* __restrict__ cells) {
-  const uint32_t v = __ballot_sync(0xffffffffu, bad);
-  const int need = __syncthreads_or(v != 0u);
-  if (need && (threadIdx.x & 31) == 0) {
-    uint32_t m8 = 0u;
-#pragma unroll
-    for (int c8 = 0; c8 < 8; ++c8) m8 |= ((v >> (4 * c8)) & 0xfu) ? 1u << c8 : 0u;
-    cells[tile * (TILE / 8) + (threadIdx.x >> 5)] = (uint8_t)m8;
-  }
-  if (threadIdx.x == 0) redo[tile] = (uint8_t)need;
-}
-
 // Tables of the Euler FP32C reconstruction, staged per tile: the G Gauss points of a cell are taken
 // as G/2 pairs (the two points of one face), whose values share a float2.  Rows of TILE float4:
 //   gam [k][j]  (gamma+_j, gamma+_j', gamma-_j, gamma-_j') at points 2k and 2k+1 (split, normalised)
@@ -500,7 +444,6 @@ struct PairTile {
   static constexpr int DG = G * TILE * 16;
   static constexpr int GOP = M * TILE * 16;
   static constexpr int STAGE = GAM + DG + GOP;  // bytes, multiple of 128
-  static constexpr int SMEM = STAGE + 16;       // one buffer + one mbarrier (padded)
 };
 
 // Indicators are clamped to kBetaMax before beta^2 and beta^3 are formed (below).  A candidate
@@ -610,46 +553,318 @@ __device__ __forceinline__ bool pair_points(const float4* __restrict__ sgam, con
   return ok;
 }
 
-// pair_points with the nonlinear weights in FP64 (IEEE division, indicators unclamped), whose
-// range holds every finite FP32 beta: the fix-up of cells whose FP32 sums of alpha left the
-// range.  Gauss points are the outer loop here, so only four sums are live.
+// The tables of one cell type as 2D tensor maps (rows of PairTile).
+struct TileMaps { CUtensorMap gam, dg, gop; };
+
+// What the tiles of one cell type work on; q counts the cells of the type, cell q is first + q and its
+// Gauss values start at point gbase + q G.
+struct TileCells {
+  const float *U, *Ulo, *area;
+  const int32_t* slot;  // [slot - 1][q]
+  int64_t N, first, gbase;
+  float* Wg;
+  float eps, gas_gamma;
+  int linear;
+};
+
+// Copies of a tile's tables into shared memory, completing on the barrier.
 template <int M, int G>
-__device__ __forceinline__ void pair_points_fp64(const float4* __restrict__ sgam, const float4* __restrict__ sdg,
-                                                 const float4* __restrict__ sgo, int cl, const float* dW, float a0,
-                                                 float eps, float w0, float l0, float* __restrict__ out) {
+__device__ __forceinline__ void load_tile(unsigned char* smem, const TileMaps* maps, int64_t tile, uint64_t* bar) {
+  using L = PairTile<M, G>;
+  const int x = (int)(tile * L::TILE * 4);
+  mbar_expect_tx(bar, L::STAGE);
+  tma_load_2d(smem, &maps->gam, x, 0, bar);
+  tma_load_2d(smem + L::GAM, &maps->dg, x, 0, bar);
+  tma_load_2d(smem + L::GAM + L::DG, &maps->gop, x, 0, bar);
+}
+
+// The cells whose sums of alpha left the FP32 range are redone with FP64 weights within the pass, each by
+// its whole warp: lane (variable v = lane % 4, Gauss point lane / 4), so that a cell costs about 300 FP64
+// instructions in a row and not 8 times as many in 4 lanes.  The warp comes here together; the tile's
+// tables are still in shared memory and the stencil is gathered again (fix_cell, fix_cell_char; not
+// inlined, so that the pass keeps its registers: 122 and 80 as without it).  A launch of its own for the
+// marked cells cost 3 to 4 us a pass where nothing was marked, which is most passes.  dU(s) is the lane's
+// difference of stencil slot s.
+template <int M, int G, typename Diff>
+__device__ __forceinline__ float fix_increment(const float4* __restrict__ sgam, const float4* __restrict__ sdg,
+                                               const float4* __restrict__ sgo, int cl, int g, Diff dU, float a0,
+                                               float eps) {
   constexpr int TILE = WENO_K1_TILE;
+  const int k = g >> 1;
+  const bool h = g & 1;
+  const float4 r = sdg[(2 * k) * TILE + cl], s = sdg[(2 * k + 1) * TILE + cl];
+  const double dx = h ? r.y : r.x, dy = h ? r.w : r.z;
+  const double2 sig = make_double2(h ? s.y : s.x, h ? s.w : s.z);
+  auto cand = [&](int j) {
+    const float4 m = sgo[j * TILE + cl];
+    const float da = dU(sub_a<M>(j)), db = dU(sub_b<M>(j));
+    const float gx = fmaf(m.x, da, m.y * db), gy = fmaf(m.z, da, m.w * db);
+    return candidate_f64((double)gx, (double)gy, (double)a0, (double)eps);
+  };
+  auto weights = [&](int, int j) {
+    const float4 w = sgam[(k * M + j) * TILE + cl];
+    return h ? make_double2(w.y, w.w) : make_double2(w.x, w.z);
+  };
+  double incr;
+  if (!face_points_f64<M, 1>(cand, weights, &dx, &dy, &sig, &incr))
+    face_points_ieee<M, 1>(cand, weights, &dx, &dy, &sig, (double)a0, (double)eps, &incr);
+  return (float)incr;
+}
+
+template <int M, int G, bool WALLS>
+__device__ __noinline__ void fix_cell(const unsigned char* smem, const TileCells& t, int64_t q, int cl) {
+  using L = PairTile<M, G>;
+  const int lane = threadIdx.x & 31, v = lane & 3, g = min(lane >> 2, G - 1);
+  const int64_t c = t.first + q;
+  const float w0 = t.U[c * 4 + v], l0 = t.Ulo[c * 4 + v];
+  const int32_t fm = flip_mask<WALLS, 4>(v);
+  float dW[M + 1];
 #pragma unroll 1
-  for (int g = 0; g < G; ++g) {
-    const int k = g >> 1, h = g & 1;
-    const float4 r = sdg[(2 * k) * TILE + cl], s = sdg[(2 * k + 1) * TILE + cl];
-    const float dxg = h ? r.y : r.x, dyg = h ? r.w : r.z;
-    double Ap = 0.0, Bp = 0.0, Am = 0.0, Bm = 0.0;
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-      const float4 m = sgo[j * TILE + cl];
-      const float da = dW[Sub<M>::a(j)], db = dW[Sub<M>::b(j)];
-      const float gx = fmaf(m.x, da, m.y * db), gy = fmaf(m.z, da, m.w * db);
-      const double b = (double)a0 * ((double)gx * gx + (double)gy * gy);
-      const double p = fmaf(gx, dxg, gy * dyg);
-      const float4 g4 = sgam[(k * M + j) * TILE + cl];
-      const double gp = h ? g4.y : g4.x, gn = h ? g4.w : g4.z;
-      const double qp = gp * b, qn = gn * b;
-      const double dp = b * (1.0 + qp + qp * qp) + eps, dn = b * (1.0 + qn + qn * qn) + eps;
-      const double ap = gp / (dp * dp), an = gn / (dn * dn);
-      Ap += ap;
-      Bp += ap * p;
-      Am += an;
-      Bm += an * p;
-    }
-    const double sp = h ? s.y : s.x, sm = h ? s.w : s.z;
-    out[g * 4] = w0 + (l0 + (float)(sp * (Bp / Ap) - sm * (Bm / Am)));
+  for (int s = 1; s <= M; ++s)
+    dW[s] = slot_delta<float, 4, WALLS, true>(t.U, t.Ulo, __ldg(t.slot + (int64_t)(s - 1) * t.N + q), v, fm, w0, l0);
+  const float4* sgam = reinterpret_cast<const float4*>(smem);
+  const float incr = fix_increment<M, G>(sgam, sgam + L::GAM / 16, sgam + (L::GAM + L::DG) / 16, cl, g,
+                                         [&](int s) { return dW[s]; }, __ldg(t.area + c), t.eps);
+  if (lane < 4 * G) t.Wg[(t.gbase + q * G + g) * 4 + v] = w0 + (l0 + incr);
+}
+
+// Calls fix(q, cell of the tile) for each cell of the warp with a lane that has `bad` set.  Warp 8 cells
+// wide: lanes 4i..4i+3 of warp w hold cell 8w + i of the tile.
+template <typename Fix>
+__device__ __forceinline__ void fix_marked(bool bad, int64_t q0, Fix fix) {
+  uint32_t m = __ballot_sync(0xffffffffu, bad);
+  while (m) {
+    const int i = (__ffs(m) - 1) >> 2;
+    m &= ~(0xfu << (4 * i));
+    const int cl = 8 * (threadIdx.x >> 5) + i;
+    fix(q0 + cl, cl);
   }
 }
 
-// FIXUP = false: the pass over every tile, FP32 weights (pair_points); each tile writes its marks
-// (write_marks) for the cells whose sums of alpha left the FP32 range.  FIXUP = true: run right
-// after on the marked tiles only (MarkScan), it redoes the marked cells with FP64 weights; the
-// decision per cell keeps every cell's result independent of which cells share its tile.
+// One tile, component-wise.  Returns false if the wait for its tables timed out.
+template <int M, int G, bool WALLS>
+__device__ __forceinline__ bool tile_points(const unsigned char* smem, uint64_t* bar, uint32_t phase, const TileCells& t,
+                                            int64_t tile) {
+  using L = PairTile<M, G>;
+  const int cl = threadIdx.x >> 2, v = threadIdx.x & 3;
+  const int64_t q = tile * L::TILE + cl;
+  const bool act = q < t.N;
+  const float4* sgam = reinterpret_cast<const float4*>(smem);
+  const float4* sdg = sgam + L::GAM / 16;
+  const float4* sgo = sdg + L::DG / 16;
+  // stencil gathers (independent of the staged tables) before the wait
+  float w0 = 0.f, l0 = 0.f, a0 = 0.f, dW[M + 1];
+  dW[0] = 0.f;
+  if (act) {
+    const int64_t c = t.first + q;
+    w0 = __ldg(t.U + c * 4 + v);
+    l0 = __ldg(t.Ulo + c * 4 + v);
+    const int32_t fm = flip_mask<WALLS, 4>(v);
+#pragma unroll
+    for (int s = 1; s <= M; ++s)
+      dW[s] = slot_delta<float, 4, WALLS, true>(t.U, t.Ulo, __ldg(t.slot + (int64_t)(s - 1) * t.N + q), v, fm, w0, l0);
+    a0 = __ldg(t.area + c);
+  }
+  const bool ok = mbar_wait_bounded(bar, phase);
+  if (__syncthreads_or(!ok)) return false;
+  bool bad = false;
+  if (act)
+    bad = !pair_points<M, G>(sgam, sdg, sgo, cl, dW, a0, t.eps, t.linear, w0, l0, t.Wg + (t.gbase + q * G) * 4 + v);
+  fix_marked(bad, tile * L::TILE, [&](int64_t qf, int cf) { fix_cell<M, G, WALLS>(smem, t, qf, cf); });
+  return true;
+}
+
+// Euler (Section 4): the Gauss points of local face k are reconstructed in the
+// characteristic variables of the normal flux Jacobian at the Roe average of
+// the cell and its neighbour across face k (stencil slot k+1; the cell itself
+// at an outflow boundary).  Four consecutive lanes hold one cell; lane l
+// gathers variable l of the stencil, projects the stencil differences onto
+// field l with row l of R^-1 (lane shuffles bring the other variables),
+// reconstructs field l, and returns variable l of W0 + R dU with row l of R.
+// Reconstructing the increment dU (zero for constant data) keeps constant
+// states exact whatever the rounding of R R^-1.
+template <typename T>
+__device__ __forceinline__ T lane_sum4(const T c[4], T x, int base) {
+  T r = T(0);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) r += c[i] * __shfl_sync(0xffffffffu, x, base + i);
+  return r;
+}
+
+// Roe frame of one face for lane l: row l of R^-1 (Lr) and row l of R (Rr), fields ordered
+// q_n - a, entropy, shear, q_n + a, from the two cells' averages and the outward unit normal.
+template <typename T>
+__device__ __forceinline__ void roe_rows(const T Wl[4], const T Wr[4], T nx, T ny, T gm1, int l, T Lr[4],
+                                         T Rr[4]) {
+  const T rl = Wl[0], ul = Wl[1] / rl, vl = Wl[2] / rl;
+  const T hl = (Wl[3] + gm1 * (Wl[3] - T(0.5) * rl * (ul * ul + vl * vl))) / rl;
+  const T rr = Wr[0], ur = Wr[1] / rr, vr = Wr[2] / rr;
+  const T hr = (Wr[3] + gm1 * (Wr[3] - T(0.5) * rr * (ur * ur + vr * vr))) / rr;
+  const T sl = sqrt(rl), sr = sqrt(rr), iw = T(1) / (sl + sr);
+  const T u = (sl * ul + sr * ur) * iw, v = (sl * vl + sr * vr) * iw, H = (sl * hl + sr * hr) * iw;
+  const T kin = T(0.5) * (u * u + v * v);
+  const T a = sqrt(gm1 * (H - kin)), ia = T(1) / a;
+  const T qn = u * nx + v * ny, qt = v * nx - u * ny;
+  const T b1 = gm1 * ia * ia, b2 = b1 * kin;
+  if (l == 0) {
+    Lr[0] = T(0.5) * (b2 + qn * ia); Lr[1] = T(-0.5) * (b1 * u + nx * ia);
+    Lr[2] = T(-0.5) * (b1 * v + ny * ia); Lr[3] = T(0.5) * b1;
+    Rr[0] = T(1); Rr[1] = T(1); Rr[2] = T(0); Rr[3] = T(1);
+  } else if (l == 1) {
+    Lr[0] = T(1) - b2; Lr[1] = b1 * u; Lr[2] = b1 * v; Lr[3] = -b1;
+    Rr[0] = u - a * nx; Rr[1] = u; Rr[2] = -ny; Rr[3] = u + a * nx;
+  } else if (l == 2) {
+    Lr[0] = -qt; Lr[1] = -ny; Lr[2] = nx; Lr[3] = T(0);
+    Rr[0] = v - a * ny; Rr[1] = v; Rr[2] = nx; Rr[3] = v + a * ny;
+  } else {
+    Lr[0] = T(0.5) * (b2 - qn * ia); Lr[1] = T(0.5) * (nx * ia - b1 * u);
+    Lr[2] = T(0.5) * (ny * ia - b1 * v); Lr[3] = T(0.5) * b1;
+    Rr[0] = H - a * qn; Rr[1] = kin; Rr[2] = qt; Rr[3] = H + a * qn;
+  }
+}
+
+#ifndef WENO_KCHAR_MIN_BLOCKS
+#define WENO_KCHAR_MIN_BLOCKS 2  // resident 256-thread blocks per SM the characteristic kernel's registers allow
+#endif
+
+// Increments R(x_G) - W0 of one field at the two Gauss points of face k from that field's stencil
+// differences dU (dU[0] = 0) and the tile's point-pair tables (PairTile rows), FP32: the arithmetic
+// of pair_points for a single face, candidates outer, both points in one paired instruction.
+// Returns false if a sum of alpha fell below kAlphaMin (the cell then goes to the FP64 fix-up).
+template <int M>
+__device__ __forceinline__ bool face_pair(const float4* __restrict__ sgam, const float4* __restrict__ sdg,
+                                          const float4* __restrict__ sgo, int cl, int k, const float* dU, float a0,
+                                          float eps, int linear, float2& incr) {
+  constexpr int TILE = WENO_K1_TILE;
+  const float4 r = sdg[(2 * k) * TILE + cl], s = sdg[(2 * k + 1) * TILE + cl];
+  const float2 dx = f2(r.x, r.y), dy = f2(r.z, r.w);
+  float2 Ap = f2(0.f, 0.f), Bp = f2(0.f, 0.f), Am = f2(0.f, 0.f), Bm = f2(0.f, 0.f);
+  if (linear) {
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+      const float4 m = sgo[j * TILE + cl];
+      const float da = dU[Sub<M>::a(j)], db = dU[Sub<M>::b(j)];
+      const float gx = fmaf(m.x, da, m.y * db), gy = fmaf(m.z, da, m.w * db);
+      const float4 g4 = sgam[(k * M + j) * TILE + cl];
+      const float2 p = __ffma2_rn(f2(gx, gx), dx, __fmul2_rn(f2(gy, gy), dy));
+      Bp = __ffma2_rn(f2(g4.x, g4.y), p, Bp);
+      Bm = __ffma2_rn(f2(g4.z, g4.w), p, Bm);
+    }
+    incr = f2(s.x * Bp.x - s.z * Bm.x, s.y * Bp.y - s.w * Bm.y);
+    return true;
+  }
+#pragma unroll
+  for (int j = 0; j < M; ++j) {
+    const float4 m = sgo[j * TILE + cl];
+    const float da = dU[Sub<M>::a(j)], db = dU[Sub<M>::b(j)];
+    const float gx = fmaf(m.x, da, m.y * db), gy = fmaf(m.z, da, m.w * db);
+    const float b0 = a0 * fmaf(gx, gx, gy * gy);
+    const float b = b0 > kBetaMax ? kBetaMax : b0;  // keeps a NaN
+    const float b2 = b * b, b3 = b2 * b, be = b + eps;
+    const float2 C0 = f2(be, be), C1 = f2(b2, b2), C2 = f2(b3, b3);
+    const float4 g4 = sgam[(k * M + j) * TILE + cl];
+    const float2 gp = f2(g4.x, g4.y), gn = f2(g4.z, g4.w);
+    const float2 p = __ffma2_rn(f2(gx, gx), dx, __fmul2_rn(f2(gy, gy), dy));
+    const float2 dp = __ffma2_rn(gp, __ffma2_rn(gp, C2, C1), C0);  // beta~+ + eps at both points
+    const float2 dn = __ffma2_rn(gn, __ffma2_rn(gn, C2, C1), C0);
+    const float2 ap = __fmul2_rn(gp, rcp2(__fmul2_rn(dp, dp)));
+    const float2 an = __fmul2_rn(gn, rcp2(__fmul2_rn(dn, dn)));
+    Ap = __fadd2_rn(Ap, ap);
+    Bp = __ffma2_rn(ap, p, Bp);
+    Am = __fadd2_rn(Am, an);
+    Bm = __ffma2_rn(an, p, Bm);
+  }
+  incr = f2(s.x * Bp.x * rcp_approx(Ap.x) - s.z * Bm.x * rcp_approx(Am.x),
+            s.y * Bp.y * rcp_approx(Ap.y) - s.w * Bm.y * rcp_approx(Am.y));
+  return !(Ap.x < kAlphaMin) && !(Ap.y < kAlphaMin) && !(Am.x < kAlphaMin) && !(Am.y < kAlphaMin);
+}
+
+// fix_cell in characteristic variables: the lane's field is lane % 4.
+template <int M, int G, bool WALLS>
+__device__ __noinline__ void fix_cell_char(const unsigned char* smem, const TileCells& t, int64_t q, int cl) {
+  using L = PairTile<M, G>;
+  const int lane = threadIdx.x & 31, base = lane & ~3, l = lane & 3, g = min(lane >> 2, G - 1), k = g >> 1;
+  const int64_t c = t.first + q;
+  const float4* sgam = reinterpret_cast<const float4*>(smem);
+  const float4* sdg = sgam + L::GAM / 16;
+  float W0[4], Wn[4], Lr[4], Rr[4];
+  load_vec<float, 4>(t.U + c * 4, W0);
+  const float w0 = t.U[c * 4 + l], l0 = t.Ulo[c * 4 + l];
+  slot_state4<float, WALLS>(t.U, __ldg(t.slot + (int64_t)k * t.N + q), Wn);
+  const float4 d0 = sdg[(2 * k) * L::TILE + cl];
+  const float tx = d0.y - d0.x, ty = d0.w - d0.z, it = rsqrtf(tx * tx + ty * ty);
+  roe_rows<float>(W0, Wn, ty * it, -tx * it, t.gas_gamma - 1.f, l, Lr, Rr);
+  const int32_t fm = flip_mask<WALLS, 4>(l);
+  float dU[M + 1];
+#pragma unroll 1
+  for (int s = 1; s <= M; ++s)
+    dU[s] = lane_sum4(Lr, slot_delta<float, 4, WALLS, true>(t.U, t.Ulo, __ldg(t.slot + (int64_t)(s - 1) * t.N + q), l,
+                                                            fm, w0, l0), base);
+  const float incr = fix_increment<M, G>(sgam, sdg, sdg + L::DG / 16, cl, g, [&](int s) { return dU[s]; },
+                                         __ldg(t.area + c), t.eps);
+  const float dWl = lane_sum4(Rr, incr, base);  // variable l of R dU
+  if (lane < 4 * G) t.Wg[(t.gbase + q * G + g) * 4 + l] = w0 + (l0 + dWl);
+}
+
+// One tile in characteristic variables.  Per face, each lane builds the Roe frame, projects the stencil
+// differences onto its field and evaluates the face's two Gauss points with face_pair; lanes of cells
+// past the end compute on the last cell's data and store nothing.
+template <int M, int G, bool WALLS>
+__device__ __forceinline__ bool tile_points_char(const unsigned char* smem, uint64_t* bar, uint32_t phase,
+                                                 const TileCells& t, int64_t tile) {
+  using L = PairTile<M, G>;
+  const int tid = threadIdx.x, base = (tid & 31) & ~3, l = tid & 3, cl = tid >> 2;
+  const int64_t qr = tile * L::TILE + cl;
+  const bool act = qr < t.N;
+  const int64_t q = act ? qr : t.N - 1;
+  const int64_t c = t.first + q;
+  const float4* sgam = reinterpret_cast<const float4*>(smem);
+  const float4* sdg = sgam + L::GAM / 16;
+  const float4* sgo = sdg + L::DG / 16;
+  // stencil gathers (independent of the staged tables) before the wait
+  float W0[4];
+  load_vec<float, 4>(t.U + c * 4, W0);
+  const float w0 = W0[l], l0 = __ldg(t.Ulo + c * 4 + l);
+  float dW[M + 1];
+  dW[0] = 0.f;
+  const int32_t fm = flip_mask<WALLS, 4>(l);
+#pragma unroll
+  for (int s = 1; s <= M; ++s)
+    dW[s] = slot_delta<float, 4, WALLS, true>(t.U, t.Ulo, __ldg(t.slot + (int64_t)(s - 1) * t.N + q), l, fm, w0, l0);
+  const float a0 = __ldg(t.area + c);
+  const bool ok = mbar_wait_bounded(bar, phase);
+  if (__syncthreads_or(!ok)) return false;
+  bool inrange = true;  // every sum of alpha of this lane's Gauss points within the FP32 range
+#pragma unroll 1
+  for (int k = 0; k < G / 2; ++k) {
+    // the frame of face k: the neighbour across it (slot k + 1) and the unit normal from the
+    // direction x_G' - x_G of its two Gauss points
+    float Wn[4];
+    slot_state4<float, WALLS>(t.U, __ldg(t.slot + (int64_t)k * t.N + q), Wn);
+    const float4 d0 = sdg[(2 * k) * L::TILE + cl];
+    const float tx = d0.y - d0.x, ty = d0.w - d0.z, it = rsqrtf(tx * tx + ty * ty);
+    float Lr[4], Rr[4];
+    roe_rows<float>(W0, Wn, ty * it, -tx * it, t.gas_gamma - 1.f, l, Lr, Rr);
+    float dU[M + 1];
+    dU[0] = 0.f;
+#pragma unroll
+    for (int s = 1; s <= M; ++s) dU[s] = lane_sum4(Lr, dW[s], base);
+    float2 incr;
+    inrange = face_pair<M>(sgam, sdg, sgo, cl, k, dU, a0, t.eps, t.linear, incr) && inrange;
+    const float d0l = lane_sum4(Rr, incr.x, base), d1l = lane_sum4(Rr, incr.y, base);  // variable l of R dU
+    if (act) {
+      t.Wg[(t.gbase + q * G + 2 * k) * 4 + l] = w0 + (l0 + d0l);
+      t.Wg[(t.gbase + q * G + 2 * k + 1) * 4 + l] = w0 + (l0 + d1l);
+    }
+  }
+  // a cell's four lanes mix all fields, so it is redone whole; lanes past the end read the zero fill of
+  // the tables and are left out
+  fix_marked(act && !inrange, tile * L::TILE, [&](int64_t qf, int cf) { fix_cell_char<M, G, WALLS>(smem, t, qf, cf); });
+  return true;
+}
+
+// FP32C Euler K1 over the tiles of both cell types (KINDS bit 0: quads, bit 1: triangles; a mesh of one
+// type has the instance sized for it), quads first.
 #ifndef WENO_K1_BLOCKS_Q
 #define WENO_K1_BLOCKS_Q (WENO_K1_MIN_BLOCKS * 64 / WENO_K1_TILE)  // resident blocks per SM, quads
 #endif
@@ -658,81 +873,58 @@ __device__ __forceinline__ void pair_points_fp64(const float4* __restrict__ sgam
 // the quads' 16 warps, whose 122 registers spill when cut to 96)
 #define WENO_K1_BLOCKS_T (WENO_K1_MIN_BLOCKS * 96 / WENO_K1_TILE)  // resident blocks per SM, triangles
 #endif
-// The register budget of k_reconstruct_tma<M, ...>: 65,536 / (blocks x TILE x 4) per thread.
-template <int M> struct K1Blocks { static constexpr int value = M == 12 ? WENO_K1_BLOCKS_Q : WENO_K1_BLOCKS_T; };
+// The register budget: 65,536 / (blocks x TILE x 4) per thread.
+template <int KINDS, bool CHAR> struct K1Blocks {
+  static constexpr int value = CHAR ? WENO_KCHAR_MIN_BLOCKS * 64 / WENO_K1_TILE : KINDS == 2 ? WENO_K1_BLOCKS_T : WENO_K1_BLOCKS_Q;
+};
+template <int KINDS> struct K1Smem {
+  static constexpr int quad = PairTile<12, 8>::STAGE, tri = PairTile<9, 6>::STAGE;
+  static constexpr int stage = (KINDS & 1) ? quad : tri, bytes = stage + 16;  // one buffer + one mbarrier (padded)
+};
 
-template <int M, int G, bool WALLS, bool FIXUP>
-__global__ void __launch_bounds__(WENO_K1_TILE * 4, K1Blocks<M>::value) k_reconstruct_tma(
-    const __grid_constant__ CUtensorMap map_gam, const __grid_constant__ CUtensorMap map_dg,
-    const __grid_constant__ CUtensorMap map_gop, const float* __restrict__ U, const float* __restrict__ Ulo,
-    const int32_t* __restrict__ slot, const float* __restrict__ area, int64_t N, int64_t first, int64_t gbase,
-    float* __restrict__ Wg, float eps, int linear, uint8_t* __restrict__ redo, uint8_t* __restrict__ cells,
-    int* __restrict__ err, int stall) {
-  using L = PairTile<M, G>;
-  static_assert(L::TILE % 8 == 0, "a byte of cell marks per 8 cells");
+template <int KINDS, bool CHAR, bool WALLS>
+__global__ void __launch_bounds__(WENO_K1_TILE * 4, K1Blocks<KINDS, CHAR>::value) k_reconstruct_tma(
+    const __grid_constant__ TileMaps mq, const __grid_constant__ TileMaps mt, const __grid_constant__ TileCells tq,
+    const __grid_constant__ TileCells tt, int* __restrict__ err, int stall) {
+  constexpr int TILE = WENO_K1_TILE;
   extern __shared__ __align__(128) unsigned char smem[];
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::STAGE);
-  const int tid = threadIdx.x, cl = tid >> 2, v = tid & 3;
-  const int64_t ntiles = (N + L::TILE - 1) / L::TILE;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + K1Smem<KINDS>::stage);
+  const int tid = threadIdx.x;
+  const int64_t nq = KINDS & 1 ? (tq.N + TILE - 1) / TILE : 0, ntiles = nq + (KINDS & 2 ? (tt.N + TILE - 1) / TILE : 0);
   if (tid == 0) {
-    mbar_init(&bar[0], stall ? 2 : 1);  // stall != 0 (testing aid): the wait runs out
+    mbar_init(bar, stall ? 2 : 1);  // stall != 0 (testing aid): the wait runs out
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
+  auto quads = [&](int64_t tile) { return KINDS == 1 || (KINDS == 3 && tile < nq); };
   auto issue = [&](int64_t tile) {
-    mbar_expect_tx(&bar[0], L::STAGE);
-    tma_load_2d(smem, &map_gam, (int)(tile * L::TILE * 4), 0, &bar[0]);
-    tma_load_2d(smem + L::GAM, &map_dg, (int)(tile * L::TILE * 4), 0, &bar[0]);
-    tma_load_2d(smem + L::GAM + L::DG, &map_gop, (int)(tile * L::TILE * 4), 0, &bar[0]);
+    if (quads(tile)) load_tile<12, 8>(smem, &mq, tile, bar);
+    else load_tile<9, 6>(smem, &mt, tile - nq, bar);
   };
-  MarkScan scan(redo, ntiles);
-  int64_t tile = FIXUP ? scan.next() : (int64_t)blockIdx.x;
-  if (!FIXUP && tid == 0 && tile < ntiles) issue(tile);
+  if (tid == 0 && blockIdx.x < ntiles) issue(blockIdx.x);
   uint32_t phase = 0u;
-  const float4* sgam = reinterpret_cast<const float4*>(smem);
-  const float4* sdg = reinterpret_cast<const float4*>(smem + L::GAM);
-  const float4* sgo = reinterpret_cast<const float4*>(smem + L::GAM + L::DG);
-  for (; tile < ntiles; tile = FIXUP ? scan.next() : tile + gridDim.x) {
-    if (FIXUP && tid == 0) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // after the previous tile's reads
-      issue(tile);
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    bool ok;
+    if (quads(tile)) {
+      if constexpr (CHAR) ok = tile_points_char<12, 8, WALLS>(smem, bar, phase, tq, tile);
+      else ok = tile_points<12, 8, WALLS>(smem, bar, phase, tq, tile);
+    } else {
+      if constexpr (CHAR) ok = tile_points_char<9, 6, WALLS>(smem, bar, phase, tt, tile - nq);
+      else ok = tile_points<9, 6, WALLS>(smem, bar, phase, tt, tile - nq);
     }
-    const int64_t next = tile + gridDim.x;
-    const int64_t q = tile * L::TILE + cl;
-    const bool act = q < N && (!FIXUP || ((cells[tile * (L::TILE / 8) + (cl >> 3)] >> (cl & 7)) & 1u));
-    // stencil gathers (independent of the staged tables) before the wait
-    float w0 = 0.f, l0 = 0.f, a0 = 0.f, dW[M + 1];
-    dW[0] = 0.f;
-    if (act) {
-      const int64_t c = first + q;
-      w0 = __ldg(U + c * 4 + v);
-      l0 = __ldg(Ulo + c * 4 + v);
-      const int32_t fm = flip_mask<WALLS, 4>(v);
-#pragma unroll
-      for (int s = 1; s <= M; ++s)
-        dW[s] = slot_delta<float, 4, WALLS, true>(U, Ulo, __ldg(slot + (int64_t)(s - 1) * N + q), v, fm, w0, l0);
-      a0 = __ldg(area + c);
-    }
-    const bool ok = mbar_wait_bounded(&bar[0], phase);
-    phase ^= 1u;
-    if (__syncthreads_or(!ok)) {
+    if (!ok) {  // the whole block: tile_points agrees on it
       if (tid == 0) *err = 1;
       return;
     }
-    bool bad = false;
-    if (act) {
-      float* out = Wg + (gbase + q * G) * 4 + v;
-      if constexpr (FIXUP)
-        pair_points_fp64<M, G>(sgam, sdg, sgo, cl, dW, a0, eps, w0, l0, out);
-      else
-        bad = !pair_points<M, G>(sgam, sdg, sgo, cl, dW, a0, eps, linear, w0, l0, out);
-    }
-    if constexpr (!FIXUP) write_marks<L::TILE>(bad, tile, redo, cells);
-    __syncthreads();  // the buffer is free for the next tile's copy
-    if (!FIXUP && tid == 0 && next < ntiles) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue(next);
+    phase ^= 1u;
+    const int64_t next = tile + gridDim.x;
+    if (next < ntiles) {
+      __syncthreads();  // the buffer is free for the next tile's copy
+      if (tid == 0) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        issue(next);
+      }
     }
   }
 }
@@ -921,261 +1113,6 @@ __global__ void k_set_dt(double* __restrict__ dt, float2* __restrict__ split, co
 __global__ void k_advance_time(double* __restrict__ t, const double* __restrict__ dt, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) t[i] += dt[i];
-}
-
-// ---------------------------------------------------------------- K1, characteristic variables
-// Euler (Section 4): the Gauss points of local face k are reconstructed in the
-// characteristic variables of the normal flux Jacobian at the Roe average of
-// the cell and its neighbour across face k (stencil slot k+1; the cell itself
-// at an outflow boundary).  Four consecutive lanes hold one cell; lane l
-// gathers variable l of the stencil, projects the stencil differences onto
-// field l with row l of R^-1 (lane shuffles bring the other variables),
-// reconstructs field l, and returns variable l of W0 + R dU with row l of R.
-// Reconstructing the increment dU (zero for constant data) keeps constant
-// states exact whatever the rounding of R R^-1.
-template <typename T>
-__device__ __forceinline__ T lane_sum4(const T c[4], T x, int base) {
-  T r = T(0);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) r += c[i] * __shfl_sync(0xffffffffu, x, base + i);
-  return r;
-}
-
-// Roe frame of one face for lane l: row l of R^-1 (Lr) and row l of R (Rr), fields ordered
-// q_n - a, entropy, shear, q_n + a, from the two cells' averages and the outward unit normal.
-template <typename T>
-__device__ __forceinline__ void roe_rows(const T Wl[4], const T Wr[4], T nx, T ny, T gm1, int l, T Lr[4],
-                                         T Rr[4]) {
-  const T rl = Wl[0], ul = Wl[1] / rl, vl = Wl[2] / rl;
-  const T hl = (Wl[3] + gm1 * (Wl[3] - T(0.5) * rl * (ul * ul + vl * vl))) / rl;
-  const T rr = Wr[0], ur = Wr[1] / rr, vr = Wr[2] / rr;
-  const T hr = (Wr[3] + gm1 * (Wr[3] - T(0.5) * rr * (ur * ur + vr * vr))) / rr;
-  const T sl = sqrt(rl), sr = sqrt(rr), iw = T(1) / (sl + sr);
-  const T u = (sl * ul + sr * ur) * iw, v = (sl * vl + sr * vr) * iw, H = (sl * hl + sr * hr) * iw;
-  const T kin = T(0.5) * (u * u + v * v);
-  const T a = sqrt(gm1 * (H - kin)), ia = T(1) / a;
-  const T qn = u * nx + v * ny, qt = v * nx - u * ny;
-  const T b1 = gm1 * ia * ia, b2 = b1 * kin;
-  if (l == 0) {
-    Lr[0] = T(0.5) * (b2 + qn * ia); Lr[1] = T(-0.5) * (b1 * u + nx * ia);
-    Lr[2] = T(-0.5) * (b1 * v + ny * ia); Lr[3] = T(0.5) * b1;
-    Rr[0] = T(1); Rr[1] = T(1); Rr[2] = T(0); Rr[3] = T(1);
-  } else if (l == 1) {
-    Lr[0] = T(1) - b2; Lr[1] = b1 * u; Lr[2] = b1 * v; Lr[3] = -b1;
-    Rr[0] = u - a * nx; Rr[1] = u; Rr[2] = -ny; Rr[3] = u + a * nx;
-  } else if (l == 2) {
-    Lr[0] = -qt; Lr[1] = -ny; Lr[2] = nx; Lr[3] = T(0);
-    Rr[0] = v - a * ny; Rr[1] = v; Rr[2] = nx; Rr[3] = v + a * ny;
-  } else {
-    Lr[0] = T(0.5) * (b2 - qn * ia); Lr[1] = T(0.5) * (nx * ia - b1 * u);
-    Lr[2] = T(0.5) * (ny * ia - b1 * v); Lr[3] = T(0.5) * b1;
-    Rr[0] = H - a * qn; Rr[1] = kin; Rr[2] = qt; Rr[3] = H + a * qn;
-  }
-}
-
-#ifndef WENO_KCHAR_MIN_BLOCKS
-#define WENO_KCHAR_MIN_BLOCKS 2  // resident 256-thread blocks per SM the characteristic kernel's registers allow
-#endif
-
-// Increments R(x_G) - W0 of one field at the two Gauss points of face k from that field's stencil
-// differences dU (dU[0] = 0) and the tile's point-pair tables (PairTile rows), FP32: the arithmetic
-// of pair_points for a single face, candidates outer, both points in one paired instruction.
-// Returns false if a sum of alpha fell below kAlphaMin (the cell then goes to the FP64 fix-up).
-template <int M>
-__device__ __forceinline__ bool face_pair(const float4* __restrict__ sgam, const float4* __restrict__ sdg,
-                                          const float4* __restrict__ sgo, int cl, int k, const float* dU, float a0,
-                                          float eps, int linear, float2& incr) {
-  constexpr int TILE = WENO_K1_TILE;
-  const float4 r = sdg[(2 * k) * TILE + cl], s = sdg[(2 * k + 1) * TILE + cl];
-  const float2 dx = f2(r.x, r.y), dy = f2(r.z, r.w);
-  float2 Ap = f2(0.f, 0.f), Bp = f2(0.f, 0.f), Am = f2(0.f, 0.f), Bm = f2(0.f, 0.f);
-  if (linear) {
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-      const float4 m = sgo[j * TILE + cl];
-      const float da = dU[Sub<M>::a(j)], db = dU[Sub<M>::b(j)];
-      const float gx = fmaf(m.x, da, m.y * db), gy = fmaf(m.z, da, m.w * db);
-      const float4 g4 = sgam[(k * M + j) * TILE + cl];
-      const float2 p = __ffma2_rn(f2(gx, gx), dx, __fmul2_rn(f2(gy, gy), dy));
-      Bp = __ffma2_rn(f2(g4.x, g4.y), p, Bp);
-      Bm = __ffma2_rn(f2(g4.z, g4.w), p, Bm);
-    }
-    incr = f2(s.x * Bp.x - s.z * Bm.x, s.y * Bp.y - s.w * Bm.y);
-    return true;
-  }
-#pragma unroll
-  for (int j = 0; j < M; ++j) {
-    const float4 m = sgo[j * TILE + cl];
-    const float da = dU[Sub<M>::a(j)], db = dU[Sub<M>::b(j)];
-    const float gx = fmaf(m.x, da, m.y * db), gy = fmaf(m.z, da, m.w * db);
-    const float b0 = a0 * fmaf(gx, gx, gy * gy);
-    const float b = b0 > kBetaMax ? kBetaMax : b0;  // keeps a NaN
-    const float b2 = b * b, b3 = b2 * b, be = b + eps;
-    const float2 C0 = f2(be, be), C1 = f2(b2, b2), C2 = f2(b3, b3);
-    const float4 g4 = sgam[(k * M + j) * TILE + cl];
-    const float2 gp = f2(g4.x, g4.y), gn = f2(g4.z, g4.w);
-    const float2 p = __ffma2_rn(f2(gx, gx), dx, __fmul2_rn(f2(gy, gy), dy));
-    const float2 dp = __ffma2_rn(gp, __ffma2_rn(gp, C2, C1), C0);  // beta~+ + eps at both points
-    const float2 dn = __ffma2_rn(gn, __ffma2_rn(gn, C2, C1), C0);
-    const float2 ap = __fmul2_rn(gp, rcp2(__fmul2_rn(dp, dp)));
-    const float2 an = __fmul2_rn(gn, rcp2(__fmul2_rn(dn, dn)));
-    Ap = __fadd2_rn(Ap, ap);
-    Bp = __ffma2_rn(ap, p, Bp);
-    Am = __fadd2_rn(Am, an);
-    Bm = __ffma2_rn(an, p, Bm);
-  }
-  incr = f2(s.x * Bp.x * rcp_approx(Ap.x) - s.z * Bm.x * rcp_approx(Am.x),
-            s.y * Bp.y * rcp_approx(Ap.y) - s.w * Bm.y * rcp_approx(Am.y));
-  return !(Ap.x < kAlphaMin) && !(Ap.y < kAlphaMin) && !(Am.x < kAlphaMin) && !(Am.y < kAlphaMin);
-}
-
-// face_pair with the nonlinear weights in FP64 (IEEE division, indicators unclamped): the fix-up
-// of cells whose FP32 sums of alpha left the range.
-template <int M>
-__device__ __forceinline__ void face_pair_fp64(const float4* __restrict__ sgam, const float4* __restrict__ sdg,
-                                               const float4* __restrict__ sgo, int cl, int k, const float* dU,
-                                               float a0, float eps, float2& incr) {
-  constexpr int TILE = WENO_K1_TILE;
-  const float4 r = sdg[(2 * k) * TILE + cl], s = sdg[(2 * k + 1) * TILE + cl];
-  float out[2];
-#pragma unroll 1
-  for (int h = 0; h < 2; ++h) {
-    const float dxg = h ? r.y : r.x, dyg = h ? r.w : r.z;
-    double Ap = 0.0, Bp = 0.0, Am = 0.0, Bm = 0.0;
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-      const float4 m = sgo[j * TILE + cl];
-      const float da = dU[Sub<M>::a(j)], db = dU[Sub<M>::b(j)];
-      const float gx = fmaf(m.x, da, m.y * db), gy = fmaf(m.z, da, m.w * db);
-      const double b = (double)a0 * ((double)gx * gx + (double)gy * gy);
-      const double pj = fmaf(gx, dxg, gy * dyg);
-      const float4 g4 = sgam[(k * M + j) * TILE + cl];
-      const double gp = h ? g4.y : g4.x, gn = h ? g4.w : g4.z;
-      const double qp = gp * b, qn = gn * b;
-      const double dp = b * (1.0 + qp + qp * qp) + eps, dn = b * (1.0 + qn + qn * qn) + eps;
-      const double ap = gp / (dp * dp), an = gn / (dn * dn);
-      Ap += ap;
-      Bp += ap * pj;
-      Am += an;
-      Bm += an * pj;
-    }
-    const double sp = h ? s.y : s.x, sm = h ? s.w : s.z;
-    out[h] = (float)(sp * (Bp / Ap) - sm * (Bm / Am));
-  }
-  incr = f2(out[0], out[1]);
-}
-
-// FP32C characteristic reconstruction with the tile's point-pair tables (split weights, Gauss
-// offsets and sigma+-, gradient operators; the PairTile layout of k_reconstruct_tma) staged in
-// shared memory by TMA.  Per face, each lane builds the Roe frame, projects the stencil
-// differences onto its field and evaluates the face's two Gauss points with face_pair; lanes of
-// cells past the end compute on the last cell's data and store nothing.
-//
-// FIXUP = false: the pass, with FP32 weights; every tile writes its marks (write_marks) for the
-// cells at which a Gauss point left the FP32 range of the weights.  FIXUP = true: run right after
-// on the marked tiles (MarkScan), it redoes those cells with the weights in FP64 (a separate
-// instance keeps that code out of the pass's register allocation); the decision per cell keeps
-// every cell's result independent of which cells share its tile.
-template <int M, int G, bool WALLS, bool FIXUP>
-__global__ void __launch_bounds__(WENO_K1_TILE * 4, WENO_KCHAR_MIN_BLOCKS * 64 / WENO_K1_TILE)
-    k_reconstruct_char_tma(const __grid_constant__ CUtensorMap map_gam, const __grid_constant__ CUtensorMap map_dg,
-                           const __grid_constant__ CUtensorMap map_gop, const float* __restrict__ U,
-                           const float* __restrict__ Ulo, const int32_t* __restrict__ slot,
-                           const float* __restrict__ area, int64_t N, int64_t first, int64_t gbase,
-                           float* __restrict__ Wg, float eps, float gas_gamma, int linear,
-                           uint8_t* __restrict__ redo, uint8_t* __restrict__ cells, int* __restrict__ err,
-                           int stall) {
-  using L = PairTile<M, G>;
-  static_assert(L::TILE % 8 == 0, "a byte of cell marks per 8 cells");
-  extern __shared__ __align__(128) unsigned char smem[];
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::STAGE);
-  const int tid = threadIdx.x, base = (tid & 31) & ~3, l = tid & 3, cl = tid >> 2;
-  const int64_t ntiles = (N + L::TILE - 1) / L::TILE;
-  if (tid == 0) {
-    mbar_init(&bar[0], stall ? 2 : 1);  // stall != 0 (testing aid): the wait runs out
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  __syncthreads();
-  auto issue = [&](int64_t tile) {
-    mbar_expect_tx(&bar[0], L::STAGE);
-    tma_load_2d(smem, &map_gam, (int)(tile * L::TILE * 4), 0, &bar[0]);
-    tma_load_2d(smem + L::GAM, &map_dg, (int)(tile * L::TILE * 4), 0, &bar[0]);
-    tma_load_2d(smem + L::GAM + L::DG, &map_gop, (int)(tile * L::TILE * 4), 0, &bar[0]);
-  };
-  MarkScan scan(redo, ntiles);
-  int64_t tile = FIXUP ? scan.next() : (int64_t)blockIdx.x;
-  if (!FIXUP && tid == 0 && tile < ntiles) issue(tile);
-  uint32_t phase = 0u;
-  const float4* sgam = reinterpret_cast<const float4*>(smem);
-  const float4* sdg = reinterpret_cast<const float4*>(smem + L::GAM);
-  const float4* sgo = reinterpret_cast<const float4*>(smem + L::GAM + L::DG);
-  for (; tile < ntiles; tile = FIXUP ? scan.next() : tile + gridDim.x) {
-    if (FIXUP && tid == 0) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // after the previous tile's reads
-      issue(tile);
-    }
-    const int64_t next = tile + gridDim.x;
-    const int64_t qr = tile * L::TILE + cl;
-    const bool act = qr < N && (!FIXUP || ((cells[tile * (L::TILE / 8) + (cl >> 3)] >> (cl & 7)) & 1u));
-    const int64_t q = act ? qr : N - 1;
-    const int64_t c = first + q;
-    // stencil gathers (independent of the staged tables) before the wait
-    float W0[4];
-    load_vec<float, 4>(U + c * 4, W0);
-    const float w0 = W0[l], l0 = __ldg(Ulo + c * 4 + l);
-    float dW[M + 1];
-    dW[0] = 0.f;
-    const int32_t fm = flip_mask<WALLS, 4>(l);
-#pragma unroll
-    for (int s = 1; s <= M; ++s)
-      dW[s] = slot_delta<float, 4, WALLS, true>(U, Ulo, __ldg(slot + (int64_t)(s - 1) * N + q), l, fm, w0, l0);
-    const float a0 = __ldg(area + c);
-    const bool ok = mbar_wait_bounded(&bar[0], phase);
-    phase ^= 1u;
-    if (__syncthreads_or(!ok)) {
-      if (tid == 0) *err = 1;
-      return;
-    }
-    bool inrange = true;  // every sum of alpha of this lane's Gauss points within the FP32 range
-#pragma unroll 1
-    for (int k = 0; k < G / 2; ++k) {
-      // the frame of face k: the neighbour across it (slot k + 1) and the unit normal from the
-      // direction x_G' - x_G of its two Gauss points
-      float Wn[4];
-      slot_state4<float, WALLS>(U, __ldg(slot + (int64_t)k * N + q), Wn);
-      const float4 d0 = sdg[(2 * k) * L::TILE + cl];
-      const float tx = d0.y - d0.x, ty = d0.w - d0.z, it = rsqrtf(tx * tx + ty * ty);
-      float Lr[4], Rr[4];
-      roe_rows<float>(W0, Wn, ty * it, -tx * it, gas_gamma - 1.f, l, Lr, Rr);
-      float dU[M + 1];
-      dU[0] = 0.f;
-#pragma unroll
-      for (int s = 1; s <= M; ++s) dU[s] = lane_sum4(Lr, dW[s], base);
-      float2 incr;
-      if constexpr (FIXUP) {
-        if (act)
-          face_pair_fp64<M>(sgam, sdg, sgo, cl, k, dU, a0, eps, incr);
-        else
-          incr = f2(0.f, 0.f);
-      } else {
-        inrange = face_pair<M>(sgam, sdg, sgo, cl, k, dU, a0, eps, linear, incr) && inrange;
-      }
-      const float d0l = lane_sum4(Rr, incr.x, base), d1l = lane_sum4(Rr, incr.y, base);  // variable l of R dU
-      if (act) {
-        Wg[(gbase + q * G + 2 * k) * 4 + l] = w0 + (l0 + d0l);
-        Wg[(gbase + q * G + 2 * k + 1) * 4 + l] = w0 + (l0 + d1l);
-      }
-    }
-    // weights outside the FP32 range at a cell of the tile (rare): the fix-up pass redoes the cell
-    // (any of its four lanes).  Lanes past the end read the zero fill of the tables and are left out.
-    if constexpr (!FIXUP) write_marks<L::TILE>(act && !inrange, tile, redo, cells);
-    __syncthreads();  // the buffer is free for the next tile's copy
-    if (!FIXUP && tid == 0 && next < ntiles) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue(next);
-    }
-  }
 }
 
 // ---------------------------------------------------------------- K3

@@ -67,8 +67,7 @@ unsigned grid_of(const Launch& l, int64_t work) {
 
 // TMA reconstruction: TILE x 4 threads per block, one TILE-cell tile per iteration.
 constexpr int kTile = weno::dev::PairTile<12, 8>::TILE;
-unsigned tma_grid(const Launch& l, int64_t cells) {
-  const int64_t tiles = (cells + kTile - 1) / kTile;
+unsigned tma_grid(const Launch& l, int64_t tiles) {
   const int64_t g = l.grid > 0 ? std::min<int64_t>(l.grid, tiles) : tiles;
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(g, 0x7fffffff));
 }
@@ -102,10 +101,8 @@ struct weno_solver_s {
   double2 *q_wt = nullptr, *q_sig = nullptr, *t_wt = nullptr, *t_sig = nullptr;   // FP64 split weights
   int64_t q_pitch = 0, t_pitch = 0;  // row pitch (cells) of the packed FP32C tables and the FP64 split weights
   bool tma = false;                   // Euler FP32C: reconstruction with TMA-staged tables
-  CUtensorMap q_map_gop{}, t_map_gop{};  // gradient operators
-  CUtensorMap q_map_pgam{}, q_map_pdg{}, t_map_pgam{}, t_map_pdg{};  // point-pair tables (both FP32C Euler kernels)
+  weno::dev::TileMaps q_maps{}, t_maps{};  // point-pair tables and gradient operators (FP32C Euler)
   int* err = nullptr;                 // set by a kernel whose bounded wait timed out
-  uint8_t* fix_marks = nullptr;       // FP32C Euler: tiles and cells whose weights left the FP32 range
   int32_t *q_slot = nullptr, *t_slot = nullptr, *q_cf = nullptr, *t_cf = nullptr;
   void *area = nullptr, *inv_area = nullptr, *inv_area_lo = nullptr;
   double* area64 = nullptr;
@@ -169,29 +166,6 @@ static_assert(weno::dev::kDevFlipX == weno::kFlipX && weno::dev::kDevFlipY == we
               "stencil table bit layout shared by the host tables and the kernels");
 
 // ------------------------------------------------------------ launches
-// Fix-up marks of the FP32C Euler reconstructions (component-wise and characteristic), per cell
-// group (quads, then triangles): one byte per tile, then one bit per cell of the tile, each part
-// padded to 16 bytes; zero bytes for every other path.
-int64_t redo_part(int64_t n) {
-  constexpr int64_t t = weno::dev::PairTile<12, 8>::TILE;
-  const int64_t tiles = (n + t - 1) / t;
-  return (tiles + 15) / 16 * 16 + (tiles * (t / 8) + 15) / 16 * 16;
-}
-int64_t redo_tiles_part(int64_t n) {
-  constexpr int64_t t = weno::dev::PairTile<12, 8>::TILE;
-  return ((n + t - 1) / t + 15) / 16 * 16;
-}
-int64_t redo_bytes(const S& s) {
-  if (s.fp64 || s.nv != 4) return 0;
-  return redo_part(s.nQ) + redo_part(s.nT);
-}
-// Grid of a fix-up pass over n cells: a block per kFixupChunk tiles of marks, at most 4 per SM.
-unsigned fix_grid(const S& s, int64_t n) {
-  constexpr int64_t t = weno::dev::PairTile<12, 8>::TILE;
-  const int64_t chunks = ((n + t - 1) / t + weno::dev::kFixupChunk - 1) / weno::dev::kFixupChunk;
-  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(chunks, 4 * s.nsm));
-}
-
 // Grid of an FP64 reconstruction over n cells of G Gauss points and M candidates: blocks of `width` (cell,
 // variable) columns with a thread for every pts points of a column, and the kernel's shared memory.  The
 // FP64 pipe, split between the quarters of the SMs, is the bound and has to be shared out evenly: tiles
@@ -213,41 +187,49 @@ F64Grid f64_grid(const S& s, int64_t n, int nv, int M, int G, bool characteristi
   return {width, pts, (unsigned)((n + tile - 1) / tile), (unsigned)threads, doubles * sizeof(double)};
 }
 
+// Mixed meshes: one launch for both cell types, quads first, up to 16 rounds of resident tiles.  It saves a
+// launch and the wait for the quads' last tiles, about 5 us; against that its triangles run at the quads'
+// register count, 16 instead of 24 warps an SM and 5 % slower.  A step of 133k cells takes 138.8 us in one
+// launch and 151.1 in two, of 241k cells (63 % triangles) 211 and 219, of 1.0M cells 815 and 796.
+bool merge_kinds(const S& s) { return s.nQ + s.nT <= (int64_t)16 * 8 * kTile * s.nsm; }
+
+// FP32C Euler reconstruction into wg.  which as below.
+template <int KINDS, bool CHAR, bool WALLS>
+void launch_tma_kinds(S& s, const Launch& l, const float* u, const float* ul, float* wg, cudaStream_t st) {
+  const weno::dev::TileCells q{u, ul, (const float*)s.area, s.q_slot, s.nQ, 0, 0, wg, (float)s.prm.eps,
+                               (float)s.prm.gas_gamma, s.prm.linear};
+  weno::dev::TileCells t = q;
+  t.slot = s.t_slot;
+  t.N = s.nT;
+  t.first = s.nQ;
+  t.gbase = 8 * s.nQ;
+  const int64_t tiles = (KINDS & 1 ? (s.nQ + kTile - 1) / kTile : 0) + (KINDS & 2 ? (s.nT + kTile - 1) / kTile : 0);
+  weno::dev::k_reconstruct_tma<KINDS, CHAR, WALLS>
+      <<<tma_grid(l, tiles), kTile * 4, weno::dev::K1Smem<KINDS>::bytes, st>>>(s.q_maps, s.t_maps, q, t, s.err, s.debug_stall);
+}
+template <bool CHAR, bool WALLS>
+void launch_tma(S& s, const void* U, const void* Ulo, void* wg, cudaStream_t st, int which) {
+  const float *u = static_cast<const float*>(U), *ul = static_cast<const float*>(Ulo);
+  float* w = static_cast<float*>(wg);
+  which &= (s.nQ ? 1 : 0) | (s.nT ? 2 : 0);
+  if (which == 3 && merge_kinds(s)) return launch_tma_kinds<3, CHAR, WALLS>(s, s.k1q, u, ul, w, st);
+  if (which & 1) launch_tma_kinds<1, CHAR, WALLS>(s, s.k1q, u, ul, w, st);
+  if (which & 2) launch_tma_kinds<2, CHAR, WALLS>(s, s.k1t, u, ul, w, st);
+}
+
 // Cell reconstruction into the Gauss-value array wg.  which: bit 0 = quad group,
 // bit 1 = triangle group.
 template <typename T, int NV, bool COMP, bool WALLS>
-void launch_reconstruct_impl(S& s, const void* U, const void* Ulo, void* wg, cudaStream_t st, int which,
-                             uint8_t* redo) {
-  const T* u = static_cast<const T*>(U);
-  const T* ul = static_cast<const T*>(Ulo);
-  const T eps = (T)s.prm.eps;
-  if constexpr (NV == 4) {
-    if (s.prm.characteristic) {
-      const T gg = (T)s.prm.gas_gamma;
-      if constexpr (COMP) {  // packed FP32C tables staged by TMA (setup_tma runs for every FP32C Euler solver)
-        using CQ = weno::dev::PairTile<12, 8>;
-        using CT = weno::dev::PairTile<9, 6>;
-        // each pass is followed by its fix-up pass over the tiles it marked (a few us when none is)
-        uint8_t* cells_q = redo + redo_tiles_part(s.nQ);
-        uint8_t* redo_t = redo + redo_part(s.nQ);
-        uint8_t* cells_t = redo_t + redo_tiles_part(s.nT);
-        if (s.nQ && (which & 1)) {
-          weno::dev::k_reconstruct_char_tma<12, 8, WALLS, false><<<tma_grid(s.k1q, s.nQ), CQ::THREADS, CQ::SMEM, st>>>(
-              s.q_map_pgam, s.q_map_pdg, s.q_map_gop, u, ul, s.q_slot, (const float*)s.area, s.nQ, 0, 0,
-              (float*)wg, eps, gg, s.prm.linear, redo, cells_q, s.err, s.debug_stall);
-          weno::dev::k_reconstruct_char_tma<12, 8, WALLS, true><<<fix_grid(s, s.nQ), CQ::THREADS, CQ::SMEM, st>>>(
-              s.q_map_pgam, s.q_map_pdg, s.q_map_gop, u, ul, s.q_slot, (const float*)s.area, s.nQ, 0, 0,
-              (float*)wg, eps, gg, s.prm.linear, redo, cells_q, s.err, s.debug_stall);
-        }
-        if (s.nT && (which & 2)) {
-          weno::dev::k_reconstruct_char_tma<9, 6, WALLS, false><<<tma_grid(s.k1t, s.nT), CT::THREADS, CT::SMEM, st>>>(
-              s.t_map_pgam, s.t_map_pdg, s.t_map_gop, u, ul, s.t_slot, (const float*)s.area, s.nT, s.nQ,
-              8 * s.nQ, (float*)wg, eps, gg, s.prm.linear, redo_t, cells_t, s.err, s.debug_stall);
-          weno::dev::k_reconstruct_char_tma<9, 6, WALLS, true><<<fix_grid(s, s.nT), CT::THREADS, CT::SMEM, st>>>(
-              s.t_map_pgam, s.t_map_pdg, s.t_map_gop, u, ul, s.t_slot, (const float*)s.area, s.nT, s.nQ,
-              8 * s.nQ, (float*)wg, eps, gg, s.prm.linear, redo_t, cells_t, s.err, s.debug_stall);
-        }
-      } else {
+void launch_reconstruct_impl(S& s, const void* U, const void* Ulo, void* wg, cudaStream_t st, int which) {
+  if constexpr (COMP && NV == 4) {
+    if (s.prm.characteristic) return launch_tma<true, WALLS>(s, U, Ulo, wg, st, which);
+    return launch_tma<false, WALLS>(s, U, Ulo, wg, st, which);
+  } else {
+    const T* u = static_cast<const T*>(U);
+    const T eps = (T)s.prm.eps;
+    if constexpr (!COMP && NV == 4) {
+      if (s.prm.characteristic) {
+        const T gg = (T)s.prm.gas_gamma;
         if (s.nQ && (which & 1)) {
           const F64Grid g = f64_grid(s, s.nQ, 4, 12, 8, true);
           const auto kernel = g.pts == 1 ? weno::dev::k_reconstruct_char_f64<12, 8, 1, WALLS>
@@ -264,58 +246,32 @@ void launch_reconstruct_impl(S& s, const void* U, const void* Ulo, void* wg, cud
               u, s.t_slot, (const double*)s.t_gop, (const double*)s.t_dg, (const double*)s.t_gam, s.t_wt, s.t_sig,
               (const double*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (double*)wg, eps, gg, s.prm.linear, g.width);
         }
+        return;
       }
-      return;
     }
-  }
-  if constexpr (COMP && NV == 4) {
-    if (s.tma) {  // each pass is followed by its fix-up pass over the cells it marked
-      using PQ = weno::dev::PairTile<12, 8>;
-      using PT = weno::dev::PairTile<9, 6>;
-      uint8_t* cells_q = redo + redo_tiles_part(s.nQ);
-      uint8_t* redo_t = redo + redo_part(s.nQ);
-      uint8_t* cells_t = redo_t + redo_tiles_part(s.nT);
+    if constexpr (COMP) {
+      if (s.nQ && (which & 1))
+        weno::dev::k_reconstruct_f32c<NV, 12, 8><<<grid_of(s.k1q, s.nQ * NV), s.k1q.block, 0, st>>>(
+            u, static_cast<const T*>(Ulo), s.q_slot, (const float4*)s.q_gop, (const float4*)s.q_dg, (const float4*)s.q_gam,
+            (const float2*)s.q_gam1, (const float*)s.area, s.nQ, s.q_pitch, 0, 0, (float*)wg, eps, s.prm.linear);
+      if (s.nT && (which & 2))
+        weno::dev::k_reconstruct_f32c<NV, 9, 6><<<grid_of(s.k1t, s.nT * NV), s.k1t.block, 0, st>>>(
+            u, static_cast<const T*>(Ulo), s.t_slot, (const float4*)s.t_gop, (const float4*)s.t_dg, (const float4*)s.t_gam,
+            (const float2*)s.t_gam1, (const float*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (float*)wg, eps,
+            s.prm.linear);
+    } else {
       if (s.nQ && (which & 1)) {
-        weno::dev::k_reconstruct_tma<12, 8, WALLS, false><<<tma_grid(s.k1q, s.nQ), PQ::THREADS, PQ::SMEM, st>>>(
-            s.q_map_pgam, s.q_map_pdg, s.q_map_gop, u, ul, s.q_slot, (const float*)s.area, s.nQ, 0, 0, (float*)wg,
-            eps, s.prm.linear, redo, cells_q, s.err, s.debug_stall);
-        weno::dev::k_reconstruct_tma<12, 8, WALLS, true><<<fix_grid(s, s.nQ), PQ::THREADS, PQ::SMEM, st>>>(
-            s.q_map_pgam, s.q_map_pdg, s.q_map_gop, u, ul, s.q_slot, (const float*)s.area, s.nQ, 0, 0, (float*)wg,
-            eps, s.prm.linear, redo, cells_q, s.err, s.debug_stall);
+        const F64Grid g = f64_grid(s, s.nQ, NV, 12, 8, false);
+        weno::dev::k_reconstruct_f64<NV, 12, 8, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
+            u, s.q_slot, (const double*)s.q_gop, (const double*)s.q_dg, (const double*)s.q_gam, s.q_wt, s.q_sig,
+            (const double*)s.area, s.nQ, s.q_pitch, 0, 0, (double*)wg, eps, s.prm.linear, g.width);
       }
       if (s.nT && (which & 2)) {
-        weno::dev::k_reconstruct_tma<9, 6, WALLS, false><<<tma_grid(s.k1t, s.nT), PT::THREADS, PT::SMEM, st>>>(
-            s.t_map_pgam, s.t_map_pdg, s.t_map_gop, u, ul, s.t_slot, (const float*)s.area, s.nT, s.nQ, 8 * s.nQ,
-            (float*)wg, eps, s.prm.linear, redo_t, cells_t, s.err, s.debug_stall);
-        weno::dev::k_reconstruct_tma<9, 6, WALLS, true><<<fix_grid(s, s.nT), PT::THREADS, PT::SMEM, st>>>(
-            s.t_map_pgam, s.t_map_pdg, s.t_map_gop, u, ul, s.t_slot, (const float*)s.area, s.nT, s.nQ, 8 * s.nQ,
-            (float*)wg, eps, s.prm.linear, redo_t, cells_t, s.err, s.debug_stall);
+        const F64Grid g = f64_grid(s, s.nT, NV, 9, 6, false);
+        weno::dev::k_reconstruct_f64<NV, 9, 6, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
+            u, s.t_slot, (const double*)s.t_gop, (const double*)s.t_dg, (const double*)s.t_gam, s.t_wt, s.t_sig,
+            (const double*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (double*)wg, eps, s.prm.linear, g.width);
       }
-      return;
-    }
-  }
-  if constexpr (COMP) {
-    if (s.nQ && (which & 1))
-      weno::dev::k_reconstruct_f32c<NV, 12, 8><<<grid_of(s.k1q, s.nQ * NV), s.k1q.block, 0, st>>>(
-          u, ul, s.q_slot, (const float4*)s.q_gop, (const float4*)s.q_dg, (const float4*)s.q_gam,
-          (const float2*)s.q_gam1, (const float*)s.area, s.nQ, s.q_pitch, 0, 0, (float*)wg, eps, s.prm.linear);
-    if (s.nT && (which & 2))
-      weno::dev::k_reconstruct_f32c<NV, 9, 6><<<grid_of(s.k1t, s.nT * NV), s.k1t.block, 0, st>>>(
-          u, ul, s.t_slot, (const float4*)s.t_gop, (const float4*)s.t_dg, (const float4*)s.t_gam,
-          (const float2*)s.t_gam1, (const float*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (float*)wg, eps,
-          s.prm.linear);
-  } else {
-    if (s.nQ && (which & 1)) {
-      const F64Grid g = f64_grid(s, s.nQ, NV, 12, 8, false);
-      weno::dev::k_reconstruct_f64<NV, 12, 8, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
-          u, s.q_slot, (const double*)s.q_gop, (const double*)s.q_dg, (const double*)s.q_gam, s.q_wt, s.q_sig,
-          (const double*)s.area, s.nQ, s.q_pitch, 0, 0, (double*)wg, eps, s.prm.linear, g.width);
-    }
-    if (s.nT && (which & 2)) {
-      const F64Grid g = f64_grid(s, s.nT, NV, 9, 6, false);
-      weno::dev::k_reconstruct_f64<NV, 9, 6, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
-          u, s.t_slot, (const double*)s.t_gop, (const double*)s.t_dg, (const double*)s.t_gam, s.t_wt, s.t_sig,
-          (const double*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (double*)wg, eps, s.prm.linear, g.width);
     }
   }
 }
@@ -323,17 +279,16 @@ void launch_reconstruct_impl(S& s, const void* U, const void* Ulo, void* wg, cud
 // Walls only change the stencil gathers (momentum flips of mirror images); meshes without
 // walls run kernels without that code.
 template <typename T, int NV, bool COMP>
-void launch_reconstruct_into(S& s, const void* U, const void* Ulo, void* wg, cudaStream_t st, int which,
-                             uint8_t* redo) {
+void launch_reconstruct_into(S& s, const void* U, const void* Ulo, void* wg, cudaStream_t st, int which) {
   if constexpr (NV == 4) {
-    if (s.walls) return launch_reconstruct_impl<T, NV, COMP, true>(s, U, Ulo, wg, st, which, redo);
+    if (s.walls) return launch_reconstruct_impl<T, NV, COMP, true>(s, U, Ulo, wg, st, which);
   }
-  launch_reconstruct_impl<T, NV, COMP, false>(s, U, Ulo, wg, st, which, redo);
+  launch_reconstruct_impl<T, NV, COMP, false>(s, U, Ulo, wg, st, which);
 }
 
 template <typename T, int NV, bool COMP>
 void launch_reconstruct(S& s, const void* U, const void* Ulo, cudaStream_t st, int which = 3) {
-  launch_reconstruct_into<T, NV, COMP>(s, U, Ulo, s.Wg, st, which, s.fix_marks);
+  launch_reconstruct_into<T, NV, COMP>(s, U, Ulo, s.Wg, st, which);
 }
 
 template <typename T>
@@ -665,43 +620,16 @@ int setup_tma(S& s) {
   cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
   if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn) return fail(WENO_ECUDA, "cuTensorMapEncodeTiled unavailable");
   EncodeTiled enc = reinterpret_cast<EncodeTiled>(fn);
-  using PQ = weno::dev::PairTile<12, 8>;
-  using PT = weno::dev::PairTile<9, 6>;
+  // point-pair tables: gamma+- (G/2) * M float4 rows, offsets and sigma+- G float4 rows; D_j^+ M rows
+  auto maps = [&](weno::dev::TileMaps& t, void* gam, void* dg, void* gop, int64_t pitch, uint32_t M, uint32_t G) -> int {
+    int r;
+    if ((r = make_map_2d(enc, &t.gam, gam, 4 * pitch, G / 2 * M, 16 * pitch, 4 * kTile, G / 2 * M))) return r;
+    if ((r = make_map_2d(enc, &t.dg, dg, 4 * pitch, G, 16 * pitch, 4 * kTile, G))) return r;
+    return make_map_2d(enc, &t.gop, gop, 4 * pitch, M, 16 * pitch, 4 * kTile, M);
+  };
   int r;
-  // point-pair tables: gamma+- (G/2) * M float4 rows, offsets and sigma+- G float4 rows
-  if (s.nQ) {
-    if ((r = make_map_2d(enc, &s.q_map_pgam, s.q_pgam, 4 * s.q_pitch, 4 * 12, 16 * s.q_pitch, 4 * kTile, 4 * 12)))
-      return r;
-    if ((r = make_map_2d(enc, &s.q_map_pdg, s.q_pdg, 4 * s.q_pitch, 8, 16 * s.q_pitch, 4 * kTile, 8))) return r;
-  }
-  if (s.nT) {
-    if ((r = make_map_2d(enc, &s.t_map_pgam, s.t_pgam, 4 * s.t_pitch, 3 * 9, 16 * s.t_pitch, 4 * kTile, 3 * 9)))
-      return r;
-    if ((r = make_map_2d(enc, &s.t_map_pdg, s.t_pdg, 4 * s.t_pitch, 6, 16 * s.t_pitch, 4 * kTile, 6))) return r;
-  }
-  for (auto fn : {weno::dev::k_reconstruct_tma<12, 8, false, false>, weno::dev::k_reconstruct_tma<12, 8, true, false>,
-                  weno::dev::k_reconstruct_tma<12, 8, false, true>, weno::dev::k_reconstruct_tma<12, 8, true, true>})
-    CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, PQ::SMEM));
-  for (auto fn : {weno::dev::k_reconstruct_tma<9, 6, false, false>, weno::dev::k_reconstruct_tma<9, 6, true, false>,
-                  weno::dev::k_reconstruct_tma<9, 6, false, true>, weno::dev::k_reconstruct_tma<9, 6, true, true>})
-    CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, PT::SMEM));
-  // D_j^+ rows: M float4 rows
-  if (s.nQ && (r = make_map_2d(enc, &s.q_map_gop, s.q_gop, 4 * s.q_pitch, 12, 16 * s.q_pitch, 4 * kTile, 12)))
-    return r;
-  if (s.nT && (r = make_map_2d(enc, &s.t_map_gop, s.t_gop, 4 * s.t_pitch, 9, 16 * s.t_pitch, 4 * kTile, 9)))
-    return r;
-  if (s.prm.characteristic) {
-    for (auto fn : {weno::dev::k_reconstruct_char_tma<12, 8, false, false>,
-                    weno::dev::k_reconstruct_char_tma<12, 8, true, false>,
-                    weno::dev::k_reconstruct_char_tma<12, 8, false, true>,
-                    weno::dev::k_reconstruct_char_tma<12, 8, true, true>})
-      CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, weno::dev::PairTile<12, 8>::SMEM));
-    for (auto fn : {weno::dev::k_reconstruct_char_tma<9, 6, false, false>,
-                    weno::dev::k_reconstruct_char_tma<9, 6, true, false>,
-                    weno::dev::k_reconstruct_char_tma<9, 6, false, true>,
-                    weno::dev::k_reconstruct_char_tma<9, 6, true, true>})
-      CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, weno::dev::PairTile<9, 6>::SMEM));
-  }
+  if (s.nQ && (r = maps(s.q_maps, s.q_pgam, s.q_pdg, s.q_gop, s.q_pitch, 12, 8))) return r;
+  if (s.nT && (r = maps(s.t_maps, s.t_pgam, s.t_pdg, s.t_gop, s.t_pitch, 9, 6))) return r;
   s.tma = true;
   return WENO_OK;
 }
@@ -1088,7 +1016,6 @@ int weno_solver_create(weno_mesh_t mesh, const weno_params* params, void* cuda_s
   CK(cudaMemsetAsync(d.flag, 0, sizeof(int) * d.n_inst, st));
   if ((r = d.alloc(&d.err, sizeof(int)))) return r;
   CK(cudaMemsetAsync(d.err, 0, sizeof(int), st));
-  if (redo_bytes(d) && (r = d.alloc(&d.fix_marks, (size_t)redo_bytes(d)))) return r;
   if (!d.fp64 && d.nv == 4 && (r = setup_tma(d))) return r;
   CK(cudaStreamCreateWithFlags(&d.cap, cudaStreamNonBlocking));
   CK(cudaStreamSynchronize(st));
@@ -1250,7 +1177,7 @@ int weno_autotune(weno_solver_t s, const void* U, const void* U_lo, void* cuda_s
   for (int b : blocks)
     for (int w : waves) generic.push_back(Launch{b, w == 0 ? 0 : w * s->nsm * std::max(1, 2048 / b)});
   // TMA reconstruction: TILE x 4 threads; 1-4 blocks of 256 threads per SM (persistent), or one block per tile
-  for (int w : {0, 1, 2, 3, 4}) tma.push_back(Launch{weno::dev::PairTile<12, 8>::THREADS, w * s->nsm * (64 / kTile)});
+  for (int w : {0, 1, 2, 3, 4}) tma.push_back(Launch{kTile * 4, w * s->nsm * (64 / kTile)});
   auto tune = [&](Launch& L, auto run, const std::vector<Launch>& cands) -> int {
     float best = 1e30f;
     Launch bestL = L;
@@ -1373,9 +1300,8 @@ int static_scratch_base(int dev, void** base) {
 }
 
 template <typename T, int NV, bool COMP>
-void launch_residual_static(S& s, const void* U, const void* Ulo, void* R, void* wg, void* fl, uint8_t* redo,
-                            cudaStream_t st) {
-  launch_reconstruct_into<T, NV, COMP>(s, U, Ulo, wg, st, 3, redo);
+void launch_residual_static(S& s, const void* U, const void* Ulo, void* R, void* wg, void* fl, cudaStream_t st) {
+  launch_reconstruct_into<T, NV, COMP>(s, U, Ulo, wg, st, 3);
   launch_update<T, NV, COMP>(s, 0, 0.0, wg, fl, nullptr, nullptr, R, st);
 }
 
@@ -1383,12 +1309,16 @@ void launch_residual_static(S& s, const void* U, const void* Ulo, void* R, void*
 
 extern "C" int weno_residual_static(weno_solver_t s, const void* U, const void* U_lo, void* R, void* cuda_stream) {
   if (!s || !U || !R || (!s->fp64 && !U_lo)) return fail(WENO_EINVAL, "null argument");
-  // Gauss-point values first, face fluxes after them on a 256-byte boundary, then (FP32C Euler
-  // solvers) the reconstruction's fix-up marks, a byte per tile and a bit per cell
+  // Gauss-point values first, face fluxes after them on a 256-byte boundary; FP32C Euler solvers keep
+  // room for a byte per 16-cell tile and a bit per cell after those (the limit the header states)
   const size_t wg_bytes = (size_t)(8 * s->nQ + 6 * s->nT) * s->nv * s->esz;
   const size_t f_off = (wg_bytes + 255) / 256 * 256;
   const size_t r_off = (f_off + (size_t)s->nF * s->nv * s->esz + 255) / 256 * 256;
-  const size_t need = r_off + (size_t)redo_bytes(*s);
+  auto reserve = [](int64_t n) -> size_t {
+    const int64_t tiles = (n + 15) / 16;
+    return (size_t)((tiles + 15) / 16 * 16 + (2 * tiles + 15) / 16 * 16);
+  };
+  const size_t need = r_off + (!s->fp64 && s->nv == 4 ? reserve(s->nQ) + reserve(s->nT) : 0);
   if (need > kStaticScratchBytes)
     return fail(WENO_EINVAL, "mesh too large for weno_residual_static: needs " + std::to_string(need) +
                                  " bytes of scratch, the fixed array holds " + std::to_string(kStaticScratchBytes));
@@ -1397,6 +1327,6 @@ extern "C" int weno_residual_static(weno_solver_t s, const void* U, const void* 
   int r = static_scratch_base(s->dev, &base);
   if (r) return r;
   unsigned char* b = static_cast<unsigned char*>(base);
-  WENO_DISPATCH(*s, launch_residual_static, *s, U, U_lo, R, b, b + f_off, b + r_off, (cudaStream_t)cuda_stream);
+  WENO_DISPATCH(*s, launch_residual_static, *s, U, U_lo, R, b, b + f_off, (cudaStream_t)cuda_stream);
   return check_launch();
 }
