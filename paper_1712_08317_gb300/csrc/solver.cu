@@ -1204,6 +1204,9 @@ int weno_autotune(weno_solver_t s, const void* U, const void* U_lo, void* cuda_s
   };
   S& d = *s;
   const std::vector<Launch>& k1c = d.tma ? tma : generic;
+  // the passes tuned below work on the Gauss values and fluxes of U
+  WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st);
+  WENO_DISPATCH(d, launch_pass2, d, st);
   if (d.nQ && !d.fp64) tune(d.k1q, [&] { WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st, 1); }, k1c);
   if (d.nT && !d.fp64) tune(d.k1t, [&] { WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st, 2); }, k1c);
   tune(d.k2, [&] { WENO_DISPATCH(d, launch_pass2, d, st); }, generic);

@@ -47,3 +47,13 @@ def test_weights_outside_the_iteration_range_match_oracle(kind):
     W = np.ones((1, mi.n_cells))
     W[0, mi.n_cells // 2] = 1.25
     _compare(mi, W, eqn="scalar", eps=1.6e-154)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32c"])
+def test_autotune_works_on_the_given_state(precision):
+    """The passes are timed on the state's own Gauss values: a physical state raises no flag."""
+    mi = S.mesh_for_config(2, n=21, seed=3, kind="mixed")
+    sol = Solver(Mesh.from_input(mi), eqn="euler", precision=precision)
+    U, Ul = sol.to_device(S.cell_average(mi, S.density_wave))
+    sol.autotune(U, Ul)
+    sol.check()
