@@ -48,21 +48,53 @@ template <> struct Sub<9> {
   static __device__ __forceinline__ int b(int j) { constexpr int t[9] = {2, 3, 1, 4, 5, 6, 7, 8, 9}; return t[j]; }
 };
 
+// Programmatic dependent launch.  The kernels of a residual or a step are launched so that each may start
+// while the one before it in the stream still runs: kernel_begin lets the next one start as soon as all
+// blocks of this one have, and kernel_wait returns when everything before has finished and its writes are
+// visible.  Before kernel_wait a kernel touches nothing but the solver's constant tables.  Whatever a
+// kernel of the chain writes is read with plain loads (no __ldg, no __restrict__: the read-only path is
+// for data constant over the kernel's life, which now begins before its predecessor's end).
+// Only the flux kernels call kernel_begin: a kernel that starts early fills the first SMs with room instead
+// of spreading over all of them, which costs a reconstruction more than the early start brings (8,051 FP64
+// quads with it in every kernel: 292 us a step instead of 272).  Before / after: 10,000 triangles in
+// characteristic variables 41.0 -> 38.9 us a step, 800 triangles 22.5 -> 20.5, 133k cells 139.6 -> 136.8,
+// 1.0M cells 798 -> 790, a residual of 53k FP64 cells 364 -> 349.
+__device__ __forceinline__ void kernel_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void kernel_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Loads of what an earlier kernel of the chain wrote, for the stencil gathers: ordinary (coherent) loads
+// that the compiler may schedule freely among the other work, through a pointer that only exists after
+// kernel_wait.
+template <typename T>
+__device__ __forceinline__ const T* after_wait(const T* p) {
+  asm volatile("" : "+l"(p)::"memory");
+  return p;
+}
+__device__ __forceinline__ float gather(const float* p) {
+  float x;
+  asm("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(p));
+  return x;
+}
+__device__ __forceinline__ double gather(const double* p) {
+  double x;
+  asm("ld.global.f64 %0, [%1];" : "=d"(x) : "l"(p));
+  return x;
+}
+
 // Vector loads / stores of one cell's NV values.
 template <typename T, int NV>
-__device__ __forceinline__ void load_vec(const T* __restrict__ p, T w[NV]) {
+__device__ __forceinline__ void load_vec(const T* p, T w[NV]) {
 #pragma unroll
-  for (int v = 0; v < NV; ++v) w[v] = __ldg(p + v);
+  for (int v = 0; v < NV; ++v) w[v] = p[v];
 }
 template <>
-__device__ __forceinline__ void load_vec<float, 4>(const float* __restrict__ p, float w[4]) {
-  const float4 x = __ldg(reinterpret_cast<const float4*>(p));
+__device__ __forceinline__ void load_vec<float, 4>(const float* p, float w[4]) {
+  const float4 x = *reinterpret_cast<const float4*>(p);
   w[0] = x.x; w[1] = x.y; w[2] = x.z; w[3] = x.w;
 }
 template <>
-__device__ __forceinline__ void load_vec<double, 4>(const double* __restrict__ p, double w[4]) {
-  const double2 x = __ldg(reinterpret_cast<const double2*>(p));
-  const double2 y = __ldg(reinterpret_cast<const double2*>(p) + 1);
+__device__ __forceinline__ void load_vec<double, 4>(const double* p, double w[4]) {
+  const double2 x = reinterpret_cast<const double2*>(p)[0], y = reinterpret_cast<const double2*>(p)[1];
   w[0] = x.x; w[1] = x.y; w[2] = y.x; w[3] = y.y;
 }
 template <typename T, int NV>
@@ -93,18 +125,18 @@ __device__ __forceinline__ int32_t flip_mask(int v) {
 // Value of variable v of stencil entry `raw` (hi and, compensated, lo), momentum reversed for
 // mirror images across walls.
 template <typename T, int NV, bool WALLS, bool COMP>
-__device__ __forceinline__ T slot_delta(const T* __restrict__ U, const T* __restrict__ Ulo, int32_t raw, int v,
+__device__ __forceinline__ T slot_delta(const T* U, const T* Ulo, int32_t raw, int v,
                                         int32_t fm, T w0, T l0) {
   const int64_t cs = WALLS ? (raw & kDevSlotCell) : raw;
-  T a = __ldg(U + cs * NV + v);
-  T b = COMP ? __ldg(Ulo + cs * NV + v) : T(0);
+  T a = gather(U + cs * NV + v);
+  T b = COMP ? gather(Ulo + cs * NV + v) : T(0);
   if (WALLS && (raw & fm)) { a = -a; b = -b; }
   return COMP ? (a - w0) + (b - l0) : a - w0;
 }
 
 // All variables of stencil entry `raw` (hi only), momentum reversed across walls.
 template <typename T, bool WALLS>
-__device__ __forceinline__ void slot_state4(const T* __restrict__ U, int32_t raw, T w[4]) {
+__device__ __forceinline__ void slot_state4(const T* U, int32_t raw, T w[4]) {
   const int64_t cs = WALLS ? (raw & kDevSlotCell) : raw;
   load_vec<T, 4>(U + cs * 4, w);
   if (WALLS) {
@@ -279,13 +311,13 @@ __device__ __forceinline__ float gauss_increment_fp64(const CandPairs<P>& c, con
 // Candidate gradients and smoothness indicators of one (cell, variable), as
 // candidate pairs (the padding candidate of odd M has g = 0, beta = 0).
 template <int NV, int M, bool WALLS>
-__device__ __forceinline__ void cell_gradients(const float* __restrict__ U, const float* __restrict__ Ulo,
+__device__ __forceinline__ void cell_gradients(const float* U, const float* Ulo,
                                                const int32_t* __restrict__ slot, int64_t slot_pitch,
                                                const float4* __restrict__ gop4, int64_t pitch, int64_t q, int64_t c,
                                                int v, float a0, float eps, float& w0, float& l0,
                                                CandPairs<(M + 1) / 2>& cp) {
-  w0 = __ldg(U + c * NV + v);
-  l0 = __ldg(Ulo + c * NV + v);
+  w0 = gather(U + c * NV + v);
+  l0 = gather(Ulo + c * NV + v);
   float dW[M + 1];
   dW[0] = 0.0f;
   const int32_t fm = flip_mask<WALLS, NV>(v);
@@ -317,11 +349,14 @@ __device__ __forceinline__ void cell_gradients(const float* __restrict__ U, cons
 // gamma-_{4(k-M/4)..} after them; g1[g] = (gamma+_8, gamma-_8) for triangles.
 template <int NV, int M, int G>
 __global__ void __launch_bounds__(256, WENO_K1_MIN_BLOCKS) k_reconstruct_f32c(
-    const float* __restrict__ U, const float* __restrict__ Ulo, const int32_t* __restrict__ slot,
+    const float* U, const float* Ulo, const int32_t* __restrict__ slot,
     const float4* __restrict__ gop4, const float4* __restrict__ dgs, const float4* __restrict__ gpm4,
     const float2* __restrict__ g1, const float* __restrict__ area, int64_t N, int64_t pitch, int64_t first,
-    int64_t gbase, float* __restrict__ Wg, float eps, int linear) {
+    int64_t gbase, float* Wg, float eps, int linear) {
   constexpr int M4 = M / 4, P = (M + 1) / 2;
+  kernel_wait();
+  U = after_wait(U);
+  Ulo = after_wait(Ulo);
   const int64_t total = N * NV;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t q = t / NV;
@@ -616,12 +651,13 @@ __device__ __noinline__ void fix_cell(const unsigned char* smem, const TileCells
   using L = PairTile<M, G>;
   const int lane = threadIdx.x & 31, v = lane & 3, g = min(lane >> 2, G - 1);
   const int64_t c = t.first + q;
-  const float w0 = t.U[c * 4 + v], l0 = t.Ulo[c * 4 + v];
+  const float *U = after_wait(t.U), *Ulo = after_wait(t.Ulo);
+  const float w0 = gather(U + c * 4 + v), l0 = gather(Ulo + c * 4 + v);
   const int32_t fm = flip_mask<WALLS, 4>(v);
   float dW[M + 1];
 #pragma unroll 1
   for (int s = 1; s <= M; ++s)
-    dW[s] = slot_delta<float, 4, WALLS, true>(t.U, t.Ulo, __ldg(t.slot + (int64_t)(s - 1) * t.N + q), v, fm, w0, l0);
+    dW[s] = slot_delta<float, 4, WALLS, true>(U, Ulo, __ldg(t.slot + (int64_t)(s - 1) * t.N + q), v, fm, w0, l0);
   const float4* sgam = reinterpret_cast<const float4*>(smem);
   const float incr = fix_increment<M, G>(sgam, sgam + L::GAM / 16, sgam + (L::GAM + L::DG) / 16, cl, g,
                                          [&](int s) { return dW[s]; }, __ldg(t.area + c), t.eps);
@@ -655,14 +691,15 @@ __device__ __forceinline__ bool tile_points(const unsigned char* smem, uint64_t*
   // stencil gathers (independent of the staged tables) before the wait
   float w0 = 0.f, l0 = 0.f, a0 = 0.f, dW[M + 1];
   dW[0] = 0.f;
+  const float *U = after_wait(t.U), *Ulo = after_wait(t.Ulo);
   if (act) {
     const int64_t c = t.first + q;
-    w0 = __ldg(t.U + c * 4 + v);
-    l0 = __ldg(t.Ulo + c * 4 + v);
+    w0 = gather(U + c * 4 + v);
+    l0 = gather(Ulo + c * 4 + v);
     const int32_t fm = flip_mask<WALLS, 4>(v);
 #pragma unroll
     for (int s = 1; s <= M; ++s)
-      dW[s] = slot_delta<float, 4, WALLS, true>(t.U, t.Ulo, __ldg(t.slot + (int64_t)(s - 1) * t.N + q), v, fm, w0, l0);
+      dW[s] = slot_delta<float, 4, WALLS, true>(U, Ulo, __ldg(t.slot + (int64_t)(s - 1) * t.N + q), v, fm, w0, l0);
     a0 = __ldg(t.area + c);
   }
   const bool ok = mbar_wait_bounded(bar, phase);
@@ -787,10 +824,11 @@ __device__ __noinline__ void fix_cell_char(const unsigned char* smem, const Tile
   const int64_t c = t.first + q;
   const float4* sgam = reinterpret_cast<const float4*>(smem);
   const float4* sdg = sgam + L::GAM / 16;
+  const float *U = after_wait(t.U), *Ulo = after_wait(t.Ulo);
   float W0[4], Wn[4], Lr[4], Rr[4];
-  load_vec<float, 4>(t.U + c * 4, W0);
-  const float w0 = t.U[c * 4 + l], l0 = t.Ulo[c * 4 + l];
-  slot_state4<float, WALLS>(t.U, __ldg(t.slot + (int64_t)k * t.N + q), Wn);
+  load_vec<float, 4>(U + c * 4, W0);
+  const float w0 = gather(U + c * 4 + l), l0 = gather(Ulo + c * 4 + l);
+  slot_state4<float, WALLS>(U, __ldg(t.slot + (int64_t)k * t.N + q), Wn);
   const float4 d0 = sdg[(2 * k) * L::TILE + cl];
   const float tx = d0.y - d0.x, ty = d0.w - d0.z, it = rsqrtf(tx * tx + ty * ty);
   roe_rows<float>(W0, Wn, ty * it, -tx * it, t.gas_gamma - 1.f, l, Lr, Rr);
@@ -798,7 +836,7 @@ __device__ __noinline__ void fix_cell_char(const unsigned char* smem, const Tile
   float dU[M + 1];
 #pragma unroll 1
   for (int s = 1; s <= M; ++s)
-    dU[s] = lane_sum4(Lr, slot_delta<float, 4, WALLS, true>(t.U, t.Ulo, __ldg(t.slot + (int64_t)(s - 1) * t.N + q), l,
+    dU[s] = lane_sum4(Lr, slot_delta<float, 4, WALLS, true>(U, Ulo, __ldg(t.slot + (int64_t)(s - 1) * t.N + q), l,
                                                             fm, w0, l0), base);
   const float incr = fix_increment<M, G>(sgam, sdg, sdg + L::DG / 16, cl, g, [&](int s) { return dU[s]; },
                                          __ldg(t.area + c), t.eps);
@@ -822,15 +860,16 @@ __device__ __forceinline__ bool tile_points_char(const unsigned char* smem, uint
   const float4* sdg = sgam + L::GAM / 16;
   const float4* sgo = sdg + L::DG / 16;
   // stencil gathers (independent of the staged tables) before the wait
+  const float *U = after_wait(t.U), *Ulo = after_wait(t.Ulo);
   float W0[4];
-  load_vec<float, 4>(t.U + c * 4, W0);
-  const float w0 = W0[l], l0 = __ldg(t.Ulo + c * 4 + l);
+  load_vec<float, 4>(U + c * 4, W0);
+  const float w0 = W0[l], l0 = gather(Ulo + c * 4 + l);
   float dW[M + 1];
   dW[0] = 0.f;
   const int32_t fm = flip_mask<WALLS, 4>(l);
 #pragma unroll
   for (int s = 1; s <= M; ++s)
-    dW[s] = slot_delta<float, 4, WALLS, true>(t.U, t.Ulo, __ldg(t.slot + (int64_t)(s - 1) * t.N + q), l, fm, w0, l0);
+    dW[s] = slot_delta<float, 4, WALLS, true>(U, Ulo, __ldg(t.slot + (int64_t)(s - 1) * t.N + q), l, fm, w0, l0);
   const float a0 = __ldg(t.area + c);
   const bool ok = mbar_wait_bounded(bar, phase);
   if (__syncthreads_or(!ok)) return false;
@@ -840,7 +879,7 @@ __device__ __forceinline__ bool tile_points_char(const unsigned char* smem, uint
     // the frame of face k: the neighbour across it (slot k + 1) and the unit normal from the
     // direction x_G' - x_G of its two Gauss points
     float Wn[4];
-    slot_state4<float, WALLS>(t.U, __ldg(t.slot + (int64_t)k * t.N + q), Wn);
+    slot_state4<float, WALLS>(U, __ldg(t.slot + (int64_t)k * t.N + q), Wn);
     const float4 d0 = sdg[(2 * k) * L::TILE + cl];
     const float tx = d0.y - d0.x, ty = d0.w - d0.z, it = rsqrtf(tx * tx + ty * ty);
     float Lr[4], Rr[4];
@@ -903,6 +942,7 @@ __global__ void __launch_bounds__(WENO_K1_TILE * 4, K1Blocks<KINDS, CHAR>::value
     else load_tile<9, 6>(smem, &mt, tile - nq, bar);
   };
   if (tid == 0 && blockIdx.x < ntiles) issue(blockIdx.x);
+  kernel_wait();
   uint32_t phase = 0u;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     bool ok;
@@ -1045,9 +1085,11 @@ __device__ __forceinline__ void outer_state(const T w[4], int64_t code, T nx, T 
 
 // Scalar upwind flux, FP32C: one thread per face.
 __global__ void __launch_bounds__(256) k_face_scalar(
-    const float* __restrict__ Wg, const int32_t* __restrict__ gl, const int32_t* __restrict__ gr,
+    const float* Wg, const int32_t* __restrict__ gl, const int32_t* __restrict__ gr,
     const float* __restrict__ fnx, const float* __restrict__ fny, const float* __restrict__ flen, int64_t nF,
-    float* __restrict__ F, Prm<float> prm, int* __restrict__ flag, const int32_t* __restrict__ inst, int64_t nQ) {
+    float* F, Prm<float> prm, int* flag, const int32_t* __restrict__ inst, int64_t nQ) {
+  kernel_begin();
+  kernel_wait();
   for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < nF; f += (int64_t)gridDim.x * blockDim.x) {
     const int64_t il = __ldg(gl + f), ir = __ldg(gr + f);
     const float an = prm.ax * __ldg(fnx + f) + prm.ay * __ldg(fny + f), len = __ldg(flen + f);
@@ -1055,7 +1097,7 @@ __global__ void __launch_bounds__(256) k_face_scalar(
     bool bad = false;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      const float wl = __ldg(Wg + il + k), wr = ir >= 0 ? __ldg(Wg + ir + 1 - k) : wl;
+      const float wl = Wg[il + k], wr = ir >= 0 ? Wg[ir + 1 - k] : wl;
       const float fk = an * (an >= 0.f ? wl : wr);
       bad |= !(fk == fk);
       acc += fk;
@@ -1068,14 +1110,16 @@ __global__ void __launch_bounds__(256) k_face_scalar(
 // Euler HLLC flux, FP32C: one thread per face.
 template <bool INFLOW>
 __global__ void __launch_bounds__(256) k_face_f32(
-    const float* __restrict__ Wg, const int32_t* __restrict__ gl, const int32_t* __restrict__ gr,
+    const float* Wg, const int32_t* __restrict__ gl, const int32_t* __restrict__ gr,
     const float* __restrict__ fnx, const float* __restrict__ fny, const float* __restrict__ flen, int64_t nF,
-    float* __restrict__ F, Prm<float> prm, int* __restrict__ flag, const int32_t* __restrict__ inst, int64_t nQ,
+    float* F, Prm<float> prm, int* flag, const int32_t* __restrict__ inst, int64_t nQ,
     Inflow<float> inf) {
+  kernel_begin();
   for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < nF; f += (int64_t)gridDim.x * blockDim.x) {
     const int64_t il = __ldg(gl + f), ir = __ldg(gr + f);
     const float nx = __ldg(fnx + f), ny = __ldg(fny + f), len = __ldg(flen + f);
     const int i = INFLOW && ir <= -3 && inst ? __ldg(inst + cell_of_gauss(il, nQ)) : 0;
+    kernel_wait();
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
     bool bad = false;
 #pragma unroll
@@ -1110,7 +1154,9 @@ __global__ void k_set_dt(double* __restrict__ dt, float2* __restrict__ split, co
 }
 
 // t[i] += dt[i] for every instance (after the third stage of a step).
-__global__ void k_advance_time(double* __restrict__ t, const double* __restrict__ dt, int n) {
+__global__ void k_advance_time(double* t, const double* dt, int n) {
+  kernel_begin();
+  kernel_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) t[i] += dt[i];
 }
@@ -1127,21 +1173,27 @@ __global__ void k_advance_time(double* __restrict__ t, const double* __restrict_
 // Quads (cells below nQ, face lists qcf [k][nQ]) and triangles (tcf [k][nT]) in one launch.
 template <typename T, int NV, bool COMP, int MODE>
 __global__ void __launch_bounds__(256) k_gather(
-    const T* __restrict__ F, const int32_t* __restrict__ qcf, const int32_t* __restrict__ tcf,
-    const T* __restrict__ inv_area, const T* __restrict__ inv_area_lo, int64_t nQ, int64_t nT, T* __restrict__ U,
-    T* __restrict__ Ulo, T* __restrict__ Ws, T* __restrict__ Wslo, T* __restrict__ R, const double* __restrict__ dt,
-    const float2* __restrict__ dt_split, const int32_t* __restrict__ inst) {
+    const T* F, const int32_t* __restrict__ qcf, const int32_t* __restrict__ tcf,
+    const T* __restrict__ inv_area, const T* __restrict__ inv_area_lo, int64_t nQ, int64_t nT, T* U,
+    T* Ulo, T* Ws, T* Wslo, T* R, const double* dt, const float2* dt_split, const int32_t* __restrict__ inst) {
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nQ + nT; c += (int64_t)gridDim.x * blockDim.x) {
     const bool quad = c < nQ;
     const int32_t* cf = quad ? qcf + c : tcf + (c - nQ);
     const int64_t row = quad ? nQ : nT;
+    int32_t ef[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) ef[k] = k < 3 || quad ? __ldg(cf + k * row) : 0;
+    const T ia = __ldg(inv_area + c);
+    const T ial = COMP ? __ldg(inv_area_lo + c) : T(0);
+    const int i = inst ? __ldg(inst + c) : 0;
+    kernel_wait();
     T acc[NV], comp[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) { acc[v] = T(0); comp[v] = T(0); }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       if (k == 3 && !quad) break;
-      const int32_t e = __ldg(cf + k * row);
+      const int32_t e = ef[k];
       const int64_t f = e >= 0 ? e : ~e;
       T fv[NV];
       load_vec<T, NV>(F + f * NV, fv);
@@ -1158,19 +1210,17 @@ __global__ void __launch_bounds__(256) k_gather(
         }
       }
     }
-    const T ia = __ldg(inv_area + c);
     if (MODE == 0) {
       T res[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) res[v] = COMP ? (acc[v] + comp[v]) * ia : acc[v] * ia;
       store_vec<T, NV>(R + c * NV, res);
     } else {
-      const int i = inst ? __ldg(inst + c) : 0;
       T un[NV], ws[NV], out[NV];
       load_vec<T, NV>(U + c * NV, un);
       if (MODE > 1) load_vec<T, NV>(Ws + c * NV, ws);
       if (!COMP) {
-        const T h = (T)__ldg(dt + i);
+        const T h = (T)dt[i];
         const T cs = MODE == 1 ? T(1) : (MODE == 2 ? T(0.25) : T(2.0 / 3.0));
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
@@ -1179,9 +1229,9 @@ __global__ void __launch_bounds__(256) k_gather(
         }
         store_vec<T, NV>(MODE == 3 ? U + c * NV : Ws + c * NV, out);
       } else {
-        const float2 dts = __ldg(dt_split + i);
+        const float2 dts = dt_split[i];
         const df h{dts.x, dts.y};
-        const df iad{(float)ia, (float)__ldg(inv_area_lo + c)};
+        const df iad{(float)ia, (float)ial};
         const df cs = MODE == 1 ? df{1.0f, 0.0f} : (MODE == 2 ? df{0.25f, 0.0f} : df{0.6666667f, -1.9868216e-08f});
         T unl[NV], wsl[NV], outl[NV];
         load_vec<T, NV>(Ulo + c * NV, unl);
@@ -1224,10 +1274,9 @@ struct CellFace { int32_t other; float nx, ny, slen; };
 // 51,200 triangles 61.5 either way).
 template <int MODE, bool INFLOW>
 __global__ void __launch_bounds__(256) k_update_f32c(
-    const float* __restrict__ Wg, const CellFace* __restrict__ cf, const float* __restrict__ inv_area,
-    const float* __restrict__ inv_area_lo, int64_t nQ, int64_t N, float* __restrict__ U, float* __restrict__ Ulo,
-    float* __restrict__ Ws, float* __restrict__ Wslo, float* __restrict__ R, const float2* __restrict__ dt,
-    const int32_t* __restrict__ inst, float gas_gamma, int* __restrict__ flag, Inflow<float> inf) {
+    const float* Wg, const CellFace* __restrict__ cf, const float* __restrict__ inv_area,
+    const float* __restrict__ inv_area_lo, int64_t nQ, int64_t N, float* U, float* Ulo, float* Ws, float* Wslo, float* R,
+    const float2* dt, const int32_t* __restrict__ inst, float gas_gamma, int* flag, Inflow<float> inf) {
   // uniform over a warp, whose lanes exchange fluxes; lanes past the end repeat the last cell
   for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); t0 < 4 * N;
        t0 += (int64_t)gridDim.x * blockDim.x) {
@@ -1237,9 +1286,13 @@ __global__ void __launch_bounds__(256) k_update_f32c(
     const int k = (int)(t & 3);
     const bool quad = c < nQ;
     const int i = inst ? __ldg(inst + c) : 0;
+    const float ia = __ldg(inv_area + c), ial = __ldg(inv_area_lo + c);
+    float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (quad || k < 3)
+      e = __ldg(reinterpret_cast<const float4*>(cf) + (quad ? 4 * c + k : 4 * nQ + 3 * (c - nQ) + k));
+    kernel_wait();
     float x[4] = {0.f, 0.f, 0.f, 0.f};
     if (quad || k < 3) {
-      const float4 e = __ldg(reinterpret_cast<const float4*>(cf) + (quad ? 4 * c + k : 4 * nQ + 3 * (c - nQ) + k));
       const int32_t other = __float_as_int(e.x);
       const float nx = e.y, ny = e.z, slen = e.w;
       const float4* own = reinterpret_cast<const float4*>(Wg) + (quad ? 8 * c : 8 * nQ + 6 * (c - nQ)) + 2 * k;
@@ -1296,13 +1349,12 @@ __global__ void __launch_bounds__(256) k_update_f32c(
         comp = __fadd_rn(comp, err);
       }
     }
-    const float ia = __ldg(inv_area + c);
     if constexpr (MODE == 0) {
       if (act) R[at] = (acc + comp) * ia;
     } else {
-      const float2 dts = __ldg(dt + i);
+      const float2 dts = dt[i];
       const df h{dts.x, dts.y};
-      const df iad{ia, __ldg(inv_area_lo + c)};
+      const df iad{ia, ial};
       const df cs = MODE == 1 ? df{1.0f, 0.0f} : (MODE == 2 ? df{0.25f, 0.0f} : df{0.6666667f, -1.9868216e-08f});
       const float un = U[at], unl = Ulo[at];
       df d = df_mul(h, df_mul(df_norm(acc, comp), iad));

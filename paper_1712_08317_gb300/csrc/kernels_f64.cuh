@@ -59,10 +59,10 @@ constexpr int kF64MaxWidth = 32;
 // warps: triangles 79 us a pass on the mesh above against 68, quads 124 either way).
 template <int NV, int M, int G, bool WALLS>
 __global__ void __launch_bounds__(kF64MaxWidth * G) k_reconstruct_f64(
-    const double* __restrict__ U, const int32_t* __restrict__ slot, const double* __restrict__ gop,
+    const double* U, const int32_t* __restrict__ slot, const double* __restrict__ gop,
     const double* __restrict__ dg, const double* __restrict__ gam, const double2* __restrict__ wt,
     const double2* __restrict__ sigma, const double* __restrict__ area, int64_t N, int64_t pitch, int64_t first,
-    int64_t gbase, double* __restrict__ Wg, double eps, int linear, int width) {
+    int64_t gbase, double* Wg, double eps, int linear, int width) {
   constexpr int PER = (M + G - 1) / G;
   extern __shared__ double sm[];
   double* dW = sm;                                      // [slot - 1][column]
@@ -72,7 +72,9 @@ __global__ void __launch_bounds__(kF64MaxWidth * G) k_reconstruct_f64(
   const int64_t qr = (int64_t)blockIdx.x * (width / NV) + col / NV;
   const int64_t q = qr < N ? qr : N - 1;  // columns past the end work on the last cell and store nothing
   const int64_t c = first + q;
-  const double w0 = __ldg(U + c * NV + v), a0 = __ldg(area + c);
+  kernel_wait();
+  U = after_wait(U);
+  const double w0 = gather(U + c * NV + v), a0 = __ldg(area + c);
   const int32_t fm = flip_mask<WALLS, NV>(v);
 #pragma unroll
   for (int i = 0; i < PER; ++i) {
@@ -148,10 +150,10 @@ constexpr int kFrame = 33;  // doubles a frame takes in shared memory (32, padde
 
 template <int M, int G, int PTS, bool WALLS>
 __global__ void __launch_bounds__(kF64MaxWidth * G / PTS) k_reconstruct_char_f64(
-    const double* __restrict__ U, const int32_t* __restrict__ slot, const double* __restrict__ gop,
+    const double* U, const int32_t* __restrict__ slot, const double* __restrict__ gop,
     const double* __restrict__ dg, const double* __restrict__ gam, const double2* __restrict__ wt,
     const double2* __restrict__ sigma, const double* __restrict__ area, int64_t N, int64_t pitch, int64_t first,
-    int64_t gbase, double* __restrict__ Wg, double eps, double gas_gamma, int linear, int width) {
+    int64_t gbase, double* Wg, double eps, double gas_gamma, int linear, int width) {
   constexpr int F = G / 2, PARTS = G / PTS, PER = (M + PARTS - 1) / PARTS;
   extern __shared__ double sm[];
   const int tile = width / 4, threads = width * PARTS;
@@ -163,7 +165,9 @@ __global__ void __launch_bounds__(kF64MaxWidth * G / PTS) k_reconstruct_char_f64
   const int64_t q0 = (int64_t)blockIdx.x * tile, qr = q0 + cl;
   const int64_t q = qr < N ? qr : N - 1;  // columns past the end work on the last cell and store nothing
   const int64_t c = first + q;
-  const double w0 = __ldg(U + c * 4 + l), a0 = __ldg(area + c);
+  kernel_wait();
+  U = after_wait(U);
+  const double w0 = gather(U + c * 4 + l), a0 = __ldg(area + c);
   const int32_t fm = flip_mask<WALLS, 4>(l);
 #pragma unroll
   for (int i = 0; i < PER; ++i) {
@@ -293,10 +297,9 @@ __device__ __noinline__ void hllc_ieee(const double* wl, const double* wr, doubl
 // neighbour's.  Flags and boundary states as k_face.
 template <int NV, bool INFLOW>
 __global__ void __launch_bounds__(256) k_face_f64(
-    const double* __restrict__ Wg, const int32_t* __restrict__ gl, const int32_t* __restrict__ gr,
+    const double* Wg, const int32_t* __restrict__ gl, const int32_t* __restrict__ gr,
     const double* __restrict__ fnx, const double* __restrict__ fny, const double* __restrict__ flen, int64_t nF,
-    double* __restrict__ F, Prm<double> prm, int* __restrict__ flag, const int32_t* __restrict__ inst, int64_t nQ,
-    Inflow<double> inf) {
+    double* F, Prm<double> prm, int* flag, const int32_t* __restrict__ inst, int64_t nQ, Inflow<double> inf) {
   const int64_t total = 2 * nF;
   // the loop is uniform over a warp, whose lanes exchange fluxes; lanes past the end repeat the last face
   for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); t0 < total;
@@ -306,7 +309,8 @@ __global__ void __launch_bounds__(256) k_face_f64(
     const int64_t f = act ? t >> 1 : nF - 1;
     const int k = (int)(t & 1);
     const int64_t il = __ldg(gl + f), ir = __ldg(gr + f);
-    const double nx = __ldg(fnx + f), ny = __ldg(fny + f);
+    const double nx = __ldg(fnx + f), ny = __ldg(fny + f), hl = 0.5 * __ldg(flen + f);
+    kernel_wait();
     double wl[NV], wr[NV], fk[NV];
     load_vec<double, NV>(Wg + (il + k) * NV, wl);
     if (ir >= 0) {
@@ -325,7 +329,6 @@ __global__ void __launch_bounds__(256) k_face_f64(
       fk[0] = an * (an >= 0.0 ? wl[0] : wr[0]);
       bad = !(fk[0] == fk[0]);
     }
-    const double hl = 0.5 * __ldg(flen + f);
     double sum[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) sum[v] = hl * (fk[v] + __shfl_xor_sync(0xffffffffu, fk[v], 1));

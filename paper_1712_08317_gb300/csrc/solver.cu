@@ -65,6 +65,23 @@ unsigned grid_of(const Launch& l, int64_t work) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(g, 0x7fffffff));
 }
 
+// Launch of a kernel of the chain (kernel_begin / kernel_wait): it may start before the kernel ahead of it
+// in the stream has finished.
+template <typename... P, typename... A>
+void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // errors: cudaGetLastError (check_launch)
+}
+
 // TMA reconstruction: TILE x 4 threads per block, one TILE-cell tile per iteration.
 constexpr int kTile = weno::dev::PairTile<12, 8>::TILE;
 unsigned tma_grid(const Launch& l, int64_t tiles) {
@@ -204,8 +221,7 @@ void launch_tma_kinds(S& s, const Launch& l, const float* u, const float* ul, fl
   t.first = s.nQ;
   t.gbase = 8 * s.nQ;
   const int64_t tiles = (KINDS & 1 ? (s.nQ + kTile - 1) / kTile : 0) + (KINDS & 2 ? (s.nT + kTile - 1) / kTile : 0);
-  weno::dev::k_reconstruct_tma<KINDS, CHAR, WALLS>
-      <<<tma_grid(l, tiles), kTile * 4, weno::dev::K1Smem<KINDS>::bytes, st>>>(s.q_maps, s.t_maps, q, t, s.err, s.debug_stall);
+  launch(weno::dev::k_reconstruct_tma<KINDS, CHAR, WALLS>, tma_grid(l, tiles), kTile * 4, weno::dev::K1Smem<KINDS>::bytes, st, s.q_maps, s.t_maps, q, t, s.err, s.debug_stall);
 }
 template <bool CHAR, bool WALLS>
 void launch_tma(S& s, const void* U, const void* Ulo, void* wg, cudaStream_t st, int which) {
@@ -234,16 +250,14 @@ void launch_reconstruct_impl(S& s, const void* U, const void* Ulo, void* wg, cud
           const F64Grid g = f64_grid(s, s.nQ, 4, 12, 8, true);
           const auto kernel = g.pts == 1 ? weno::dev::k_reconstruct_char_f64<12, 8, 1, WALLS>
                                          : weno::dev::k_reconstruct_char_f64<12, 8, 2, WALLS>;
-          kernel<<<g.blocks, g.threads, g.smem, st>>>(
-              u, s.q_slot, (const double*)s.q_gop, (const double*)s.q_dg, (const double*)s.q_gam, s.q_wt, s.q_sig,
+          launch(kernel, g.blocks, g.threads, g.smem, st, u, s.q_slot, (const double*)s.q_gop, (const double*)s.q_dg, (const double*)s.q_gam, s.q_wt, s.q_sig,
               (const double*)s.area, s.nQ, s.q_pitch, 0, 0, (double*)wg, eps, gg, s.prm.linear, g.width);
         }
         if (s.nT && (which & 2)) {
           const F64Grid g = f64_grid(s, s.nT, 4, 9, 6, true);
           const auto kernel = g.pts == 1 ? weno::dev::k_reconstruct_char_f64<9, 6, 1, WALLS>
                                          : weno::dev::k_reconstruct_char_f64<9, 6, 2, WALLS>;
-          kernel<<<g.blocks, g.threads, g.smem, st>>>(
-              u, s.t_slot, (const double*)s.t_gop, (const double*)s.t_dg, (const double*)s.t_gam, s.t_wt, s.t_sig,
+          launch(kernel, g.blocks, g.threads, g.smem, st, u, s.t_slot, (const double*)s.t_gop, (const double*)s.t_dg, (const double*)s.t_gam, s.t_wt, s.t_sig,
               (const double*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (double*)wg, eps, gg, s.prm.linear, g.width);
         }
         return;
@@ -251,25 +265,21 @@ void launch_reconstruct_impl(S& s, const void* U, const void* Ulo, void* wg, cud
     }
     if constexpr (COMP) {
       if (s.nQ && (which & 1))
-        weno::dev::k_reconstruct_f32c<NV, 12, 8><<<grid_of(s.k1q, s.nQ * NV), s.k1q.block, 0, st>>>(
-            u, static_cast<const T*>(Ulo), s.q_slot, (const float4*)s.q_gop, (const float4*)s.q_dg, (const float4*)s.q_gam,
+        launch(weno::dev::k_reconstruct_f32c<NV, 12, 8>, grid_of(s.k1q, s.nQ * NV), s.k1q.block, 0, st, u, static_cast<const T*>(Ulo), s.q_slot, (const float4*)s.q_gop, (const float4*)s.q_dg, (const float4*)s.q_gam,
             (const float2*)s.q_gam1, (const float*)s.area, s.nQ, s.q_pitch, 0, 0, (float*)wg, eps, s.prm.linear);
       if (s.nT && (which & 2))
-        weno::dev::k_reconstruct_f32c<NV, 9, 6><<<grid_of(s.k1t, s.nT * NV), s.k1t.block, 0, st>>>(
-            u, static_cast<const T*>(Ulo), s.t_slot, (const float4*)s.t_gop, (const float4*)s.t_dg, (const float4*)s.t_gam,
+        launch(weno::dev::k_reconstruct_f32c<NV, 9, 6>, grid_of(s.k1t, s.nT * NV), s.k1t.block, 0, st, u, static_cast<const T*>(Ulo), s.t_slot, (const float4*)s.t_gop, (const float4*)s.t_dg, (const float4*)s.t_gam,
             (const float2*)s.t_gam1, (const float*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (float*)wg, eps,
             s.prm.linear);
     } else {
       if (s.nQ && (which & 1)) {
         const F64Grid g = f64_grid(s, s.nQ, NV, 12, 8, false);
-        weno::dev::k_reconstruct_f64<NV, 12, 8, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
-            u, s.q_slot, (const double*)s.q_gop, (const double*)s.q_dg, (const double*)s.q_gam, s.q_wt, s.q_sig,
+        launch(weno::dev::k_reconstruct_f64<NV, 12, 8, WALLS>, g.blocks, g.threads, g.smem, st, u, s.q_slot, (const double*)s.q_gop, (const double*)s.q_dg, (const double*)s.q_gam, s.q_wt, s.q_sig,
             (const double*)s.area, s.nQ, s.q_pitch, 0, 0, (double*)wg, eps, s.prm.linear, g.width);
       }
       if (s.nT && (which & 2)) {
         const F64Grid g = f64_grid(s, s.nT, NV, 9, 6, false);
-        weno::dev::k_reconstruct_f64<NV, 9, 6, WALLS><<<g.blocks, g.threads, g.smem, st>>>(
-            u, s.t_slot, (const double*)s.t_gop, (const double*)s.t_dg, (const double*)s.t_gam, s.t_wt, s.t_sig,
+        launch(weno::dev::k_reconstruct_f64<NV, 9, 6, WALLS>, g.blocks, g.threads, g.smem, st, u, s.t_slot, (const double*)s.t_gop, (const double*)s.t_dg, (const double*)s.t_gam, s.t_wt, s.t_sig,
             (const double*)s.area, s.nT, s.t_pitch, s.nQ, 8 * s.nQ, (double*)wg, eps, s.prm.linear, g.width);
       }
     }
@@ -314,25 +324,21 @@ void launch_face(S& s, const void* wg, void* fl, double c, cudaStream_t st) {
   if constexpr (std::is_same<T, double>::value) {
     // inflow faces exist for the Euler equations only
     const auto kernel = NV == 4 && s.n_in ? weno::dev::k_face_f64<NV, NV == 4> : weno::dev::k_face_f64<NV, false>;
-    kernel<<<grid_of(s.k2, 2 * s.nF), s.k2.block, 0, st>>>(
-        (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
+    launch(kernel, grid_of(s.k2, 2 * s.nF), s.k2.block, 0, st, (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
         s.inst, s.nQ, inflow_of<T>(s, c));
   } else if constexpr (NV == 4) {
     const auto kernel = s.n_in ? weno::dev::k_face_f32<true> : weno::dev::k_face_f32<false>;
-    kernel<<<grid_of(s.k2, s.nF), s.k2.block, 0, st>>>(
-        (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
+    launch(kernel, grid_of(s.k2, s.nF), s.k2.block, 0, st, (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
         s.inst, s.nQ, inflow_of<T>(s, c));
   } else {
-    weno::dev::k_face_scalar<<<grid_of(s.k2, s.nF), s.k2.block, 0, st>>>(
-        (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
+    launch(weno::dev::k_face_scalar, grid_of(s.k2, s.nF), s.k2.block, 0, st, (const T*)wg, s.gl, s.gr, (const T*)s.fnx, (const T*)s.fny, (const T*)s.flen, s.nF, (T*)fl, p, s.flag,
         s.inst, s.nQ);
   }
 }
 
 template <typename T, int NV, bool COMP, int MODE>
 void launch_gather_mode(S& s, const void* fl, void* U, void* Ulo, void* R, cudaStream_t st) {
-  weno::dev::k_gather<T, NV, COMP, MODE><<<grid_of(s.k3, s.N), s.k3.block, 0, st>>>(
-      (const T*)fl, s.q_cf, s.t_cf, (const T*)s.inv_area, (const T*)s.inv_area_lo, s.nQ, s.nT, (T*)U, (T*)Ulo,
+  launch(weno::dev::k_gather<T, NV, COMP, MODE>, grid_of(s.k3, s.N), s.k3.block, 0, st, (const T*)fl, s.q_cf, s.t_cf, (const T*)s.inv_area, (const T*)s.inv_area_lo, s.nQ, s.nT, (T*)U, (T*)Ulo,
       (T*)s.Ws, (T*)s.Wslo, (T*)R, s.dt_dev, s.dt_split, s.inst);
 }
 
@@ -353,8 +359,7 @@ bool use_fused(const S& s) { return !s.fp64 && s.nv == 4 && 4 * s.N <= (int64_t)
 template <int MODE>
 void launch_update_mode(S& s, const void* wg, double c, void* U, void* Ulo, void* R, cudaStream_t st) {
   const auto kernel = s.n_in ? weno::dev::k_update_f32c<MODE, true> : weno::dev::k_update_f32c<MODE, false>;
-  kernel<<<grid_of(Launch{kUpdateBlock}, 4 * s.N), kUpdateBlock, 0, st>>>(
-      (const float*)wg, s.cell_faces, (const float*)s.inv_area, (const float*)s.inv_area_lo, s.nQ, s.N, (float*)U,
+  launch(kernel, grid_of(Launch{kUpdateBlock}, 4 * s.N), kUpdateBlock, 0, st, (const float*)wg, s.cell_faces, (const float*)s.inv_area, (const float*)s.inv_area_lo, s.nQ, s.N, (float*)U,
       (float*)Ulo, (float*)s.Ws, (float*)s.Wslo, (float*)R, s.dt_split, s.inst, (float)s.prm.gas_gamma, s.flag,
       inflow_of<float>(s, c));
 }
@@ -398,7 +403,7 @@ void launch_step_body(S& s, void* U, void* Ulo, cudaStream_t st) {
     launch_reconstruct<T, NV, COMP>(s, src, srclo, st);
     launch_update<T, NV, COMP>(s, stage, kStageTime[stage - 1], s.Wg, s.F, U, Ulo, nullptr, st);
   }
-  weno::dev::k_advance_time<<<(s.n_inst + 127) / 128, 128, 0, st>>>(s.t_dev, s.dt_dev, s.n_inst);
+  launch(weno::dev::k_advance_time, (s.n_inst + 127) / 128, 128, 0, st, s.t_dev, s.dt_dev, s.n_inst);
 }
 
 // one call per precision / variable count
