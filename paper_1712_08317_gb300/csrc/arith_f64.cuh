@@ -76,15 +76,32 @@ template <int M> __device__ __forceinline__ int sub_b(int j) { return (int)(SubB
 // What a Gauss point needs of one candidate: gradient, beta + eps, beta^2, beta^3.
 struct CandF64 { double gx, gy, be, b2, b3; };
 
+// beta + eps is set to infinity where beta^3 overflows, so that face_points_f64 sees it.
 __device__ __forceinline__ CandF64 candidate_f64(double gx, double gy, double a0, double eps) {
-  const double b = a0 * (gx * gx + gy * gy), b2 = b * b;
-  return CandF64{gx, gy, b + eps, b2, b2 * b};
+  const double b = a0 * (gx * gx + gy * gy), b2 = b * b, b3 = b2 * b;
+  return CandF64{gx, gy, hi_word(b3) < 0x7ff00000u ? b + eps : __longlong_as_double(0x7ff0000000000000ll), b2, b3};
 }
 
 // Positive numbers t 2^(e - 1086) with a 64-bit t (the value of a biased FP64 exponent e and a mantissa
-// left-justified in t): the nonlinear weights and their sums are formed on the integer pipe, which the
-// FP64 pipe never sees.
+// left-justified in t; t may have a few leading zeros): the indicators, the nonlinear weights and their
+// sums are formed on the integer pipe, which the FP64 pipe never sees.  Each operation below loses less
+// than 2^-58 of its result; all numbers are positive, so nothing cancels.
 struct PosNum { uint64_t t; int e; };
+
+// A positive FP64 number; zero and subnormals become about 2^-1023.
+__device__ __forceinline__ PosNum pos_of(double x) {
+  const uint32_t h = hi_word(x), l = (uint32_t)__double2loint(x);
+  return PosNum{(uint64_t)(0x80000000u | __funnelshift_l(l, h, 11)) << 32 | (l << 11), (int)(h >> 20)};
+}
+__device__ __forceinline__ PosNum pos_mul(PosNum a, PosNum b) {
+  const uint32_t ah = (uint32_t)(a.t >> 32), al = (uint32_t)a.t, bh = (uint32_t)(b.t >> 32), bl = (uint32_t)b.t;
+  return PosNum{(uint64_t)ah * bh + __umulhi(ah, bl) + __umulhi(al, bh), a.e + b.e - 1022};
+}
+__device__ __forceinline__ PosNum pos_sum(PosNum a, PosNum b) {
+  const int de = a.e - b.e;
+  const uint64_t big = de < 0 ? b.t : a.t, small = de < 0 ? a.t : b.t;
+  return PosNum{(big >> 1) + (small >> min(abs(de) + 1, 63)), max(a.e, b.e) + 1};
+}
 
 // 2^64 / m for m = (mh, ml) / 2^63 in [1, 2), low by at most 2^-58: Newton's iteration r <- r + r (1 - r m)
 // from the single-precision reciprocal's seed, biased to stay below 1/m (so that 1 - r m >= 0 and all
@@ -105,22 +122,20 @@ __device__ __forceinline__ double pos_to_f64(uint64_t t, int e) {
   return e <= 0 ? 0.0 : __longlong_as_double((long long)bits);
 }
 
-// gamma / d^2 for 0 <= gamma <= 1 and d in [2^-510, 2^400): 5 FP64 instructions, 320 cycles of a warp, in
-// FP64; here about 55 integer ones and a single-precision reciprocal, good to 2^-57.  gamma below 2^-1022
-// comes out smaller than 2^-900 of any weight that matters.
-__device__ __forceinline__ PosNum alpha_f64(double gamma, double d) {
-  const uint32_t dh = hi_word(d), dl = (uint32_t)__double2loint(d), gh = hi_word(gamma), gl = (uint32_t)__double2loint(gamma);
-  const uint64_t r = recip_fixed(0x80000000u | __funnelshift_l(dl, dh, 11), dl << 11);
+// gamma / d^2 for 0 <= gamma <= 1 and d in [2^-510, 2^400), good to 2^-56, with a normalised t; e_d gets
+// the biased exponent of d.  gamma below 2^-1022 comes out smaller than 2^-900 of any weight that matters.
+__device__ __forceinline__ PosNum pos_alpha(PosNum gamma, PosNum d, int& e_d) {
+  const int ld = __clzll((long long)d.t);
+  const uint64_t m = d.t << ld, r = recip_fixed((uint32_t)(m >> 32), (uint32_t)m);
   const uint32_t rh = (uint32_t)(r >> 32), rl = (uint32_t)r;
-  const uint64_t s = (uint64_t)rh * rh + (((uint64_t)rh * rl) >> 31);  // 2^64 / m^2
-  const uint32_t sh = (uint32_t)(s >> 32), sl = (uint32_t)s;
-  const uint32_t g1 = 0x80000000u | __funnelshift_l(gl, gh, 11), g0 = gl << 11;
-  const uint64_t t = (uint64_t)sh * g1 + __umulhi(sh, g0) + __umulhi(sl, g1);  // in (2^61, 2^64)
-  const int lz = __clz((int)(uint32_t)(t >> 32));
-  return PosNum{t << lz, (int)(gh >> 20) - 2 * (int)(dh >> 20) + 2046 - lz};
+  e_d = d.e - ld;
+  const PosNum s{(uint64_t)rh * rh + (((uint64_t)rh * rl) >> 31), 3068 - 2 * e_d};  // 1 / d^2
+  const PosNum a = pos_mul(s, gamma);                                              // t in [2^61, 2^64)
+  const int lz = __clz((int)(uint32_t)(a.t >> 32));
+  return PosNum{a.t << lz, a.e - lz};
 }
-// The range of d above, as bounds of its high word.
-constexpr uint32_t kAlphaHiMin = (1023u - 510u) << 20, kAlphaHiMax = (1023u + 400u) << 20;
+// The range of d above, as biased exponents.
+constexpr int kAlphaExpMin = 1023 - 510, kAlphaExpMax = 1023 + 400;
 
 // Sum of up to 16 weights: four bits of headroom in t instead of a carry, so 2^-59 of the sum is lost.
 __device__ __forceinline__ PosNum pos_first(PosNum a) { return PosNum{a.t >> 4, a.e}; }
@@ -143,24 +158,30 @@ __device__ __forceinline__ double pos_rcp(PosNum s) {
 // the split weights wt(h, j) = (gamma+, gamma-) of point h:
 //   alpha+- = gamma+- / (beta~+- + eps)^2,  beta~+- + eps = (beta + eps) + gamma (beta^2 + gamma beta^3),
 //   R - W0 = sigma+ sum alpha+ p / sum alpha+  -  sigma- sum alpha- p / sum alpha-.
-// 8 FP64 instructions per point and candidate.  Returns false if an indicator left the range of
-// alpha_f64 (or was NaN): the increments are then redone by face_points_ieee.
+// Only p and the sums of alpha p are FP64, 4 instructions per point and candidate.  Returns false if an
+// indicator left the range of pos_alpha (or was NaN): the increments are then redone by face_points_ieee.
 template <int M, int PTS, typename Cand, typename Weights>
 __device__ __forceinline__ bool face_points_f64(Cand cand, Weights wt, const double* dx, const double* dy,
                                                 const double2* sig, double* incr) {
   PosNum Ap[PTS], Am[PTS];
   double Bp[PTS], Bm[PTS];
-  uint32_t lo = 0xffffffffu, hi = 0u;
+  int lo = kAlphaExpMax, hi = 0;
+  auto weight = [&](double g, PosNum be, PosNum b2, PosNum b3) {
+    const PosNum gamma = pos_of(g);
+    int e;
+    const PosNum a = pos_alpha(gamma, pos_sum(be, pos_mul(gamma, pos_sum(b2, pos_mul(gamma, b3)))), e);
+    lo = min(lo, e);
+    hi = max(hi, e);
+    return a;
+  };
   auto one = [&](int j, bool first) {
     const CandF64 c = cand(j);
+    const PosNum be = pos_of(c.be), b2 = pos_of(c.b2), b3 = pos_of(c.b3);
 #pragma unroll
     for (int h = 0; h < PTS; ++h) {
       const double2 g = wt(h, j);
       const double p = c.gx * dx[h] + c.gy * dy[h];
-      const double dp = fma(g.x, fma(g.x, c.b3, c.b2), c.be), dn = fma(g.y, fma(g.y, c.b3, c.b2), c.be);
-      lo = min(lo, min(hi_word(dp), hi_word(dn)));
-      hi = max(hi, max(hi_word(dp), hi_word(dn)));
-      const PosNum ap = alpha_f64(g.x, dp), an = alpha_f64(g.y, dn);
+      const PosNum ap = weight(g.x, be, b2, b3), an = weight(g.y, be, b2, b3);
       const double vp = pos_to_f64(ap.t, ap.e), vn = pos_to_f64(an.t, an.e);
       Ap[h] = first ? pos_first(ap) : pos_add(Ap[h], ap);
       Am[h] = first ? pos_first(an) : pos_add(Am[h], an);
@@ -173,7 +194,7 @@ __device__ __forceinline__ bool face_points_f64(Cand cand, Weights wt, const dou
   for (int j = 1; j < M; ++j) one(j, false);
 #pragma unroll
   for (int h = 0; h < PTS; ++h) incr[h] = sig[h].x * (Bp[h] * pos_rcp(Ap[h])) - sig[h].y * (Bm[h] * pos_rcp(Am[h]));
-  return lo >= kAlphaHiMin && hi < kAlphaHiMax;
+  return lo >= kAlphaExpMin && hi < kAlphaExpMax;
 }
 
 // The same with IEEE division and the indicator as printed, beta (1 + q + q^2) with q = gamma beta:

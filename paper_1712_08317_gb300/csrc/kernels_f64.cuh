@@ -8,14 +8,14 @@
 //   - the splitting of the linear weights (geometry only) is done once per solver (k_split_weights),
 //   - differences, gradients and indicators are computed once per (cell, variable) and shared through
 //     shared memory by the threads of the cell's faces,
-//   - the new indicator is a polynomial in the split weight, two fused multiply-adds,
-//   - the nonlinear weights gamma / d^2 are formed on the integer pipe (alpha_f64),
+//   - the indicators, the nonlinear weights and their sums are formed on the integer pipe (PosNum),
 //   - other reciprocals start from the special-function unit's 20-bit seed and take one third-order step.
 // K1 measured (one pass; first: one thread per (cell, variable), IEEE division, the splitting repeated
 // by every variable, 5,350 FP64 issue slots a (cell, variable) of quads; then: as here with all of the
-// weights in FP64, 2,140 slots; then: gamma / d^2 on the integer pipe, 1,200; now: their sums too, 940):
-// 17,920 Euler quads 662 -> 277 -> 154 -> 124 us, 15,360 triangles 384 -> 144 -> 83 -> 68 us, 1,600 scalar
-// quads 332 -> 30 us and now 18; the FP64 pipe is 86 % busy, the issue slots 32 %.
+// weights in FP64, 2,140 slots; then: gamma / d^2 on the integer pipe, 1,200; their sums too, 940; now: the
+// indicators d too, 560): 17,920 Euler quads 662 -> 277 -> 154 -> 124 -> 103 us, 15,360 triangles
+// 384 -> 144 -> 83 -> 68 -> 57 us, 1,600 scalar quads 332 -> 30 us and now 18.  The FP64 pipe is 66 % and the
+// integer pipe 62 % busy: the two now balance, and what is left is how well they overlap.
 #pragma once
 
 #include "kernels.cuh"
