@@ -1373,87 +1373,151 @@ __global__ void __launch_bounds__(256) k_update_f32c(
 }
 
 // ---------------------------------------------------------------- K4 (reductions, not on the hot path)
-// Per-cell stable step 2|Omega| / sum_p (|v.n_p| + c)|l_p| (FP64).
-template <typename T, int NV, int NFACE, bool COMP>
-__global__ void k_cell_dt(const T* __restrict__ U, const T* __restrict__ Ulo, const int32_t* __restrict__ cf,
-                          const double* __restrict__ fnx, const double* __restrict__ fny,
-                          const double* __restrict__ flen, const double* __restrict__ area, int64_t N,
-                          int64_t first, double gas_gamma, double ax, double ay, double* __restrict__ out) {
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < N; q += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = first + q;
-    double w[NV];
-    for (int v = 0; v < NV; ++v) w[v] = (double)U[c * NV + v] + (COMP ? (double)Ulo[c * NV + v] : 0.0);
-    double u = ax, vv = ay, snd = 0.0;
-    if (NV == 4) {
-      u = w[1] / w[0];
-      vv = w[2] / w[0];
-      const double p = (gas_gamma - 1.0) * (w[3] - 0.5 * w[0] * (u * u + vv * vv));
-      snd = sqrt(gas_gamma * p / w[0]);
-    }
-    double s = 0.0;
-    for (int k = 0; k < NFACE; ++k) {
-      const int32_t e = cf[(int64_t)k * N + q];
-      const int64_t f = e >= 0 ? e : ~e;
-      s += (fabs(u * fnx[f] + vv * fny[f]) + snd) * flen[f];
-    }
-    out[c] = 2.0 * area[c] / s;
-  }
+// Largest stable step min 2|Omega| / sum_p (|v.n_p| + c)|l_p| and integrals sum |Omega| (U + U_lo) of each
+// instance, in FP64 and in two levels over a fixed partition (`chunks`), so that results do not depend on
+// scheduling.  What bounds them is the FP64 pipe (2 lanes a clock and SM) and, on small meshes, latency:
+// the time step is formed and reduced in one kernel with the reciprocals and roots of arith_f64.cuh (39
+// FP64 instructions a quad, not about 110 with IEEE division), FP32 states are widened on the integer
+// pipe, minima are taken on the bits of the numbers, and a chunk is as many cells as spread a mesh over
+// all SMs.
+// 260k FP32C cells, both results: 170 -> 80 us (k_chunk_dt 24, k_chunk_sum 14, the rest launches and waits for
+// the host); 8k FP64 quads, time step: 27 us less.
+
+// A float as a double by integer operations, except for subnormals, infinities and NaN.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), m = b & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+  return m == 0 ? __hiloint2double((int)b, 0) : (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// The state of cell c in FP64.
+template <typename T, int NV, bool COMP>
+__device__ __forceinline__ void state_f64(const T* __restrict__ U, const T* __restrict__ Ulo, int64_t c, double w[NV]) {
+  T h[NV], l[NV];
+  load_vec<T, NV>(U + c * NV, h);
+  if (COMP) load_vec<T, NV>(Ulo + c * NV, l);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) w[v] = COMP ? widen(h[v]) + widen(l[v]) : widen(h[v]);
 }
 
-// Deterministic reductions in two levels with a fixed partition, so results do
-// not depend on scheduling.  Level 1: one block per chunk [c0, c1) of cells of
-// one instance; mode 0: min of x[c]; mode 1: sums of area[c] * (U + U_lo)[c][v].
+// Half of a cell's stable step, |Omega| / sum_p (|v.n_p| + c)|l_p|; never negative, NaN for a negative pressure.
+template <int NV, int NFACE>
+__device__ __forceinline__ double half_dt(const double w[NV], const int32_t* __restrict__ cf, int64_t row,
+                                          const double* __restrict__ fnx, const double* __restrict__ fny,
+                                          const double* __restrict__ flen, double area, double gas_gamma, double ax,
+                                          double ay) {
+  double u = ax, vv = ay, snd = 0.0;
+  if constexpr (NV == 4) {
+    const double r = rcp_any(w[0]);
+    u = w[1] * r;
+    vv = w[2] * r;
+    const double p = (gas_gamma - 1.0) * (w[3] - 0.5 * (w[1] * u + w[2] * vv));
+    snd = sqrt_any(gas_gamma * p * r);
+  }
+  double s = 0.0;
+#pragma unroll
+  for (int k = 0; k < NFACE; ++k) {
+    const int32_t e = __ldg(cf + k * row);
+    const int64_t f = e >= 0 ? e : ~e;
+    s += (fabs(u * __ldg(fnx + f) + vv * __ldg(fny + f)) + snd) * __ldg(flen + f);
+  }
+  return area * rcp_any(s);
+}
+
+// Smaller of two numbers that are >= 0 or NaN, by their bits: a NaN of either sign is above every number,
+// so it is left out like by fmin.
+__device__ __forceinline__ uint64_t bits_of(double x) { return (uint64_t)__double_as_longlong(x); }
+__device__ __forceinline__ uint64_t block_min(uint64_t m) {
+  __shared__ uint64_t sh[8];
+#pragma unroll
+  for (int o = 16; o; o >>= 1) m = min(m, (uint64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)m, o));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) m = min(m, sh[i]);
+  return m;
+}
+constexpr double kNoDt = 0.5e300;  // where no cell has a step
+
+// Level 1, time step: one block per chunk [c0, c1) of cells of one instance and one type.
+template <typename T, int NV, bool COMP>
+__global__ void __launch_bounds__(256) k_chunk_dt(
+    const T* __restrict__ U, const T* __restrict__ Ulo, const int32_t* __restrict__ qcf,
+    const int32_t* __restrict__ tcf, const double* __restrict__ fnx, const double* __restrict__ fny,
+    const double* __restrict__ flen, const double* __restrict__ area, const int64_t* __restrict__ chunks, int64_t nQ,
+    int64_t nT, double gas_gamma, double ax, double ay, double* __restrict__ partial) {
+  kernel_begin();
+  const int64_t c0 = __ldg(chunks + 2 * blockIdx.x), c1 = __ldg(chunks + 2 * blockIdx.x + 1);
+  uint64_t m = bits_of(kNoDt);
+  for (int64_t c = c0 + threadIdx.x; c < c1; c += 256) {
+    double w[NV];
+    state_f64<T, NV, COMP>(U, Ulo, c, w);
+    const double a = __ldg(area + c);
+    const double h = c < nQ ? half_dt<NV, 4>(w, qcf + c, nQ, fnx, fny, flen, a, gas_gamma, ax, ay)
+                            : half_dt<NV, 3>(w, tcf + (c - nQ), nT, fnx, fny, flen, a, gas_gamma, ax, ay);
+    m = min(m, bits_of(h));
+  }
+  m = block_min(m);
+  if (threadIdx.x == 0) partial[blockIdx.x] = __longlong_as_double((long long)m);
+}
+
+// Level 1, integrals.
 template <int NV>
-__device__ __forceinline__ void block_reduce_store(double acc[NV], int mode, double* __restrict__ out) {
+__device__ __forceinline__ void block_sum_store(const double acc[NV], double* __restrict__ out) {
   __shared__ double sh[256 * NV];
+#pragma unroll
   for (int v = 0; v < NV; ++v) sh[v * 256 + threadIdx.x] = acc[v];
   __syncthreads();
   for (int s = 128; s > 0; s >>= 1) {
     if ((int)threadIdx.x < s)
-      for (int v = 0; v < NV; ++v) {
-        const double a = sh[v * 256 + threadIdx.x], b = sh[v * 256 + threadIdx.x + s];
-        sh[v * 256 + threadIdx.x] = mode == 0 ? fmin(a, b) : a + b;
-      }
+      for (int v = 0; v < NV; ++v) sh[v * 256 + threadIdx.x] += sh[v * 256 + threadIdx.x + s];
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    if (mode == 0) out[0] = sh[0];
-    else for (int v = 0; v < NV; ++v) out[v] = sh[v * 256];
-  }
+  if (threadIdx.x < NV) out[threadIdx.x] = sh[threadIdx.x * 256];
 }
-
 template <typename T, int NV, bool COMP>
-__global__ void __launch_bounds__(256) k_chunk_reduce(const double* __restrict__ x, const T* __restrict__ U,
-                                                      const T* __restrict__ Ulo, const double* __restrict__ area,
-                                                      const int64_t* __restrict__ chunks, int mode,
-                                                      double* __restrict__ partial) {
-  const int64_t c0 = chunks[2 * blockIdx.x], c1 = chunks[2 * blockIdx.x + 1];
+__global__ void __launch_bounds__(256) k_chunk_sum(const T* __restrict__ U, const T* __restrict__ Ulo,
+                                                   const double* __restrict__ area,
+                                                   const int64_t* __restrict__ chunks, double* __restrict__ partial) {
+  kernel_begin();
+  const int64_t c0 = __ldg(chunks + 2 * blockIdx.x), c1 = __ldg(chunks + 2 * blockIdx.x + 1);
   double acc[NV];
-  for (int v = 0; v < NV; ++v) acc[v] = mode == 0 ? 1e300 : 0.0;
-  for (int64_t c = c0 + threadIdx.x; c < c1; c += blockDim.x) {
-    if (mode == 0) {
-      acc[0] = fmin(acc[0], x[c]);
-    } else {
-      for (int v = 0; v < NV; ++v)
-        acc[v] += area[c] * ((double)U[c * NV + v] + (COMP ? (double)Ulo[c * NV + v] : 0.0));
-    }
+#pragma unroll
+  for (int v = 0; v < NV; ++v) acc[v] = 0.0;
+  for (int64_t c = c0 + threadIdx.x; c < c1; c += 256) {
+    double w[NV];
+    state_f64<T, NV, COMP>(U, Ulo, c, w);
+    const double a = __ldg(area + c);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) acc[v] += a * w[v];
   }
-  block_reduce_store<NV>(acc, mode, partial + (int64_t)blockIdx.x * (mode == 0 ? 1 : NV));
+  block_sum_store<NV>(acc, partial + (int64_t)blockIdx.x * NV);
 }
 
-// Level 2: one block per instance over its chunks' partials [k0, k1).
+// Level 2: one block per instance over its chunks' partials [k0, k1); out is in the host's memory.
+__global__ void __launch_bounds__(256) k_instance_dt(const double* partial, const int64_t* __restrict__ chunk_off,
+                                                     double* out) {
+  const int64_t k0 = __ldg(chunk_off + blockIdx.x), k1 = __ldg(chunk_off + blockIdx.x + 1);
+  kernel_wait();
+  uint64_t m = bits_of(kNoDt);
+  for (int64_t k = k0 + threadIdx.x; k < k1; k += 256) m = min(m, bits_of(partial[k]));
+  m = block_min(m);
+  if (threadIdx.x == 0) out[blockIdx.x] = 2.0 * __longlong_as_double((long long)m);
+}
 template <int NV>
-__global__ void __launch_bounds__(256) k_instance_reduce(const double* __restrict__ partial,
-                                                         const int64_t* __restrict__ chunk_off, int mode,
-                                                         double* __restrict__ out) {
-  const int inst = blockIdx.x;
-  const int64_t k0 = chunk_off[inst], k1 = chunk_off[inst + 1];
-  const int w = mode == 0 ? 1 : NV;
+__global__ void __launch_bounds__(256) k_instance_sum(const double* partial, const int64_t* __restrict__ chunk_off,
+                                                      double* out) {
+  const int64_t k0 = __ldg(chunk_off + blockIdx.x), k1 = __ldg(chunk_off + blockIdx.x + 1);
+  kernel_wait();
   double acc[NV];
-  for (int v = 0; v < NV; ++v) acc[v] = mode == 0 ? 1e300 : 0.0;
-  for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x)
-    for (int v = 0; v < w; ++v) acc[v] = mode == 0 ? fmin(acc[v], partial[k]) : acc[v] + partial[k * NV + v];
-  block_reduce_store<NV>(acc, mode, out + (int64_t)inst * w);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) acc[v] = 0.0;
+  for (int64_t k = k0 + threadIdx.x; k < k1; k += 256)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) acc[v] += partial[k * NV + v];
+  block_sum_store<NV>(acc, out + (int64_t)blockIdx.x * NV);
 }
 
 __global__ void k_fill(double* __restrict__ p, double v, int n) {

@@ -134,7 +134,8 @@ struct weno_solver_s {
   // scratch
   void *Wg = nullptr, *F = nullptr, *Ws = nullptr, *Wslo = nullptr;
   float2* dt_split = nullptr;  // dt_dev as (hi, lo), for the FP32C stages
-  double *dt_dev = nullptr, *red = nullptr, *cell_dt = nullptr;
+  double* dt_dev = nullptr;
+  double* red = nullptr;     // results of the reductions, in pinned host memory that the device writes
   double* t_dev = nullptr;   // time of each instance (advanced by every step)
   int64_t n_in = 0;          // inflow faces
   double* in_xi = nullptr;   // [n_in][2] n . x_G - c0 of their Gauss points
@@ -158,6 +159,7 @@ struct weno_solver_s {
     for (auto& x : graphs) cudaGraphExecDestroy(x.exec);
     if (cap) cudaStreamDestroy(cap);
     for (void* p : allocs) cudaFree(p);
+    if (red) cudaFreeHost(red);
   }
   template <typename P>
   int alloc(P** p, size_t bytes) {
@@ -418,26 +420,22 @@ void launch_step_body(S& s, void* U, void* Ulo, cudaStream_t st) {
     }                                                              \
   } while (0)
 
+// Level 1 of a reduction follows whatever the stream holds; level 2 may start before it has drained.
 template <typename T, int NV, bool COMP>
-void launch_cell_dt(S& s, const void* U, const void* Ulo, cudaStream_t st) {
-  const T* u = (const T*)U;
-  const T* ul = (const T*)Ulo;
-  if (s.nQ)
-    weno::dev::k_cell_dt<T, NV, 4, COMP><<<(unsigned)((s.nQ + 255) / 256), 256, 0, st>>>(
-        u, ul, s.q_cf, s.fnx64, s.fny64, s.flen64, s.area64, s.nQ, 0, s.prm.gas_gamma, s.prm.adv[0], s.prm.adv[1],
-        s.cell_dt);
-  if (s.nT)
-    weno::dev::k_cell_dt<T, NV, 3, COMP><<<(unsigned)((s.nT + 255) / 256), 256, 0, st>>>(
-        u, ul, s.t_cf, s.fnx64, s.fny64, s.flen64, s.area64, s.nT, s.nQ, s.prm.gas_gamma, s.prm.adv[0],
-        s.prm.adv[1], s.cell_dt);
+void launch_max_dt(S& s, const void* U, const void* Ulo, cudaStream_t st) {
+  if (s.n_chunks)
+    weno::dev::k_chunk_dt<T, NV, COMP><<<(unsigned)s.n_chunks, 256, 0, st>>>(
+        (const T*)U, (const T*)Ulo, s.q_cf, s.t_cf, s.fnx64, s.fny64, s.flen64, s.area64, s.chunks, s.nQ, s.nT,
+        s.prm.gas_gamma, s.prm.adv[0], s.prm.adv[1], s.partial);
+  launch(weno::dev::k_instance_dt, s.n_inst, 256, 0, st, s.partial, s.chunk_off, s.red);
 }
 
 template <typename T, int NV, bool COMP>
-void launch_reduce(S& s, const void* U, const void* Ulo, int mode, cudaStream_t st) {
+void launch_sums(S& s, const void* U, const void* Ulo, cudaStream_t st) {
   if (s.n_chunks)
-    weno::dev::k_chunk_reduce<T, NV, COMP><<<(unsigned)s.n_chunks, 256, 0, st>>>(
-        s.cell_dt, (const T*)U, (const T*)Ulo, s.area64, s.chunks, mode, s.partial);
-  weno::dev::k_instance_reduce<NV><<<s.n_inst, 256, 0, st>>>(s.partial, s.chunk_off, mode, s.red);
+    weno::dev::k_chunk_sum<T, NV, COMP><<<(unsigned)s.n_chunks, 256, 0, st>>>(
+        (const T*)U, (const T*)Ulo, s.area64, s.chunks, s.partial);
+  launch(weno::dev::k_instance_sum<NV>, s.n_inst, 256, 0, st, s.partial, s.chunk_off, s.red);
 }
 
 int check_launch() {
@@ -984,14 +982,16 @@ int weno_solver_create(weno_mesh_t mesh, const weno_params* params, void* cuda_s
       ranges[4 * i + part + 1] = c + 1;
     }
     for (auto& x : ranges) if (x < 0) x = 0;
-    // fixed partition of each instance's quad and triangle ranges into chunks (deterministic reductions)
-    constexpr int64_t kChunk = 8192;
+    // fixed partition of each instance's quad and triangle ranges into chunks, a block each (deterministic
+    // reductions): 256 cells, one a thread, up to about eight blocks an SM, then multiples of 256 so that
+    // the second level, one block an instance, stays short
+    const int64_t chunk = 256 * ((d.N + 256 * 8 * d.nsm - 1) / (256 * 8 * d.nsm));
     std::vector<int64_t> chunks, chunk_off(1, 0);
     for (int i = 0; i < d.n_inst; ++i) {
       for (int part = 0; part < 2; ++part)
-        for (int64_t c = ranges[4 * i + 2 * part]; c < ranges[4 * i + 2 * part + 1]; c += kChunk) {
+        for (int64_t c = ranges[4 * i + 2 * part]; c < ranges[4 * i + 2 * part + 1]; c += chunk) {
           chunks.push_back(c);
-          chunks.push_back(std::min(c + kChunk, ranges[4 * i + 2 * part + 1]));
+          chunks.push_back(std::min(c + chunk, ranges[4 * i + 2 * part + 1]));
         }
       chunk_off.push_back((int64_t)chunks.size() / 2);
     }
@@ -1015,8 +1015,7 @@ int weno_solver_create(weno_mesh_t mesh, const weno_params* params, void* cuda_s
   if ((r = d.alloc(&d.t_dev, sizeof(double) * d.n_inst))) return r;
   CK(cudaMemsetAsync(d.t_dev, 0, sizeof(double) * d.n_inst, st));
   CK(cudaMemsetAsync(d.dt_dev, 0, sizeof(double) * d.n_inst, st));
-  if ((r = d.alloc(&d.red, sizeof(double) * d.n_inst * d.nv))) return r;
-  if ((r = d.alloc(&d.cell_dt, sizeof(double) * d.N))) return r;
+  CK(cudaHostAlloc((void**)&d.red, sizeof(double) * d.n_inst * d.nv, cudaHostAllocPortable | cudaHostAllocMapped));
   if ((r = d.alloc(&d.flag, sizeof(int) * d.n_inst))) return r;
   CK(cudaMemsetAsync(d.flag, 0, sizeof(int) * d.n_inst, st));
   if ((r = d.alloc(&d.err, sizeof(int)))) return r;
@@ -1095,14 +1094,11 @@ int weno_max_dt(weno_solver_t s, const void* U, const void* U_lo, double cfl, do
   if (!s || !U || !dt_out || (!s->fp64 && !U_lo)) return fail(WENO_EINVAL, "null argument");
   DeviceGuard g(s->dev);
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  WENO_DISPATCH(*s, launch_cell_dt, *s, U, U_lo, st);
-  WENO_DISPATCH(*s, launch_reduce, *s, U, U_lo, 0, st);
+  WENO_DISPATCH(*s, launch_max_dt, *s, U, U_lo, st);
   int r = check_launch();
   if (r) return r;
-  std::vector<double> h(s->n_inst);
-  CK(cudaMemcpyAsync(h.data(), s->red, sizeof(double) * s->n_inst, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  for (int i = 0; i < s->n_inst; ++i) dt_out[i] = cfl * h[i];
+  for (int i = 0; i < s->n_inst; ++i) dt_out[i] = cfl * s->red[i];
   return WENO_OK;
 }
 
@@ -1110,11 +1106,11 @@ int weno_conservation(weno_solver_t s, const void* U, const void* U_lo, double* 
   if (!s || !U || !sums || (!s->fp64 && !U_lo)) return fail(WENO_EINVAL, "null argument");
   DeviceGuard g(s->dev);
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  WENO_DISPATCH(*s, launch_reduce, *s, U, U_lo, 1, st);
+  WENO_DISPATCH(*s, launch_sums, *s, U, U_lo, st);
   int r = check_launch();
   if (r) return r;
-  CK(cudaMemcpyAsync(sums, s->red, sizeof(double) * s->n_inst * s->nv, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
+  std::memcpy(sums, s->red, sizeof(double) * s->n_inst * s->nv);
   return WENO_OK;
 }
 
