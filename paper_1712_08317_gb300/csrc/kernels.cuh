@@ -81,6 +81,10 @@ __device__ __forceinline__ double gather(const double* p) {
   return x;
 }
 
+// Products that the compiler may not merge into a following addition.
+__device__ __forceinline__ float mulr(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mulr(double a, double b) { return __dmul_rn(a, b); }
+
 // Vector loads / stores of one cell's NV values.
 template <typename T, int NV>
 __device__ __forceinline__ void load_vec(const T* p, T w[NV]) {
@@ -664,15 +668,27 @@ __device__ __noinline__ void fix_cell(const unsigned char* smem, const TileCells
   if (lane < 4 * G) t.Wg[(t.gbase + q * G + g) * 4 + v] = w0 + (l0 + incr);
 }
 
-// Calls fix(q, cell of the tile) for each cell of the warp with a lane that has `bad` set.  Warp 8 cells
-// wide: lanes 4i..4i+3 of warp w hold cell 8w + i of the tile.
-template <typename Fix>
+// Calls fix(q, cell of the tile) for each cell of the tile with a lane that has `bad` set, on the warp of the
+// first TILE x 4 threads that holds it: lanes 4i..4i+3 of warp w hold cell 8w + i of the tile.  With PARTS > 1
+// the block has that many warps for every such cell, which agree on it first: none of the cell's regular
+// values is then still to be stored.
+template <int PARTS, typename Fix>
 __device__ __forceinline__ void fix_marked(bool bad, int64_t q0, Fix fix) {
+  constexpr int WARPS = WENO_K1_TILE / 8;
   uint32_t m = __ballot_sync(0xffffffffu, bad);
+  const int w = threadIdx.x >> 5;
+  if constexpr (PARTS > 1) {
+    if (!__syncthreads_or((int)m)) return;
+    __shared__ uint32_t marks[PARTS * WARPS];
+    if ((threadIdx.x & 31) == 0) marks[w] = m;
+    __syncthreads();
+    if (w >= WARPS) return;
+    for (int i = 1; i < PARTS; ++i) m |= marks[w + i * WARPS];
+  }
   while (m) {
     const int i = (__ffs(m) - 1) >> 2;
     m &= ~(0xfu << (4 * i));
-    const int cl = 8 * (threadIdx.x >> 5) + i;
+    const int cl = 8 * w + i;
     fix(q0 + cl, cl);
   }
 }
@@ -707,7 +723,7 @@ __device__ __forceinline__ bool tile_points(const unsigned char* smem, uint64_t*
   bool bad = false;
   if (act)
     bad = !pair_points<M, G>(sgam, sdg, sgo, cl, dW, a0, t.eps, t.linear, w0, l0, t.Wg + (t.gbase + q * G) * 4 + v);
-  fix_marked(bad, tile * L::TILE, [&](int64_t qf, int cf) { fix_cell<M, G, WALLS>(smem, t, qf, cf); });
+  fix_marked<1>(bad, tile * L::TILE, [&](int64_t qf, int cf) { fix_cell<M, G, WALLS>(smem, t, qf, cf); });
   return true;
 }
 
@@ -720,43 +736,44 @@ __device__ __forceinline__ bool tile_points(const unsigned char* smem, uint64_t*
 // reconstructs field l, and returns variable l of W0 + R dU with row l of R.
 // Reconstructing the increment dU (zero for constant data) keeps constant
 // states exact whatever the rounding of R R^-1.
-template <typename T>
-__device__ __forceinline__ T lane_sum4(const T c[4], T x, int base) {
-  T r = T(0);
+// Products here are rounded or inside an explicit fma, so that the instances of the kernel (one that walks
+// the faces and keeps the cell's part of a frame, one with a thread for each) give the same bits.
+__device__ __forceinline__ float lane_sum4(const float c[4], float x, int base) {
+  float r = mulr(c[0], __shfl_sync(0xffffffffu, x, base));
 #pragma unroll
-  for (int i = 0; i < 4; ++i) r += c[i] * __shfl_sync(0xffffffffu, x, base + i);
+  for (int i = 1; i < 4; ++i) r = fmaf(c[i], __shfl_sync(0xffffffffu, x, base + i), r);
   return r;
 }
 
 // Roe frame of one face for lane l: row l of R^-1 (Lr) and row l of R (Rr), fields ordered
 // q_n - a, entropy, shear, q_n + a, from the two cells' averages and the outward unit normal.
-template <typename T>
-__device__ __forceinline__ void roe_rows(const T Wl[4], const T Wr[4], T nx, T ny, T gm1, int l, T Lr[4],
-                                         T Rr[4]) {
-  const T rl = Wl[0], ul = Wl[1] / rl, vl = Wl[2] / rl;
-  const T hl = (Wl[3] + gm1 * (Wl[3] - T(0.5) * rl * (ul * ul + vl * vl))) / rl;
-  const T rr = Wr[0], ur = Wr[1] / rr, vr = Wr[2] / rr;
-  const T hr = (Wr[3] + gm1 * (Wr[3] - T(0.5) * rr * (ur * ur + vr * vr))) / rr;
-  const T sl = sqrt(rl), sr = sqrt(rr), iw = T(1) / (sl + sr);
-  const T u = (sl * ul + sr * ur) * iw, v = (sl * vl + sr * vr) * iw, H = (sl * hl + sr * hr) * iw;
-  const T kin = T(0.5) * (u * u + v * v);
-  const T a = sqrt(gm1 * (H - kin)), ia = T(1) / a;
-  const T qn = u * nx + v * ny, qt = v * nx - u * ny;
-  const T b1 = gm1 * ia * ia, b2 = b1 * kin;
+__device__ __forceinline__ void roe_rows(const float Wl[4], const float Wr[4], float nx, float ny, float gm1, int l,
+                                         float Lr[4], float Rr[4]) {
+  const float rl = Wl[0], ul = Wl[1] / rl, vl = Wl[2] / rl;
+  const float hl = fmaf(gm1, fmaf(-mulr(0.5f, rl), fmaf(ul, ul, mulr(vl, vl)), Wl[3]), Wl[3]) / rl;
+  const float rr = Wr[0], ur = Wr[1] / rr, vr = Wr[2] / rr;
+  const float hr = fmaf(gm1, fmaf(-mulr(0.5f, rr), fmaf(ur, ur, mulr(vr, vr)), Wr[3]), Wr[3]) / rr;
+  const float sl = sqrtf(rl), sr = sqrtf(rr), iw = 1.f / (sl + sr);
+  const float u = mulr(fmaf(sl, ul, mulr(sr, ur)), iw), v = mulr(fmaf(sl, vl, mulr(sr, vr)), iw);
+  const float H = mulr(fmaf(sl, hl, mulr(sr, hr)), iw);
+  const float kin = mulr(0.5f, fmaf(u, u, mulr(v, v)));
+  const float a = sqrtf(mulr(gm1, H - kin)), ia = 1.f / a;
+  const float qn = fmaf(u, nx, mulr(v, ny)), qt = fmaf(v, nx, -mulr(u, ny));
+  const float b1 = mulr(mulr(gm1, ia), ia), b2 = mulr(b1, kin);
   if (l == 0) {
-    Lr[0] = T(0.5) * (b2 + qn * ia); Lr[1] = T(-0.5) * (b1 * u + nx * ia);
-    Lr[2] = T(-0.5) * (b1 * v + ny * ia); Lr[3] = T(0.5) * b1;
-    Rr[0] = T(1); Rr[1] = T(1); Rr[2] = T(0); Rr[3] = T(1);
+    Lr[0] = mulr(0.5f, fmaf(qn, ia, b2)); Lr[1] = mulr(-0.5f, fmaf(b1, u, mulr(nx, ia)));
+    Lr[2] = mulr(-0.5f, fmaf(b1, v, mulr(ny, ia))); Lr[3] = mulr(0.5f, b1);
+    Rr[0] = 1.f; Rr[1] = 1.f; Rr[2] = 0.f; Rr[3] = 1.f;
   } else if (l == 1) {
-    Lr[0] = T(1) - b2; Lr[1] = b1 * u; Lr[2] = b1 * v; Lr[3] = -b1;
-    Rr[0] = u - a * nx; Rr[1] = u; Rr[2] = -ny; Rr[3] = u + a * nx;
+    Lr[0] = 1.f - b2; Lr[1] = mulr(b1, u); Lr[2] = mulr(b1, v); Lr[3] = -b1;
+    Rr[0] = fmaf(-a, nx, u); Rr[1] = u; Rr[2] = -ny; Rr[3] = fmaf(a, nx, u);
   } else if (l == 2) {
-    Lr[0] = -qt; Lr[1] = -ny; Lr[2] = nx; Lr[3] = T(0);
-    Rr[0] = v - a * ny; Rr[1] = v; Rr[2] = nx; Rr[3] = v + a * ny;
+    Lr[0] = -qt; Lr[1] = -ny; Lr[2] = nx; Lr[3] = 0.f;
+    Rr[0] = fmaf(-a, ny, v); Rr[1] = v; Rr[2] = nx; Rr[3] = fmaf(a, ny, v);
   } else {
-    Lr[0] = T(0.5) * (b2 - qn * ia); Lr[1] = T(0.5) * (nx * ia - b1 * u);
-    Lr[2] = T(0.5) * (ny * ia - b1 * v); Lr[3] = T(0.5) * b1;
-    Rr[0] = H - a * qn; Rr[1] = kin; Rr[2] = qt; Rr[3] = H + a * qn;
+    Lr[0] = mulr(0.5f, fmaf(-qn, ia, b2)); Lr[1] = mulr(0.5f, fmaf(nx, ia, -mulr(b1, u)));
+    Lr[2] = mulr(0.5f, fmaf(ny, ia, -mulr(b1, v))); Lr[3] = mulr(0.5f, b1);
+    Rr[0] = fmaf(-a, qn, H); Rr[1] = kin; Rr[2] = qt; Rr[3] = fmaf(a, qn, H);
   }
 }
 
@@ -811,8 +828,8 @@ __device__ __forceinline__ bool face_pair(const float4* __restrict__ sgam, const
     Am = __fadd2_rn(Am, an);
     Bm = __ffma2_rn(an, p, Bm);
   }
-  incr = f2(s.x * Bp.x * rcp_approx(Ap.x) - s.z * Bm.x * rcp_approx(Am.x),
-            s.y * Bp.y * rcp_approx(Ap.y) - s.w * Bm.y * rcp_approx(Am.y));
+  incr = f2(fmaf(mulr(s.x, Bp.x), rcp_approx(Ap.x), -mulr(mulr(s.z, Bm.x), rcp_approx(Am.x))),
+            fmaf(mulr(s.y, Bp.y), rcp_approx(Ap.y), -mulr(mulr(s.w, Bm.y), rcp_approx(Am.y))));
   return !(Ap.x < kAlphaMin) && !(Ap.y < kAlphaMin) && !(Am.x < kAlphaMin) && !(Am.y < kAlphaMin);
 }
 
@@ -830,8 +847,8 @@ __device__ __noinline__ void fix_cell_char(const unsigned char* smem, const Tile
   const float w0 = gather(U + c * 4 + l), l0 = gather(Ulo + c * 4 + l);
   slot_state4<float, WALLS>(U, __ldg(t.slot + (int64_t)k * t.N + q), Wn);
   const float4 d0 = sdg[(2 * k) * L::TILE + cl];
-  const float tx = d0.y - d0.x, ty = d0.w - d0.z, it = rsqrtf(tx * tx + ty * ty);
-  roe_rows<float>(W0, Wn, ty * it, -tx * it, t.gas_gamma - 1.f, l, Lr, Rr);
+  const float tx = d0.y - d0.x, ty = d0.w - d0.z, it = rsqrtf(fmaf(tx, tx, mulr(ty, ty)));
+  roe_rows(W0, Wn, ty * it, -tx * it, t.gas_gamma - 1.f, l, Lr, Rr);
   const int32_t fm = flip_mask<WALLS, 4>(l);
   float dU[M + 1];
 #pragma unroll 1
@@ -847,11 +864,12 @@ __device__ __noinline__ void fix_cell_char(const unsigned char* smem, const Tile
 // One tile in characteristic variables.  Per face, each lane builds the Roe frame, projects the stencil
 // differences onto its field and evaluates the face's two Gauss points with face_pair; lanes of cells
 // past the end compute on the last cell's data and store nothing.
-template <int M, int G, bool WALLS>
+template <int M, int G, int PARTS, bool WALLS>
 __device__ __forceinline__ bool tile_points_char(const unsigned char* smem, uint64_t* bar, uint32_t phase,
                                                  const TileCells& t, int64_t tile) {
   using L = PairTile<M, G>;
-  const int tid = threadIdx.x, base = (tid & 31) & ~3, l = tid & 3, cl = tid >> 2;
+  const int tid = threadIdx.x % L::THREADS, part = threadIdx.x / L::THREADS;
+  const int base = (tid & 31) & ~3, l = tid & 3, cl = tid >> 2;
   const int64_t qr = tile * L::TILE + cl;
   const bool act = qr < t.N;
   const int64_t q = act ? qr : t.N - 1;
@@ -875,15 +893,15 @@ __device__ __forceinline__ bool tile_points_char(const unsigned char* smem, uint
   if (__syncthreads_or(!ok)) return false;
   bool inrange = true;  // every sum of alpha of this lane's Gauss points within the FP32 range
 #pragma unroll 1
-  for (int k = 0; k < G / 2; ++k) {
+  for (int k = part; k < G / 2; k += PARTS) {
     // the frame of face k: the neighbour across it (slot k + 1) and the unit normal from the
     // direction x_G' - x_G of its two Gauss points
     float Wn[4];
     slot_state4<float, WALLS>(U, __ldg(t.slot + (int64_t)k * t.N + q), Wn);
     const float4 d0 = sdg[(2 * k) * L::TILE + cl];
-    const float tx = d0.y - d0.x, ty = d0.w - d0.z, it = rsqrtf(tx * tx + ty * ty);
+    const float tx = d0.y - d0.x, ty = d0.w - d0.z, it = rsqrtf(fmaf(tx, tx, mulr(ty, ty)));
     float Lr[4], Rr[4];
-    roe_rows<float>(W0, Wn, ty * it, -tx * it, t.gas_gamma - 1.f, l, Lr, Rr);
+    roe_rows(W0, Wn, ty * it, -tx * it, t.gas_gamma - 1.f, l, Lr, Rr);
     float dU[M + 1];
     dU[0] = 0.f;
 #pragma unroll
@@ -898,7 +916,7 @@ __device__ __forceinline__ bool tile_points_char(const unsigned char* smem, uint
   }
   // a cell's four lanes mix all fields, so it is redone whole; lanes past the end read the zero fill of
   // the tables and are left out
-  fix_marked(act && !inrange, tile * L::TILE, [&](int64_t qf, int cf) { fix_cell_char<M, G, WALLS>(smem, t, qf, cf); });
+  fix_marked<PARTS>(act && !inrange, tile * L::TILE, [&](int64_t qf, int cf) { fix_cell_char<M, G, WALLS>(smem, t, qf, cf); });
   return true;
 }
 
@@ -912,20 +930,28 @@ __device__ __forceinline__ bool tile_points_char(const unsigned char* smem, uint
 // the quads' 16 warps, whose 122 registers spill when cut to 96)
 #define WENO_K1_BLOCKS_T (WENO_K1_MIN_BLOCKS * 96 / WENO_K1_TILE)  // resident blocks per SM, triangles
 #endif
-// The register budget: 65,536 / (blocks x TILE x 4) per thread.
-template <int KINDS, bool CHAR> struct K1Blocks {
-  static constexpr int value = CHAR ? WENO_KCHAR_MIN_BLOCKS * 64 / WENO_K1_TILE : KINDS == 2 ? WENO_K1_BLOCKS_T : WENO_K1_BLOCKS_Q;
+// Threads of a block.  SPLIT (characteristic variables on small meshes): TILE x 4 threads for every face instead
+// of threads that walk the faces, whose frames, projections and candidates are one serial chain of about
+// 600 instructions a face; what is repeated is the gathers.  80 registers (768 threads an SM; with 64, which
+// spill more, 6,400 quads take 33.0 us a step instead of 30.9).
+template <int KINDS, bool SPLIT> struct K1Threads {
+  static constexpr int value = WENO_K1_TILE * 4 * (!SPLIT ? 1 : KINDS & 1 ? 4 : 3);
+};
+// The register budget: 65,536 / (blocks x threads) per thread.
+template <int KINDS, bool CHAR, bool SPLIT> struct K1Blocks {
+  static constexpr int value = SPLIT ? 768 / K1Threads<KINDS, true>::value
+      : CHAR ? WENO_KCHAR_MIN_BLOCKS * 64 / WENO_K1_TILE : KINDS == 2 ? WENO_K1_BLOCKS_T : WENO_K1_BLOCKS_Q;
 };
 template <int KINDS> struct K1Smem {
   static constexpr int quad = PairTile<12, 8>::STAGE, tri = PairTile<9, 6>::STAGE;
   static constexpr int stage = (KINDS & 1) ? quad : tri, bytes = stage + 16;  // one buffer + one mbarrier (padded)
 };
 
-template <int KINDS, bool CHAR, bool WALLS>
-__global__ void __launch_bounds__(WENO_K1_TILE * 4, K1Blocks<KINDS, CHAR>::value) k_reconstruct_tma(
+template <int KINDS, bool CHAR, bool WALLS, bool SPLIT>
+__global__ void __launch_bounds__(K1Threads<KINDS, SPLIT>::value, K1Blocks<KINDS, CHAR, SPLIT>::value) k_reconstruct_tma(
     const __grid_constant__ TileMaps mq, const __grid_constant__ TileMaps mt, const __grid_constant__ TileCells tq,
     const __grid_constant__ TileCells tt, int* __restrict__ err, int stall) {
-  constexpr int TILE = WENO_K1_TILE;
+  constexpr int TILE = WENO_K1_TILE, PARTS = K1Threads<KINDS, SPLIT>::value / (TILE * 4);
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + K1Smem<KINDS>::stage);
   const int tid = threadIdx.x;
@@ -947,10 +973,10 @@ __global__ void __launch_bounds__(WENO_K1_TILE * 4, K1Blocks<KINDS, CHAR>::value
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     bool ok;
     if (quads(tile)) {
-      if constexpr (CHAR) ok = tile_points_char<12, 8, WALLS>(smem, bar, phase, tq, tile);
+      if constexpr (CHAR) ok = tile_points_char<12, 8, PARTS, WALLS>(smem, bar, phase, tq, tile);
       else ok = tile_points<12, 8, WALLS>(smem, bar, phase, tq, tile);
     } else {
-      if constexpr (CHAR) ok = tile_points_char<9, 6, WALLS>(smem, bar, phase, tt, tile - nq);
+      if constexpr (CHAR) ok = tile_points_char<9, 6, PARTS, WALLS>(smem, bar, phase, tt, tile - nq);
       else ok = tile_points<9, 6, WALLS>(smem, bar, phase, tt, tile - nq);
     }
     if (!ok) {  // the whole block: tile_points agrees on it
@@ -996,10 +1022,6 @@ template <> struct FluxMath<float> {
   }
 };
 #endif
-
-// Products that the compiler may not merge into a following addition.
-__device__ __forceinline__ float mulr(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mulr(double a, double b) { return __dmul_rn(a, b); }
 
 // HLLC in the frame of the unit normal (nx, ny); returns the flux rotated back.  The side of the contact
 // is taken by selection, not by branches: a warp's faces rarely agree on one.  Every product is either

@@ -212,6 +212,15 @@ F64Grid f64_grid(const S& s, int64_t n, int nv, int M, int G, bool characteristi
 // launch and 151.1 in two, of 241k cells (63 % triangles) 211 and 219, of 1.0M cells 815 and 796.
 bool merge_kinds(const S& s) { return s.nQ + s.nT <= (int64_t)16 * 8 * kTile * s.nsm; }
 
+// Characteristic variables, FP32C: a set of threads for every face of a cell while the blocks, three or four
+// an SM with 256 or 192 threads, are all resident at once; above, the longer chain of a thread is hidden by
+// other blocks and the gathers are not repeated.  A step: 1,600 quads 30.9 -> 22.7 us, 6,400 quads 37.0 -> 30.9,
+// 6,370 mixed cells (2.6 tiles an SM) 37.0 -> 30.9, 8,192 triangles (3.4 an SM) 30.9 -> 28.9; but 8,320 mixed
+// cells (3.4) equal and 10,000 triangles (4.1) 35.2 -> 39.1.
+bool split_faces(const S& s) {
+  return (s.nQ + kTile - 1) / kTile + (s.nT + kTile - 1) / kTile <= (int64_t)3 * s.nsm;
+}
+
 // FP32C Euler reconstruction into wg.  which as below.
 template <int KINDS, bool CHAR, bool WALLS>
 void launch_tma_kinds(S& s, const Launch& l, const float* u, const float* ul, float* wg, cudaStream_t st) {
@@ -223,7 +232,16 @@ void launch_tma_kinds(S& s, const Launch& l, const float* u, const float* ul, fl
   t.first = s.nQ;
   t.gbase = 8 * s.nQ;
   const int64_t tiles = (KINDS & 1 ? (s.nQ + kTile - 1) / kTile : 0) + (KINDS & 2 ? (s.nT + kTile - 1) / kTile : 0);
-  launch(weno::dev::k_reconstruct_tma<KINDS, CHAR, WALLS>, tma_grid(l, tiles), kTile * 4, weno::dev::K1Smem<KINDS>::bytes, st, s.q_maps, s.t_maps, q, t, s.err, s.debug_stall);
+  auto run = [&](auto split) {
+    constexpr bool SPLIT = decltype(split)::value;
+    launch(weno::dev::k_reconstruct_tma<KINDS, CHAR, WALLS, SPLIT>, SPLIT ? (unsigned)tiles : tma_grid(l, tiles),
+           weno::dev::K1Threads<KINDS, SPLIT>::value, weno::dev::K1Smem<KINDS>::bytes, st, s.q_maps, s.t_maps, q, t, s.err,
+           s.debug_stall);
+  };
+  if constexpr (CHAR) {
+    if (split_faces(s)) return run(std::true_type{});
+  }
+  run(std::false_type{});
 }
 template <bool CHAR, bool WALLS>
 void launch_tma(S& s, const void* U, const void* Ulo, void* wg, cudaStream_t st, int which) {

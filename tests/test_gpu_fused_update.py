@@ -1,4 +1,4 @@
-"""FP32C Euler update: one fused kernel on small meshes, face and gather kernels on large ones."""
+"""FP32C Euler kernels of small meshes against those of large ones: the fused update, faces split over threads."""
 import numpy as np
 import pytest
 
@@ -41,3 +41,30 @@ def test_mesh_alone_and_in_a_large_batch_give_the_same_bits(kind, n):
         cells = slice(k * mi.n_cells, (k + 1) * mi.n_cells)
         assert np.array_equal(Rb[:, cells], R)
         assert np.array_equal(b[:, cells], a)
+
+
+# characteristic variables on a mesh whose blocks have a set of threads for every face (few tiles for every
+# SM), with indicators inside and outside the FP32 range; the last tile of a type is partly filled
+@pytest.mark.parametrize("flow", ["wave", "ramp"])
+@pytest.mark.parametrize("kind,n", [("quad", 9), ("tri", 5), ("mixed", 13)])
+def test_faces_split_over_threads_give_the_same_bits(kind, n, flow):
+    """In a large batch a thread walks all faces of its cell; the arithmetic of a Gauss point is the same."""
+    def ramp(x, y):
+        rho = 1.0 + 1e7 * (x + 0.3 * y)
+        one = np.ones_like(rho)
+        return S.euler_prim_to_cons(rho, one, 0.5 * one, rho, 1.4)
+
+    mi = S.mesh_for_config(3, n=n, seed=7, kind=kind)
+    mi.walls = (0, 3)
+    mesh = Mesh.from_input(mi)
+    W = S.cell_average(mi, S.density_wave if flow == "wave" else ramp)
+    prm = dict(eqn="euler", precision="fp32c", characteristic=True)
+    one = Solver(mesh, **prm)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    copies = 16 * 8 * sms // mi.n_cells + 1  # more than eight tiles of 16 cells for every SM
+    big = Solver(Mesh.concat([mesh] * copies), **prm)
+    U, Ul = one.to_device(W)
+    V, Vl = big.to_device(np.tile(W, (1, copies)))
+    R, Rb = one.to_host(one.residual(U, Ul)), big.to_host(big.residual(V, Vl))
+    for k in (0, copies - 1):
+        assert np.array_equal(Rb[:, k * mi.n_cells:(k + 1) * mi.n_cells], R, equal_nan=True)
