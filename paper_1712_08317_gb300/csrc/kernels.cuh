@@ -460,6 +460,17 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
+// The same; the lines are the first to leave L2.
+__device__ __forceinline__ void tma_load_2d_once(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+  uint64_t policy;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], "
+      "[%4], %5;" ::"r"(smem_addr(dst)),
+      "l"((uint64_t)map), "r"(x), "r"(y), "r"(smem_addr(bar)), "l"(policy)
+      : "memory");
+}
+
 #ifndef WENO_K1_TILE
 #define WENO_K1_TILE 16  // cells per block tile of the TMA reconstruction (8, 16, 32 or 64)
 #endif
@@ -606,15 +617,22 @@ struct TileCells {
   int linear;
 };
 
-// Copies of a tile's tables into shared memory, completing on the barrier.
+// Copies of a tile's tables into shared memory, completing on the barrier.  A pass reads each table once:
+// with `once` they leave L2 before what the kernels of a stage hand to one another (see tables_once).
 template <int M, int G>
-__device__ __forceinline__ void load_tile(unsigned char* smem, const TileMaps* maps, int64_t tile, uint64_t* bar) {
+__device__ __forceinline__ void load_tile(unsigned char* smem, const TileMaps* maps, int64_t tile, uint64_t* bar, int once) {
   using L = PairTile<M, G>;
   const int x = (int)(tile * L::TILE * 4);
   mbar_expect_tx(bar, L::STAGE);
-  tma_load_2d(smem, &maps->gam, x, 0, bar);
-  tma_load_2d(smem + L::GAM, &maps->dg, x, 0, bar);
-  tma_load_2d(smem + L::GAM + L::DG, &maps->gop, x, 0, bar);
+  if (once) {
+    tma_load_2d_once(smem, &maps->gam, x, 0, bar);
+    tma_load_2d_once(smem + L::GAM, &maps->dg, x, 0, bar);
+    tma_load_2d_once(smem + L::GAM + L::DG, &maps->gop, x, 0, bar);
+  } else {
+    tma_load_2d(smem, &maps->gam, x, 0, bar);
+    tma_load_2d(smem + L::GAM, &maps->dg, x, 0, bar);
+    tma_load_2d(smem + L::GAM + L::DG, &maps->gop, x, 0, bar);
+  }
 }
 
 // The cells whose sums of alpha left the FP32 range are redone with FP64 weights within the pass, each by
@@ -950,7 +968,7 @@ template <int KINDS> struct K1Smem {
 template <int KINDS, bool CHAR, bool WALLS, bool SPLIT>
 __global__ void __launch_bounds__(K1Threads<KINDS, SPLIT>::value, K1Blocks<KINDS, CHAR, SPLIT>::value) k_reconstruct_tma(
     const __grid_constant__ TileMaps mq, const __grid_constant__ TileMaps mt, const __grid_constant__ TileCells tq,
-    const __grid_constant__ TileCells tt, int* __restrict__ err, int stall) {
+    const __grid_constant__ TileCells tt, int* __restrict__ err, int stall, int once) {
   constexpr int TILE = WENO_K1_TILE, PARTS = K1Threads<KINDS, SPLIT>::value / (TILE * 4);
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + K1Smem<KINDS>::stage);
@@ -964,8 +982,8 @@ __global__ void __launch_bounds__(K1Threads<KINDS, SPLIT>::value, K1Blocks<KINDS
   __syncthreads();
   auto quads = [&](int64_t tile) { return KINDS == 1 || (KINDS == 3 && tile < nq); };
   auto issue = [&](int64_t tile) {
-    if (quads(tile)) load_tile<12, 8>(smem, &mq, tile, bar);
-    else load_tile<9, 6>(smem, &mt, tile - nq, bar);
+    if (quads(tile)) load_tile<12, 8>(smem, &mq, tile, bar, once);
+    else load_tile<9, 6>(smem, &mt, tile - nq, bar, once);
   };
   if (tid == 0 && blockIdx.x < ntiles) issue(blockIdx.x);
   kernel_wait();
