@@ -93,6 +93,25 @@ __device__ __forceinline__ PosNum pos_of(double x) {
   const uint32_t h = hi_word(x), l = (uint32_t)__double2loint(x);
   return PosNum{(uint64_t)(0x80000000u | __funnelshift_l(l, h, 11)) << 32 | (l << 11), (int)(h >> 20)};
 }
+// The same number in one word, for tables and shared memory: t, whose low 11 bits are zero, with the biased
+// exponent in them.  Two instructions unpack it where pos_of takes four:
+// of about 110 integer instructions a point and candidate, ten.  33k-cell vortex step 584.8 -> 575.7 us, 53k-cell
+// residual 293.6 -> 290.1, 8k-quad CFL step 245.1 -> 241.5; in characteristic variables, where no thread shares
+// its indicators, 434.1 -> 437.4: it keeps FP64 weights.
+struct PosWord { uint64_t bits; };
+__device__ __forceinline__ PosWord pos_word(double x) {
+  const uint64_t u = (uint64_t)__double_as_longlong(x);
+  return PosWord{1ull << 63 | u << 11 | (u >> 52 & 0x7ffu)};
+}
+__device__ __forceinline__ PosNum pos_of(PosWord w) { return PosNum{w.bits & ~0x7ffull, (int)(w.bits & 0x7ffu)}; }
+__device__ __forceinline__ double f64_of(PosWord w) {
+  return __longlong_as_double((long long)((w.bits & 0x7ffu) << 52 | (w.bits << 1) >> 12));
+}
+__device__ __forceinline__ double f64_of(double x) { return x; }
+struct PosPair { PosWord x, y; };  // (gamma+, gamma-)
+// A candidate with its indicators in that form.
+struct CandPos { double gx, gy; PosWord be, b2, b3; };
+
 __device__ __forceinline__ PosNum pos_mul(PosNum a, PosNum b) {
   const uint32_t ah = (uint32_t)(a.t >> 32), al = (uint32_t)a.t, bh = (uint32_t)(b.t >> 32), bl = (uint32_t)b.t;
   return PosNum{(uint64_t)ah * bh + __umulhi(ah, bl) + __umulhi(al, bh), a.e + b.e - 1022};
@@ -155,7 +174,7 @@ __device__ __forceinline__ double pos_rcp(PosNum s) {
 }
 
 // Increments R(x_G) - W0 at PTS Gauss points of one face (Section 3.4), from the candidates cand(j) and
-// the split weights wt(h, j) = (gamma+, gamma-) of point h:
+// the split weights wt(h, j) = (gamma+, gamma-) of point h (indicators and weights as FP64 or as PosWord):
 //   alpha+- = gamma+- / (beta~+- + eps)^2,  beta~+- + eps = (beta + eps) + gamma (beta^2 + gamma beta^3),
 //   R - W0 = sigma+ sum alpha+ p / sum alpha+  -  sigma- sum alpha- p / sum alpha-.
 // Only p and the sums of alpha p are FP64, 4 instructions per point and candidate.  Returns false if an
@@ -166,7 +185,7 @@ __device__ __forceinline__ bool face_points_f64(Cand cand, Weights wt, const dou
   PosNum Ap[PTS], Am[PTS];
   double Bp[PTS], Bm[PTS];
   int lo = kAlphaExpMax, hi = 0;
-  auto weight = [&](double g, PosNum be, PosNum b2, PosNum b3) {
+  auto weight = [&](auto g, PosNum be, PosNum b2, PosNum b3) {
     const PosNum gamma = pos_of(g);
     int e;
     const PosNum a = pos_alpha(gamma, pos_sum(be, pos_mul(gamma, pos_sum(b2, pos_mul(gamma, b3)))), e);
@@ -175,11 +194,11 @@ __device__ __forceinline__ bool face_points_f64(Cand cand, Weights wt, const dou
     return a;
   };
   auto one = [&](int j, bool first) {
-    const CandF64 c = cand(j);
+    const auto c = cand(j);
     const PosNum be = pos_of(c.be), b2 = pos_of(c.b2), b3 = pos_of(c.b3);
 #pragma unroll
     for (int h = 0; h < PTS; ++h) {
-      const double2 g = wt(h, j);
+      const auto g = wt(h, j);
       const double p = c.gx * dx[h] + c.gy * dy[h];
       const PosNum ap = weight(g.x, be, b2, b3), an = weight(g.y, be, b2, b3);
       const double vp = pos_to_f64(ap.t, ap.e), vn = pos_to_f64(an.t, an.e);
@@ -207,8 +226,9 @@ __device__ __forceinline__ void face_points_ieee(Cand cand, Weights wt, const do
     double Ap = 0.0, Bp = 0.0, Am = 0.0, Bm = 0.0;
 #pragma unroll 1
     for (int j = 0; j < M; ++j) {
-      const CandF64 c = cand(j);
-      const double2 g = wt(h, j);
+      const auto c = cand(j);
+      const auto w = wt(h, j);
+      const double2 g = make_double2(f64_of(w.x), f64_of(w.y));
       const double p = c.gx * dx[h] + c.gy * dy[h], b = a0 * (c.gx * c.gx + c.gy * c.gy);
       const double qp = g.x * b, qn = g.y * b;
       const double dp = b * (1.0 + qp + qp * qp) + eps, dn = b * (1.0 + qn + qn * qn) + eps;

@@ -25,10 +25,13 @@ namespace dev {
 
 // Split linear weights of a group from its linear weights gam [g][j][q] (Section 3.4):
 // gt+ = (gamma + theta |gamma|) / 2, gt- = gt+ - gamma, sigma+- = sum gt+-, gamma+- = gt+- / sigma+-.
-// wt [g][j][q] = (gamma+, gamma-) and sig [g][q] = (sigma+, sigma-), rows of `pitch` cells.
-template <int M>
+// wt [g][j][q] = (gamma+, gamma-) and sig [g][q] = (sigma+, sigma-), rows of `pitch` cells; wt as PosPair for
+// the component-wise kernel (W = PosPair), as double2 in characteristic variables.
+__device__ __forceinline__ void put(PosPair* p, double x, double y) { *p = PosPair{pos_word(x), pos_word(y)}; }
+__device__ __forceinline__ void put(double2* p, double x, double y) { *p = make_double2(x, y); }
+template <int M, typename W>
 __global__ void k_split_weights(const double* __restrict__ gam, int64_t N, int G, double theta, int64_t pitch,
-                                double2* __restrict__ wt, double2* __restrict__ sig) {
+                                W* __restrict__ wt, double2* __restrict__ sig) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N * G) return;
   const int64_t g = t / N, q = t - g * N;
@@ -44,7 +47,12 @@ __global__ void k_split_weights(const double* __restrict__ gam, int64_t N, int G
   sig[g * pitch + q] = make_double2(sp, sm);
   const double isp = 1.0 / sp, ism = 1.0 / sm;
 #pragma unroll
-  for (int j = 0; j < M; ++j) wt[(g * M + j) * pitch + q] = make_double2(tp[j] * isp, tm[j] * ism);
+  for (int j = 0; j < M; ++j) put(wt + (g * M + j) * pitch + q, tp[j] * isp, tm[j] * ism);
+}
+
+__device__ __forceinline__ PosPair pos_pair(const PosPair* p) {
+  const ulonglong2 w = __ldg(reinterpret_cast<const ulonglong2*>(p));
+  return PosPair{{w.x}, {w.y}};
 }
 
 // Layout of a block of either kernel: `width` = cells x variables of its tile; thread t holds column
@@ -60,14 +68,15 @@ constexpr int kF64MaxWidth = 32;
 template <int NV, int M, int G, bool WALLS>
 __global__ void __launch_bounds__(kF64MaxWidth * G) k_reconstruct_f64(
     const double* U, const int32_t* __restrict__ slot, const double* __restrict__ gop,
-    const double* __restrict__ dg, const double* __restrict__ gam, const double2* __restrict__ wt,
+    const double* __restrict__ dg, const double* __restrict__ gam, const PosPair* __restrict__ wt,
     const double2* __restrict__ sigma, const double* __restrict__ area, int64_t N, int64_t pitch, int64_t first,
     int64_t gbase, double* Wg, double eps, int linear, int width) {
   constexpr int PER = (M + G - 1) / G;
   extern __shared__ double sm[];
   double* dW = sm;                                      // [slot - 1][column]
   double *gx = sm + M * width, *gy = gx + M * width;    // [candidate][column]
-  double *be = gy + M * width, *b2 = be + M * width, *b3 = b2 + M * width;
+  PosWord* be = reinterpret_cast<PosWord*>(gy + M * width);
+  PosWord *b2 = be + M * width, *b3 = b2 + M * width;
   const int col = threadIdx.x % width, g = threadIdx.x / width, v = col % NV;
   const int64_t qr = (int64_t)blockIdx.x * (width / NV) + col / NV;
   const int64_t q = qr < N ? qr : N - 1;  // columns past the end work on the last cell and store nothing
@@ -92,7 +101,8 @@ __global__ void __launch_bounds__(kF64MaxWidth * G) k_reconstruct_f64(
     const CandF64 cd =
         candidate_f64(__ldg(o) * da + __ldg(o + N) * db, __ldg(o + 2 * N) * da + __ldg(o + 3 * N) * db, a0, eps);
     const int k = j * width + col;
-    gx[k] = cd.gx; gy[k] = cd.gy; be[k] = cd.be; b2[k] = cd.b2; b3[k] = cd.b3;
+    gx[k] = cd.gx; gy[k] = cd.gy;
+    be[k] = pos_word(cd.be); b2[k] = pos_word(cd.b2); b3[k] = pos_word(cd.b3);
   }
   __syncthreads();
   const double dx = __ldg(dg + (int64_t)(2 * g) * N + q), dy = __ldg(dg + (int64_t)(2 * g + 1) * N + q);
@@ -105,11 +115,11 @@ __global__ void __launch_bounds__(kF64MaxWidth * G) k_reconstruct_f64(
   } else {
     auto cand = [&](int j) {
       const int k = j * width + col;
-      return CandF64{gx[k], gy[k], be[k], b2[k], b3[k]};
+      return CandPos{gx[k], gy[k], be[k], b2[k], b3[k]};
     };
-    const double2* w = wt + (int64_t)(g * M) * pitch + q;
+    const PosPair* w = wt + (int64_t)(g * M) * pitch + q;
     const double2 sig = __ldg(sigma + (int64_t)g * pitch + q);
-    auto weights = [&](int, int j) { return __ldg(w + j * pitch); };
+    auto weights = [&](int, int j) { return pos_pair(w + j * pitch); };
     if (!face_points_f64<M, 1>(cand, weights, &dx, &dy, &sig, &incr))
       face_points_ieee<M, 1>(cand, weights, &dx, &dy, &sig, a0, eps, &incr);
   }

@@ -116,7 +116,8 @@ struct weno_solver_s {
   void *q_gop = nullptr, *q_dg = nullptr, *q_gam = nullptr, *t_gop = nullptr, *t_dg = nullptr, *t_gam = nullptr;
   void *q_gam1 = nullptr, *t_gam1 = nullptr;
   void *q_pgam = nullptr, *q_pdg = nullptr, *t_pgam = nullptr, *t_pdg = nullptr;  // point-pair tables (Euler FP32C)
-  double2 *q_wt = nullptr, *q_sig = nullptr, *t_wt = nullptr, *t_sig = nullptr;   // FP64 split weights
+  void *q_wt = nullptr, *t_wt = nullptr;        // FP64 split weights: PosPair, in characteristic variables double2,
+  double2 *q_sig = nullptr, *t_sig = nullptr;   // and their sums
   int64_t q_pitch = 0, t_pitch = 0;  // row pitch (cells) of the packed FP32C tables and the FP64 split weights
   bool tma = false;                   // Euler FP32C: reconstruction with TMA-staged tables
   weno::dev::TileMaps q_maps{}, t_maps{};  // point-pair tables and gradient operators (FP32C Euler)
@@ -605,7 +606,7 @@ int upload_pairs(S& s, const GroupTables& T, int64_t P, double theta, void** gam
 // FP64 tables of the linear weights: gam itself for the linear scheme, otherwise the split weights,
 // formed on the device from a temporary copy of gam.
 template <int M>
-int upload_split(S& s, const GroupTables& T, int64_t pitch, void** gam, double2** wt, double2** sig, cudaStream_t st) {
+int upload_split(S& s, const GroupTables& T, int64_t pitch, void** gam, void** wt, double2** sig, cudaStream_t st) {
   if (s.prm.linear) return upload_real(s, gam, T.gam, st);
   int r;
   if ((r = s.alloc(wt, sizeof(double2) * (size_t)T.G * M * pitch))) return r;
@@ -616,8 +617,11 @@ int upload_split(S& s, const GroupTables& T, int64_t pitch, void** gam, double2*
   if (e != cudaSuccess) return fail(WENO_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   e = cudaMemcpyAsync(tmp, T.gam.data(), T.gam.size() * sizeof(double), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
-    weno::dev::k_split_weights<M><<<(unsigned)((T.N * T.G + 127) / 128), 128, 0, st>>>(tmp, T.N, T.G, s.prm.theta, pitch,
-                                                                                       *wt, *sig);
+    const unsigned blocks = (unsigned)((T.N * T.G + 127) / 128);
+    if (s.prm.characteristic)
+      weno::dev::k_split_weights<M><<<blocks, 128, 0, st>>>(tmp, T.N, T.G, s.prm.theta, pitch, (double2*)*wt, *sig);
+    else
+      weno::dev::k_split_weights<M><<<blocks, 128, 0, st>>>(tmp, T.N, T.G, s.prm.theta, pitch, (weno::dev::PosPair*)*wt, *sig);
     e = cudaGetLastError();
   }
   const cudaError_t es = cudaStreamSynchronize(st);
