@@ -52,6 +52,7 @@ __device__ __forceinline__ double sqrt_f64(double x) {
 // Guarded forms: IEEE outside the range the iterations are valid in.
 __device__ __noinline__ double rcp_ieee(double x) { return 1.0 / x; }
 __device__ __noinline__ double sqrt_ieee(double x) { return sqrt(x); }
+__device__ __noinline__ double quotient_ieee(double a, double b) { return a / b; }
 __device__ __noinline__ double rsqrt_ieee(double x) { return 1.0 / sqrt(x); }
 __device__ __forceinline__ double rcp_any(double x) {
   const uint32_t h = hi_word(x) & 0x7fffffffu;

@@ -1416,7 +1416,7 @@ __global__ void __launch_bounds__(256) k_update_f32c(
 // Largest stable step min 2|Omega| / sum_p (|v.n_p| + c)|l_p| and integrals sum |Omega| (U + U_lo) of each
 // instance, in FP64 and in two levels over a fixed partition (`chunks`), so that results do not depend on
 // scheduling.  What bounds them is the FP64 pipe (2 lanes a clock and SM) and, on small meshes, latency:
-// the time step is formed and reduced in one kernel with the reciprocals and roots of arith_f64.cuh (39
+// the time step is formed and reduced in one kernel with the reciprocals and roots of arith_f64.cuh (48
 // FP64 instructions a quad, not about 110 with IEEE division), FP32 states are widened on the integer
 // pipe, minima are taken on the bits of the numbers, and a chunk is as many cells as spread a mesh over
 // all SMs.
@@ -1442,6 +1442,14 @@ __device__ __forceinline__ void state_f64(const T* __restrict__ U, const T* __re
   for (int v = 0; v < NV; ++v) w[v] = COMP ? widen(h[v]) + widen(l[v]) : widen(h[v]);
 }
 
+// a / b from r = rcp_any(b), corrected with the remainder to the rounded quotient (but for near ties), so that
+// a step is as close to the exact one as with IEEE division.
+__device__ __forceinline__ double quotient(double a, double b, double r) {
+  const uint32_t h = hi_word(b) & 0x7fffffffu;
+  const double q = a * r;
+  if (!rcp_safe(h, h) || (hi_word(q) & 0x7fffffffu) >= 0x7ff00000u) return quotient_ieee(a, b);
+  return fma(fma(-q, b, a), r, q);
+}
 // Half of a cell's stable step, |Omega| / sum_p (|v.n_p| + c)|l_p|; never negative, NaN for a negative pressure.
 template <int NV, int NFACE>
 __device__ __forceinline__ double half_dt(const double w[NV], const int32_t* __restrict__ cf, int64_t row,
@@ -1451,10 +1459,10 @@ __device__ __forceinline__ double half_dt(const double w[NV], const int32_t* __r
   double u = ax, vv = ay, snd = 0.0;
   if constexpr (NV == 4) {
     const double r = rcp_any(w[0]);
-    u = w[1] * r;
-    vv = w[2] * r;
-    const double p = (gas_gamma - 1.0) * (w[3] - 0.5 * (w[1] * u + w[2] * vv));
-    snd = sqrt_any(gas_gamma * p * r);
+    u = quotient(w[1], w[0], r);
+    vv = quotient(w[2], w[0], r);
+    const double p = (gas_gamma - 1.0) * (w[3] - 0.5 * w[0] * (u * u + vv * vv));
+    snd = sqrt_any(quotient(gas_gamma * p, w[0], r));
   }
   double s = 0.0;
 #pragma unroll
@@ -1463,7 +1471,7 @@ __device__ __forceinline__ double half_dt(const double w[NV], const int32_t* __r
     const int64_t f = e >= 0 ? e : ~e;
     s += (fabs(u * __ldg(fnx + f) + vv * __ldg(fny + f)) + snd) * __ldg(flen + f);
   }
-  return area * rcp_any(s);
+  return quotient(area, s, rcp_any(s));
 }
 
 // Smaller of two numbers that are >= 0 or NaN, by their bits: a NaN of either sign is above every number,
