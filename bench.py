@@ -30,7 +30,7 @@ METRIC = "WENO3 cell-updates/s (×RK stages) on 1 GB300, FP32+batched vs FP64 at
 UNIT = "cell-updates/s"
 FALLBACK_HBM_GBS = 6800.0
 # DRAM bytes per cell of one reconstruction launch: ncu dram__bytes_read.sum + dram__bytes_write.sum of
-# k_reconstruct_tma and of k_reconstruct_char_tma (each pass with its FP64 fix-up launch) on the
+# k_reconstruct_tma, component-wise and in characteristic variables, on the
 # 637k-cell mesh of the benchmark family (n = 700), divided by its cells of each type.  They describe
 # the kernel source they were captured on (SHA-256 of csrc/kernels.cuh); for any other source the
 # bench line reports traffic null.
@@ -407,13 +407,13 @@ def k1_rcp(nQ, nT, nv=4):
 
 
 def k1_ops_fp64(nQ, nT, nv=4):
-    """Algorithmic FP64 operations (an FMA or a division counts one) of one FP64 reconstruction pass,
-    which splits the linear weights at every Gauss point: per (cell, variable) 1 per stencil slot and
-    8 per candidate; per Gauss point and candidate 4 (split sums) + 25 (split weights 5, P^1_j(x_G) -
-    W0 2, per sign q, beta~ + eps (3), its square, alpha = gamma / square, sums 2: 9); per Gauss
-    point 6 (two reciprocals of sigma, the combination)."""
+    """Instructions of the FP64 pipe (an FMA counts one) of one FP64 reconstruction pass: per (cell, variable)
+    1 per stencil slot and 10 per candidate (gradient 4, beta 3, beta + eps, beta^2, beta^3); per Gauss point
+    and candidate 4 (P^1_j(x_G) - W0: 2; per sign sum alpha p); per Gauss point 5 for the combination.  The
+    indicators, the weights and their sums are formed on the integer pipe and are not counted; the splitting
+    is done once per solver."""
     def per(M, G):
-        return nv * (9 * M + G * (29 * M + 6))
+        return nv * (11 * M + G * (4 * M + 5))
     return nQ * per(12, 8) + nT * per(9, 6)
 
 
@@ -1131,9 +1131,12 @@ def main():
                                                     for n in (20, 40, 80, args.acc_n)], precs),
                   "vortex_lowq": ladder_orders([ladder_point("vortex-lowq", n, precs) for n in (40, 80, 160)], precs)}
 
-    # k_fill of dt, the three stages (per cell type the reconstruction, its fix-up pass and the
-    # gather; the face kernel), k_advance_time
-    launches_per_step = 2 + 3 * (3 * (1 if nQ else 0) + 3 * (1 if nT else 0) + 1)
+    # k_set_dt, the three stages, k_advance_time.  A stage: the reconstruction (one launch for both cell
+    # types up to 16 rounds of eight 16-cell tiles an SM), then the fluxes and the gather, in one kernel
+    # while four lanes a cell fit 1,024 threads an SM
+    sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+    k1_launches = 2 if nQ and nT and N > 16 * 8 * 16 * sms else 1
+    launches_per_step = 2 + 3 * (k1_launches + (1 if 4 * N <= 1024 * sms else 2))
     launch_cfg = sol.launch_config().tolist()
     del sol64, V
     batched = None
@@ -1177,9 +1180,9 @@ def main():
             "kernel_ms": {"reconstruct": k_ms, "face": face_ms, "gather": gather_ms},
             "fp64": {"value": fp64_value, "unit": UNIT, "steps": fp64_steps, "ms_per_step": fp64_ms / fp64_steps,
                      "fp32c_over_fp64": value / fp64_value,
-                     "roofline": {"kernel": "k_reconstruct<double> (quad + triangle launches of one pass)",
+                     "roofline": {"kernel": "k_reconstruct_f64 (quad + triangle launches of one pass)",
                                   "bound": "alu", "achieved": k64_ops / (k64_ms / 1e3) / 1e12,
-                                  "peak": peaks["dfma"], "unit": "Top/s (FP64 ops, FMA or division = 1)",
+                                  "peak": peaks["dfma"], "unit": "Top/s (instructions of the FP64 pipe, FMA = 1)",
                                   "frac": k64_ops / (k64_ms / 1e3) / 1e12 / peaks["dfma"],
                                   "algorithmic_ops_per_launch": k64_ops, "ms_per_launch": k64_ms}},
             "batched": batched,
