@@ -14,7 +14,7 @@
 // by every variable, 5,350 FP64 issue slots a (cell, variable) of quads; then: as here with all of the
 // weights in FP64, 2,140 slots; then: gamma / d^2 on the integer pipe, 1,200; their sums too, 940; now: the
 // indicators d too, 560): 17,920 Euler quads 662 -> 277 -> 154 -> 124 -> 103 us, 15,360 triangles
-// 384 -> 144 -> 83 -> 68 -> 57 us, 1,600 scalar quads 332 -> 30 us and now 18.  The FP64 pipe is 66 % and the
+// 384 -> 144 -> 83 -> 68 -> 57 us, 1,600 scalar quads 332 -> 30 us and now 17.  The FP64 pipe is 66 % and the
 // integer pipe 62 % busy: the two now balance, and what is left is how well they overlap.
 #pragma once
 
@@ -62,7 +62,7 @@ constexpr int kF64MaxWidth = 32;
 
 // Component-wise FP64 K1.  The threads of a column share out its M stencil differences, then its M
 // candidates, both into shared memory; then each evaluates its Gauss point.  A thread a point: no FP64
-// instruction is repeated (a warp takes whole shares of the candidates), 62 registers leave 30 warps an
+// instruction is repeated (a warp takes whole shares of the candidates), 64 registers leave 30 warps an
 // SM, and the last wave is short (with both points of a face in a thread, 96 registers and 16 to 19
 // warps: triangles 79 us a pass on the mesh above against 68, quads 124 either way).
 template <int NV, int M, int G, bool WALLS>
