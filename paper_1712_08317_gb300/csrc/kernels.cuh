@@ -688,8 +688,9 @@ __device__ __noinline__ void fix_cell(const unsigned char* smem, const TileCells
 
 // Calls fix(q, cell of the tile) for each cell of the tile with a lane that has `bad` set, on the warp of the
 // first TILE x 4 threads that holds it: lanes 4i..4i+3 of warp w hold cell 8w + i of the tile.  With PARTS > 1
-// the block has that many warps for every such cell, which agree on it first: none of the cell's regular
-// values is then still to be stored.
+// the block has that many warps for every such cell, which agree on it first.  The redone values go to the
+// addresses of the cell's regular ones and are stored by other lanes; the barriers (a vote orders no memory)
+// put them after those.
 template <int PARTS, typename Fix>
 __device__ __forceinline__ void fix_marked(bool bad, int64_t q0, Fix fix) {
   constexpr int WARPS = WENO_K1_TILE / 8;
@@ -703,6 +704,7 @@ __device__ __forceinline__ void fix_marked(bool bad, int64_t q0, Fix fix) {
     if (w >= WARPS) return;
     for (int i = 1; i < PARTS; ++i) m |= marks[w + i * WARPS];
   }
+  if (m) __syncwarp();
   while (m) {
     const int i = (__ffs(m) - 1) >> 2;
     m &= ~(0xfu << (4 * i));
