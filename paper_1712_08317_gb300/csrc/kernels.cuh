@@ -1434,12 +1434,27 @@ __device__ __forceinline__ double widen(float x) {
 }
 __device__ __forceinline__ double widen(double x) { return x; }
 
-// The state of cell c in FP64.
+// Whether the cells of a state start on 16-byte boundaries, as load_vec needs it.  The reductions take a state
+// that starts at any element of a buffer.
+template <typename T, bool COMP>
+__device__ __forceinline__ bool vec_aligned(const T* U, const T* Ulo) {
+  return ((reinterpret_cast<uintptr_t>(U) | (COMP ? reinterpret_cast<uintptr_t>(Ulo) : 0)) & 15) == 0;
+}
+
+// The state of cell c in FP64; vec as vec_aligned (the same for all cells of a launch).
 template <typename T, int NV, bool COMP>
-__device__ __forceinline__ void state_f64(const T* __restrict__ U, const T* __restrict__ Ulo, int64_t c, double w[NV]) {
+__device__ __forceinline__ void state_f64(const T* __restrict__ U, const T* __restrict__ Ulo, int64_t c, bool vec, double w[NV]) {
   T h[NV], l[NV];
-  load_vec<T, NV>(U + c * NV, h);
-  if (COMP) load_vec<T, NV>(Ulo + c * NV, l);
+  if (NV == 1 || vec) {
+    load_vec<T, NV>(U + c * NV, h);
+    if (COMP) load_vec<T, NV>(Ulo + c * NV, l);
+  } else {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      h[v] = U[c * NV + v];
+      if (COMP) l[v] = Ulo[c * NV + v];
+    }
+  }
 #pragma unroll
   for (int v = 0; v < NV; ++v) w[v] = COMP ? widen(h[v]) + widen(l[v]) : widen(h[v]);
 }
@@ -1500,10 +1515,11 @@ __global__ void __launch_bounds__(256) k_chunk_dt(
     int64_t nT, double gas_gamma, double ax, double ay, double* __restrict__ partial) {
   kernel_begin();
   const int64_t c0 = __ldg(chunks + 2 * blockIdx.x), c1 = __ldg(chunks + 2 * blockIdx.x + 1);
+  const bool vec = vec_aligned<T, COMP>(U, Ulo);
   uint64_t m = bits_of(kNoDt);
   for (int64_t c = c0 + threadIdx.x; c < c1; c += 256) {
     double w[NV];
-    state_f64<T, NV, COMP>(U, Ulo, c, w);
+    state_f64<T, NV, COMP>(U, Ulo, c, vec, w);
     const double a = __ldg(area + c);
     const double h = c < nQ ? half_dt<NV, 4>(w, qcf + c, nQ, fnx, fny, flen, a, gas_gamma, ax, ay)
                             : half_dt<NV, 3>(w, tcf + (c - nQ), nT, fnx, fny, flen, a, gas_gamma, ax, ay);
@@ -1533,12 +1549,13 @@ __global__ void __launch_bounds__(256) k_chunk_sum(const T* __restrict__ U, cons
                                                    const int64_t* __restrict__ chunks, double* __restrict__ partial) {
   kernel_begin();
   const int64_t c0 = __ldg(chunks + 2 * blockIdx.x), c1 = __ldg(chunks + 2 * blockIdx.x + 1);
+  const bool vec = vec_aligned<T, COMP>(U, Ulo);
   double acc[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) acc[v] = 0.0;
   for (int64_t c = c0 + threadIdx.x; c < c1; c += 256) {
     double w[NV];
-    state_f64<T, NV, COMP>(U, Ulo, c, w);
+    state_f64<T, NV, COMP>(U, Ulo, c, vec, w);
     const double a = __ldg(area + c);
 #pragma unroll
     for (int v = 0; v < NV; ++v) acc[v] += a * w[v];
