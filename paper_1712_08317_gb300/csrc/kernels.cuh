@@ -1182,11 +1182,10 @@ __global__ void __launch_bounds__(256) k_face_f32(
   }
 }
 
-// The time steps of the next step: dt[i] = src[i], or v for every instance (src == nullptr), and for the
+// The time steps of the next step: dt[i] = src[i] (src may be dt), or v for every instance (src == nullptr), and for the
 // FP32C stages split[i] = (hi, lo) with hi + lo ~ dt[i] to 2^-48 (split once here: every cell would spend
 // FP64 instructions on it).
-__global__ void k_set_dt(double* __restrict__ dt, float2* __restrict__ split, const double* __restrict__ src, double v,
-                         int n) {
+__global__ void k_set_dt(double* dt, float2* __restrict__ split, const double* src, double v, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double d = src ? src[i] : v;

@@ -1284,8 +1284,23 @@ int capture_step(S& s, void* U, void* Ulo) {
   return WENO_OK;
 }
 
+// Whether k_set_dt may read p itself: doubles in the memory of the solver's device.  A copy also reaches another
+// device's memory and starts at any byte.
+bool readable_here(const S& s, const double* p) {
+  cudaPointerAttributes a{};
+  if (reinterpret_cast<uintptr_t>(p) % alignof(double) || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();  // an error here is the copy's to report
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == s.dev;
+}
+
 // One step with the time steps dts[instance] (device), or dt for every instance.
 int run_step(S& s, void* U, void* Ulo, const double* dts, double dt, cudaStream_t st) {
+  if (dts && !readable_here(s, dts)) {
+    CK(cudaMemcpyAsync(s.dt_dev, dts, sizeof(double) * s.n_inst, cudaMemcpyDeviceToDevice, st));
+    dts = s.dt_dev;
+  }
   weno::dev::k_set_dt<<<(s.n_inst + 127) / 128, 128, 0, st>>>(s.dt_dev, s.dt_split, dts, dt, s.n_inst);
   int r = check_launch();
   if (r) return r;
