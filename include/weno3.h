@@ -268,6 +268,9 @@ int weno_check_instances(weno_solver_t s, int32_t* flags, void* cuda_stream);
  *           (Sections 3.1-3.4);
  *   pass 2: face fluxes from that scratch into the solver's flux scratch (Eqs. 5-6);
  *   pass 3: signed gather of the face fluxes into the solver's stage buffer (Eq. 4).
+ * On small FP32C Euler meshes (4 threads a cell fit 1,024 threads an SM) one
+ * kernel takes the Gauss-point scratch to the residual: there pass 2 launches
+ * nothing and pass 3 runs that kernel.
  * U / U_lo are used by pass 1 only.  Stream-ordered. */
 int weno_pass(weno_solver_t s, int32_t pass, const void* U, const void* U_lo, void* cuda_stream);
 

@@ -416,14 +416,16 @@ void launch_update(S& s, int mode, double c, const void* wg, void* fl, void* U, 
   launch_gather<T, NV, COMP>(s, mode, fl, U, Ulo, R, st);
 }
 
-// The passes after the reconstruction on their own (weno_pass, weno_autotune).
+// The passes after the reconstruction on their own (weno_pass, weno_autotune), in the kernels that launch_update
+// takes: where one does both passes, it is pass 3.
 template <typename T, int NV, bool COMP>
 void launch_pass2(S& s, cudaStream_t st) {
-  launch_face<T, NV>(s, s.Wg, s.F, 0.0, st);
+  if (!s.fused) launch_face<T, NV>(s, s.Wg, s.F, 0.0, st);
 }
 template <typename T, int NV, bool COMP>
 void launch_pass3(S& s, cudaStream_t st) {
-  launch_gather<T, NV, COMP>(s, 0, s.F, nullptr, nullptr, s.Ws, st);
+  if (s.fused) launch_update<T, NV, COMP>(s, 0, 0.0, s.Wg, s.F, nullptr, nullptr, s.Ws, st);
+  else launch_gather<T, NV, COMP>(s, 0, s.F, nullptr, nullptr, s.Ws, st);
 }
 
 template <typename T, int NV, bool COMP>
