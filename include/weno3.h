@@ -274,13 +274,17 @@ int weno_check_instances(weno_solver_t s, int32_t* flags, void* cuda_stream);
  * U / U_lo are used by pass 1 only.  Stream-ordered. */
 int weno_pass(weno_solver_t s, int32_t pass, const void* U, const void* U_lo, void* cuda_stream);
 
-/* Times each kernel over a set of block sizes and grid sizes (cells per
- * thread) on this mesh and keeps the fastest; rebuilds the step graphs.
+/* Times each kernel of a residual over a set of block sizes and grid sizes
+ * (cells per thread) on this mesh and keeps the fastest; rebuilds the step
+ * graphs.  Kernels whose shape follows from the mesh are left as they are.
  * Does not modify U / U_lo.  Synchronising. */
 int weno_autotune(weno_solver_t s, const void* U, const void* U_lo, void* cuda_stream);
 
-/* Current launch configuration: cfg[6] = {cell block, cell grid, face block,
- * face grid, gather block, gather grid}. */
+/* Launch shapes of a residual's kernels: cfg[6] = {cell block, cell grid, face
+ * block, face grid, gather block, gather grid}; grid 0: as many blocks as the
+ * work takes.  Where quads and triangles take launches of their own, the cell
+ * entries are the quads'; where fluxes and gather are one kernel (weno_pass),
+ * face and gather entries are both its. */
 int weno_solver_launch_config(weno_solver_t s, int32_t* cfg);
 
 /* Testing aid for the bounded device waits (the paper has no counterpart).

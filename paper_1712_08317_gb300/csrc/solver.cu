@@ -212,7 +212,7 @@ F64Grid f64_grid(const S& s, int64_t n, int nv, int M, int G, bool characteristi
 // launch and the wait for the quads' last tiles, about 5 us; against that its triangles run at the quads'
 // register count, 16 instead of 24 warps an SM and 5 % slower.  A step of 133k cells takes 138.8 us in one
 // launch and 151.1 in two, of 241k cells (63 % triangles) 211 and 219, of 1.0M cells 815 and 796.
-bool merge_kinds(const S& s) { return s.nQ + s.nT <= (int64_t)16 * 8 * kTile * s.nsm; }
+bool merge_kinds(const S& s) { return s.nQ && s.nT && s.nQ + s.nT <= (int64_t)16 * 8 * kTile * s.nsm; }
 
 // Characteristic variables, FP32C: a set of threads for every face of a cell while the blocks, three or four
 // an SM with 256 or 192 threads, are all resident at once; above, the longer chain of a thread is hidden by
@@ -389,6 +389,22 @@ void launch_gather(S& s, int mode, const void* fl, void* U, void* Ulo, void* R, 
 constexpr int kUpdateBlock = 128;
 // While the pass's four lanes per cell fit the SMs at once (its 60 registers allow 1,024 threads an SM).
 bool use_fused(const S& s) { return !s.fp64 && s.nv == 4 && 4 * s.N <= (int64_t)1024 * s.nsm; }
+
+// Launch shapes of a residual's kernels as they are chosen now; grid 0: as many blocks as the work takes.  Where the
+// cell types take launches of their own, cell_launch is that of the quads.
+bool split_form(const S& s) { return s.tma && s.prm.characteristic && split_faces(s); }
+Launch cell_launch(const S& s) {
+  if (s.fp64) {
+    const F64Grid g = s.nQ ? f64_grid(s, s.nQ, s.nv, 12, 8, s.prm.characteristic) : f64_grid(s, s.nT, s.nv, 9, 6, s.prm.characteristic);
+    return {(int)g.threads, 0};
+  }
+  if (split_form(s)) return {s.nQ ? weno::dev::K1Threads<1, true>::value : weno::dev::K1Threads<2, true>::value, 0};
+  const Launch& l = s.nQ ? s.k1q : s.k1t;
+  return s.tma ? Launch{kTile * 4, l.grid} : l;
+}
+Launch face_launch(const S& s) { return s.fused ? Launch{kUpdateBlock} : s.k2; }
+Launch gather_launch(const S& s) { return s.fused ? Launch{kUpdateBlock} : s.k3; }
+
 template <int MODE>
 void launch_update_mode(S& s, const void* wg, double c, void* U, void* Ulo, void* R, cudaStream_t st) {
   const auto kernel = s.n_in ? weno::dev::k_update_f32c<MODE, true> : weno::dev::k_update_f32c<MODE, false>;
@@ -912,8 +928,6 @@ int weno_solver_create(weno_mesh_t mesh, const weno_params* params, void* cuda_s
     if ((r = upload_split<12>(d, tq, d.q_pitch, &d.q_gam, &d.q_wt, &d.q_sig, st))) return r;
     if ((r = upload_split<9>(d, tt, d.t_pitch, &d.t_gam, &d.t_wt, &d.t_sig, st))) return r;
     d.k2.block = 128;  // a warp for each quarter of an SM: the FP64 pipe is split four ways
-    // the FP64 reconstruction's block follows from the mesh (f64_grid) and is not tuned
-    if (d.nQ) d.k1q.block = (int)f64_grid(d, d.nQ, d.nv, 12, 8, p.characteristic).threads;
   } else {
     d.q_pitch = (d.nQ + 63) / 64 * 64;
     d.t_pitch = (d.nT + 63) / 64 * 64;
@@ -1187,9 +1201,11 @@ int weno_check_instances(weno_solver_t s, int32_t* flags, void* cuda_stream) {
 
 int weno_solver_launch_config(weno_solver_t s, int32_t* cfg) {
   if (!s || !cfg) return fail(WENO_EINVAL, "null argument");
-  cfg[0] = s->k1q.block; cfg[1] = s->k1q.grid;
-  cfg[2] = s->k2.block;  cfg[3] = s->k2.grid;
-  cfg[4] = s->k3.block; cfg[5] = s->k3.grid;
+  const Launch l[3] = {cell_launch(*s), face_launch(*s), gather_launch(*s)};
+  for (int i = 0; i < 3; ++i) {
+    cfg[2 * i] = l[i].block;
+    cfg[2 * i + 1] = l[i].grid;
+  }
   return WENO_OK;
 }
 
@@ -1242,13 +1258,22 @@ int weno_autotune(weno_solver_t s, const void* U, const void* U_lo, void* cuda_s
   };
   S& d = *s;
   const std::vector<Launch>& k1c = d.tma ? tma : generic;
-  // the passes tuned below work on the Gauss values and fluxes of U
+  // What is tuned is what a residual launches: the blocks of the FP64 reconstruction and of the characteristic one
+  // with a set of threads for every face follow from the mesh; both cell types in one launch take k1q; fluxes and
+  // gather in one kernel have a lane for every face.  The passes after the reconstruction work on the Gauss values
+  // and fluxes of U.
   WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st);
   WENO_DISPATCH(d, launch_pass2, d, st);
-  if (d.nQ && !d.fp64) tune(d.k1q, [&] { WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st, 1); }, k1c);
-  if (d.nT && !d.fp64) tune(d.k1t, [&] { WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st, 2); }, k1c);
-  tune(d.k2, [&] { WENO_DISPATCH(d, launch_pass2, d, st); }, generic);
-  tune(d.k3, [&] { WENO_DISPATCH(d, launch_pass3, d, st); }, generic);
+  if (!d.fp64 && !split_form(d)) {
+    const bool merged = d.tma && merge_kinds(d);
+    const int first = merged ? 3 : 1;
+    if (d.nQ) tune(d.k1q, [&] { WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st, first); }, k1c);
+    if (d.nT && !merged) tune(d.k1t, [&] { WENO_DISPATCH(d, launch_reconstruct, d, U, U_lo, st, 2); }, k1c);
+  }
+  if (!d.fused) {
+    tune(d.k2, [&] { WENO_DISPATCH(d, launch_pass2, d, st); }, generic);
+    tune(d.k3, [&] { WENO_DISPATCH(d, launch_pass3, d, st); }, generic);
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   CK(cudaStreamSynchronize(st));
