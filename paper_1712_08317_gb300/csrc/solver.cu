@@ -247,9 +247,12 @@ void launch_tma_kinds(S& s, const Launch& l, const float* u, const float* ul, fl
   const int64_t tiles = (KINDS & 1 ? (s.nQ + kTile - 1) / kTile : 0) + (KINDS & 2 ? (s.nT + kTile - 1) / kTile : 0);
   auto run = [&](auto split) {
     constexpr bool SPLIT = decltype(split)::value;
-    launch(weno::dev::k_reconstruct_tma<KINDS, CHAR, WALLS, SPLIT>, SPLIT ? (unsigned)tiles : tma_grid(l, tiles),
-           weno::dev::K1Threads<KINDS, SPLIT>::value, weno::dev::K1Smem<KINDS>::bytes, st, s.q_maps, s.t_maps, q, t, s.err,
-           s.debug_stall, tables_once(s));
+    constexpr int smem = weno::dev::K1Smem<KINDS>::bytes;
+    const auto kernel = weno::dev::k_reconstruct_tma<KINDS, CHAR, WALLS, SPLIT>;
+    if constexpr (smem > 48 * 1024)  // tiles of 64 cells (WENO_K1_TILE)
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    launch(kernel, SPLIT ? (unsigned)tiles : tma_grid(l, tiles), weno::dev::K1Threads<KINDS, SPLIT>::value, smem, st, s.q_maps,
+           s.t_maps, q, t, s.err, s.debug_stall, tables_once(s));
   };
   if constexpr (CHAR) {
     if (split_faces(s)) return run(std::true_type{});
@@ -668,7 +671,7 @@ int make_map_2d(EncodeTiled enc, CUtensorMap* map, void* base, uint64_t inner, u
   return WENO_OK;
 }
 
-// Tensor maps of the TMA reconstruction (Euler FP32C) and its shared-memory opt-in.
+// Tensor maps of the TMA reconstruction (Euler FP32C).
 int setup_tma(S& s) {
   void* fn = nullptr;
   cudaDriverEntryPointQueryResult q;
