@@ -356,6 +356,16 @@ def k1_traffic(nQ, nT, kind=""):
     return nQ * K1_TRAFFIC[kind + "quad"] + nT * K1_TRAFFIC[kind + "tri"]
 
 
+def step_launches(nQ, nT, sms):
+    """Kernel launches of one FP32C Euler step (a test holds this against the launches themselves): k_set_dt,
+    the three stages, k_advance_time.  A stage: the reconstruction (one launch for both cell types up to 16 rounds
+    of eight 16-cell tiles an SM), then the fluxes and the gather, in one kernel while four lanes a cell fit 1,024
+    threads an SM."""
+    n = nQ + nT
+    k1 = 2 if nQ and nT and n > 16 * 8 * 16 * sms else 1
+    return 2 + 3 * (k1 + (1 if 4 * n <= 1024 * sms else 2))
+
+
 def measure_peaks():
     """Measured pipe throughputs of this GPU (weno_probe_peak), in Top/s with an FMA counted as one
     operation: FP32 FMA (the better of scalar and paired instructions), FP64 FMA, MUFU reciprocal."""
@@ -1110,7 +1120,7 @@ def main():
         char = {"value": whole_job_rate(ws, N, 3 * args.char_steps, char_ms), "unit": UNIT,
                 "steps": args.char_steps, "ms_per_step": char_ms / args.char_steps, "precision": "fp32c",
                 "reconstruction": "characteristic variables (Roe-averaged normal Jacobian per face)",
-                "roofline": {"kernel": "k_reconstruct_char_tma (quad + triangle launches of one pass)",
+                "roofline": {"kernel": "k_reconstruct_tma, characteristic variables (quad + triangle launches of one pass)",
                              "bound": "alu", "achieved": char_ops / (char_k1 / 1e3) / 1e12, "peak": alu_peak,
                              "unit": "Top/s (FP32 ops, FMA = 1)",
                              "frac": char_ops / (char_k1 / 1e3) / 1e12 / alu_peak,
@@ -1131,12 +1141,8 @@ def main():
                                                     for n in (20, 40, 80, args.acc_n)], precs),
                   "vortex_lowq": ladder_orders([ladder_point("vortex-lowq", n, precs) for n in (40, 80, 160)], precs)}
 
-    # k_set_dt, the three stages, k_advance_time.  A stage: the reconstruction (one launch for both cell
-    # types up to 16 rounds of eight 16-cell tiles an SM), then the fluxes and the gather, in one kernel
-    # while four lanes a cell fit 1,024 threads an SM
     sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-    k1_launches = 2 if nQ and nT and N > 16 * 8 * 16 * sms else 1
-    launches_per_step = 2 + 3 * (k1_launches + (1 if 4 * N <= 1024 * sms else 2))
+    launches_per_step = step_launches(nQ, nT, sms)
     launch_cfg = sol.launch_config().tolist()
     del sol64, V
     batched = None

@@ -95,8 +95,8 @@ __device__ __forceinline__ PosNum pos_of(double x) {
   return PosNum{(uint64_t)(0x80000000u | __funnelshift_l(l, h, 11)) << 32 | (l << 11), (int)(h >> 20)};
 }
 // The same number in one word, for tables and shared memory: t, whose low 11 bits are zero, with the biased
-// exponent in them.  Two instructions unpack it where pos_of takes four:
-// of about 110 integer instructions a point and candidate, ten.  33k-cell vortex step 584.8 -> 575.7 us, 53k-cell
+// exponent in them.  Two instructions unpack it where pos_of takes four, which saves ten of the about 110 integer
+// instructions a point and candidate.  33k-cell vortex step 584.8 -> 575.7 us, 53k-cell
 // residual 293.6 -> 290.1, 8k-quad CFL step 245.1 -> 241.5; in characteristic variables, where no thread shares
 // its indicators, 434.1 -> 437.4: it keeps FP64 weights.
 struct PosWord { uint64_t bits; };

@@ -54,8 +54,9 @@ template <> struct Sub<9> {
 // visible.  Before kernel_wait a kernel touches nothing but the solver's constant tables.  Whatever a
 // kernel of the chain writes is read with plain loads (no __ldg, no __restrict__: the read-only path is
 // for data constant over the kernel's life, which now begins before its predecessor's end).
-// Only the flux kernels call kernel_begin: a kernel that starts early fills the first SMs with room instead
-// of spreading over all of them, which costs a reconstruction more than the early start brings (8,051 FP64
+// Only short kernels call kernel_begin: the FP32C fluxes, k_advance_time and the first level of the
+// reductions.  A kernel that starts early fills the first SMs with room instead of spreading over all of
+// them, which costs a reconstruction more than the early start brings (8,051 FP64
 // quads with it in every kernel: 292 us a step instead of 272).  Before / after: 10,000 triangles in
 // characteristic variables 41.0 -> 38.9 us a step, 800 triangles 22.5 -> 20.5, 133k cells 139.6 -> 136.8,
 // 1.0M cells 798 -> 790, a residual of 53k FP64 cells 364 -> 349.
@@ -499,7 +500,7 @@ struct PairTile {
 // Indicators are clamped to kBetaMax before beta^2 and beta^3 are formed (below).  A candidate
 // with beta that large has alpha = gamma / (beta~ + eps)^2 < 1e-40 whether clamped or not, i.e.
 // zero in FP32; where every candidate of a group is that large, the sum of alpha is zero and the
-// cell goes to the FP64 fix-up, which uses the unclamped value.
+// cell is redone with FP64 weights, from the unclamped value.
 constexpr float kBetaMax = 1e12f;
 
 // All G Gauss values of one (cell, variable) from its stencil differences dW (dW[0] = 0) and the
@@ -804,7 +805,7 @@ __device__ __forceinline__ void roe_rows(const float Wl[4], const float Wr[4], f
 // Increments R(x_G) - W0 of one field at the two Gauss points of face k from that field's stencil
 // differences dU (dU[0] = 0) and the tile's point-pair tables (PairTile rows), FP32: the arithmetic
 // of pair_points for a single face, candidates outer, both points in one paired instruction.
-// Returns false if a sum of alpha fell below kAlphaMin (the cell then goes to the FP64 fix-up).
+// Returns false if a sum of alpha fell below kAlphaMin (the cell is then redone, fix_cell_char).
 template <int M>
 __device__ __forceinline__ bool face_pair(const float4* __restrict__ sgam, const float4* __restrict__ sdg,
                                           const float4* __restrict__ sgo, int cl, int k, const float* dU, float a0,
@@ -1421,7 +1422,7 @@ __global__ void __launch_bounds__(256) k_update_f32c(
 // FP64 instructions a quad, not about 110 with IEEE division), FP32 states are widened on the integer
 // pipe, minima are taken on the bits of the numbers, and a chunk is as many cells as spread a mesh over
 // all SMs.
-// 260k FP32C cells, both results: 170 -> 80 us (k_chunk_dt 24, k_chunk_sum 14, the rest launches and waits for
+// 260k FP32C cells, both results: 170 -> 80 us (k_chunk_dt 29, k_chunk_sum 13, the rest launches and waits for
 // the host); 8k FP64 quads, time step: 27 us less.
 
 // A float as a double by integer operations, except for subnormals, infinities and NaN.

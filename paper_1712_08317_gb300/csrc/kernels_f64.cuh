@@ -13,9 +13,10 @@
 // K1 measured (one pass; first: one thread per (cell, variable), IEEE division, the splitting repeated
 // by every variable, 5,350 FP64 issue slots a (cell, variable) of quads; then: as here with all of the
 // weights in FP64, 2,140 slots; then: gamma / d^2 on the integer pipe, 1,200; their sums too, 940; now: the
-// indicators d too, 560): 17,920 Euler quads 662 -> 277 -> 154 -> 124 -> 103 us, 15,360 triangles
-// 384 -> 144 -> 83 -> 68 -> 57 us, 1,600 scalar quads 332 -> 30 us and now 17.  The FP64 pipe is 66 % and the
-// integer pipe 62 % busy: the two now balance, and what is left is how well they overlap.
+// indicators d too, 560): 17,920 Euler quads 662 -> 277 -> 154 -> 124 -> 100 us, 15,360 triangles
+// 384 -> 144 -> 83 -> 68 -> 56 us, 1,600 scalar quads 332 -> 30 us and now 16.  On 343k quads and 295k triangles
+// the FP64 pipe is 72 and 76 %, the integer pipe 67 and 64 % busy: the two balance, and what is left is how
+// well they overlap.
 #pragma once
 
 #include "kernels.cuh"

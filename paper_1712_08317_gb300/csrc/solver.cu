@@ -1393,8 +1393,9 @@ void launch_residual_static(S& s, const void* U, const void* Ulo, void* R, void*
 
 extern "C" int weno_residual_static(weno_solver_t s, const void* U, const void* U_lo, void* R, void* cuda_stream) {
   if (!s || !U || !R || (!s->fp64 && !U_lo)) return fail(WENO_EINVAL, "null argument");
-  // Gauss-point values first, face fluxes after them on a 256-byte boundary; FP32C Euler solvers keep
-  // room for a byte per 16-cell tile and a bit per cell after those (the limit the header states)
+  // Gauss-point values first, face fluxes after them on a 256-byte boundary; after those FP32C Euler solvers
+  // count, but do not use, a byte per 16-cell tile and a bit per cell: the limit the header states, which
+  // keeps refusing what it refused
   const size_t wg_bytes = (size_t)(8 * s->nQ + 6 * s->nT) * s->nv * s->esz;
   const size_t f_off = (wg_bytes + 255) / 256 * 256;
   const size_t r_off = (f_off + (size_t)s->nF * s->nv * s->esz + 255) / 256 * 256;
