@@ -34,8 +34,8 @@ FALLBACK_HBM_GBS = 6800.0
 # 637k-cell mesh of the benchmark family (n = 700), divided by its cells of each type.  They describe
 # the kernel source they were captured on (SHA-256 of csrc/kernels.cuh); for any other source the
 # bench line reports traffic null.
-K1_TRAFFIC = {"kernels_cuh_sha256": "5b667bd92fe3de3efdeffa43428cf0a413db9e55103b26e2c10e98df825471e7",
-              "quad": 1304.7, "tri": 847.5, "char_quad": 1308.3, "char_tri": 857.1}
+K1_TRAFFIC = {"kernels_cuh_sha256": "1db65e7f5e2a2bdc7fd6f4543b5646cbf19c29fe7ca0eb9784434dc2a7171344",
+              "quad": 1304.4, "tri": 849.4, "char_quad": 1311.7, "char_tri": 853.1}
 WORKLOAD_N = 1754
 
 

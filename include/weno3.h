@@ -193,7 +193,8 @@ int weno_solver_create(weno_mesh_t mesh, const weno_params* params, void* cuda_s
 int weno_solver_get_info(weno_solver_t s, weno_mesh_info* info);
 
 /* R = L(U) (Eq. 4) at the solver's time.  U, U_lo, R: device arrays
- * [n_cells * n_v] (U_lo only for FP32C, else NULL).  Stream-ordered. */
+ * [n_cells * n_v] (U_lo only for FP32C, else NULL); for the Euler equations
+ * they start on 16-byte boundaries, here and in the steps.  Stream-ordered. */
 int weno_residual(weno_solver_t s, const void* U, const void* U_lo, void* R, void* cuda_stream);
 
 /* R = L(U) exactly like weno_residual, but without touching any memory the
@@ -241,11 +242,13 @@ int weno_step_instances(weno_solver_t s, void* U, void* U_lo, const double* dt_d
 
 /* Largest stable dt (reading of the CFL rule: dt = cfl * min_i 2|Omega_i| /
  * sum_p (|v_i . n_p| + c_i) |l_p|, c = 0 for scalar advection), per
- * instance: dt_out[n_instances] on the host.  Synchronising. */
+ * instance: dt_out[n_instances] on the host.  U and U_lo may start at any
+ * element of a buffer.  Synchronising. */
 int weno_max_dt(weno_solver_t s, const void* U, const void* U_lo, double cfl, double* dt_out, void* cuda_stream);
 
 /* sum_i |Omega_i| (U + U_lo)_i in FP64 per instance and variable:
- * sums[n_instances * n_v] on the host.  Deterministic order. Synchronising. */
+ * sums[n_instances * n_v] on the host.  U and U_lo may start at any element of
+ * a buffer.  Deterministic order.  Synchronising. */
 int weno_conservation(weno_solver_t s, const void* U, const void* U_lo, double* sums, void* cuda_stream);
 
 /* Reads and clears the device flags raised by residual / step launches since
